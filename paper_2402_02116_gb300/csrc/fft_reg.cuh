@@ -25,6 +25,7 @@
 #include <utility>
 
 #include "fft.cuh"
+#include "fft_pair.cuh"
 
 namespace dbi {
 
@@ -101,6 +102,10 @@ template <int L, int V> constexpr int layout_of(int p) {
   else return p == 0 ? 1 : (p == 1 ? (V == 0 ? 2 : 1) : 0);
 }
 
+// Type of the twiddles of a transform on elements of type C (pairs of components share them).
+template <typename C> struct TwOf { using type = C; };
+template <> struct TwOf<cpair> { using type = float2; };
+
 template <typename C, int L, int V = 0> struct TwReg {
   static constexpr int NW = PlanInfo<L, V>::nw;
   C w[NW];
@@ -124,9 +129,14 @@ template <typename C, int L, int V = 0> struct TwReg {
 };
 
 template <typename C, int L> struct RegFFT {
+  using W = typename TwOf<C>::type;
   static constexpr int T = L / 8;                 // threads per line
-  // padded line length (and pitch of consecutive lines) in shared memory
-  static constexpr int LP = L == 16 ? 18 : L == 64 ? 72 : L + L / 16 + 2;
+  // Padded line length (and pitch of consecutive lines) in shared memory. 16-byte pairs are served
+  // a quarter warp at a time: with one padding slot per 8 points every store and load of every
+  // exchange of every plan (and lines side by side in a warp, L <= 32) hits 8 distinct 16-byte bank
+  // slots, and every offset is an immediate of one per-thread base address.
+  static constexpr bool kPairs = std::is_same_v<C, cpair>;
+  static constexpr int LP = kPairs ? L + L / 8 : L == 16 ? 18 : L == 64 ? 72 : L + L / 16 + 2;
   static constexpr int TWS = kTwiddleN / L;       // table stride of W_L
 
   // Position of point i of a line in shared memory, by layout (chosen per exchange, see
@@ -151,7 +161,7 @@ template <typename C, int L> struct RegFFT {
   // The NB = 8/R butterflies of one pass on registers in natural order: twiddle by the powers
   // wp[i][r] (NS > 1), R-point DFT. HIN (first pass only): v[4..7] are zero and not read.
   template <int R, int NS, bool INV, bool HIN>
-  __host__ __device__ __forceinline__ static void butterflies(C (&v)[8], const C (&wp)[8 / R][R]) {
+  __host__ __device__ __forceinline__ static void butterflies(C (&v)[8], const W (&wp)[8 / R][R]) {
     constexpr int NB = 8 / R;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
@@ -162,7 +172,8 @@ template <typename C, int L> struct RegFFT {
 #pragma unroll
         for (int r = 1; r < R; ++r) x[r] = hmul(x[r], wp[i][r]);
       }
-      if constexpr (HIN) dft_half_in<C, R, INV>(x);
+      if constexpr (kPairs) pair_dft<R, INV, HIN>(x);
+      else if constexpr (HIN) dft_half_in<C, R, INV>(x);
       else dft<C, R, INV>(x);
 #pragma unroll
       for (int r = 0; r < R; ++r) v[i + r * NB] = x[r];
@@ -176,15 +187,27 @@ template <typename C, int L> struct RegFFT {
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
       const int j = t + i * T, k = j % NS, base = (j - k) * R + k;
+      if constexpr (kPairs) {  // base mod 8 + (r NS mod 8) < 8 in every plan: pad() splits into the sum
+        C *d = line + pad<LAY>(base);
 #pragma unroll
-      for (int r = 0; r < R; ++r) line[pad<LAY>(base + r * NS)] = v[i + r * NB];
+        for (int r = 0; r < R; ++r) d[r * NS + r * NS / 8] = v[i + r * NB];
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) line[pad<LAY>(base + r * NS)] = v[i + r * NB];
+      }
     }
   }
 
   // Load the next pass's input (natural order) from a shared-memory line.
   template <int LAY> __host__ __device__ __forceinline__ static void gather(C (&v)[8], const C *line, int t) {
+    if constexpr (kPairs) {  // t mod 8 + (m T mod 8) < 8, as in scatter()
+      const C *d = line + pad<LAY>(t);
 #pragma unroll
-    for (int m = 0; m < 8; ++m) v[m] = line[pad<LAY>(t + m * T)];
+      for (int m = 0; m < 8; ++m) v[m] = d[m * T + m * T / 8];
+    } else {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) v[m] = line[pad<LAY>(t + m * T)];
+    }
   }
 };
 
@@ -208,20 +231,21 @@ __host__ __device__ __forceinline__ void pass_powers(const C *w1, C (&wp)[NB][R]
 template <int L, int V = 0> struct RegPlan {
   template <typename C, int NLT, bool INV, bool HIN = false, typename Sync>
   __host__ __device__ __forceinline__ static void run(C (&v)[NLT][8], C *const (&lines)[NLT], int t,
-                                                      const TwReg<C, L, V> &tr, Sync &&sync) {
+                                                      const TwReg<typename TwOf<C>::type, L, V> &tr, Sync &&sync) {
     using F = RegFFT<C, L>;
+    using W = typename TwOf<C>::type;
     using P = PlanInfo<L, V>;
     [&]<int... p>(std::integer_sequence<int, p...>) {
       (
           [&] {
             constexpr int R = P::radix(p), NS = P::ns(p), NB = 8 / R;
             constexpr bool H = HIN && p == 0, LAST = p == P::np - 1;
-            C wp[NB][R];
-            if constexpr (NS > 1) pass_powers<C, R, INV, NB>(tr.w + P::woff(p), wp);
+            W wp[NB][R];
+            if constexpr (NS > 1) pass_powers<W, R, INV, NB>(tr.w + P::woff(p), wp);
 #pragma unroll
             for (int l = 0; l < NLT; ++l) F::template butterflies<R, NS, INV, H>(v[l], wp);
             if constexpr (!LAST) {
-              constexpr int LAY = layout_of<L, V>(p);
+              constexpr int LAY = F::kPairs ? 3 : layout_of<L, V>(p);
 #pragma unroll
               for (int l = 0; l < NLT; ++l) F::template scatter<R, NS, LAY>(v[l], lines[l], t);
               sync();

@@ -253,8 +253,12 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(C) == 8 ? 2 : 1) kk_cols(
     for (int mm = 0; mm < kHalf; ++mm) {
       const int z = t + mm * T;
       if (z < nz) {
-        o[size_t(kx) * nz + z] = acc[0][mm];
-        o[(size_t(lx) + kx) * nz + z] = acc[1][mm];
+        if constexpr (kPairSpectra<C>) {
+          reinterpret_cast<cpair *>(o)[size_t(kx) * nz + z] = mkpair(acc[0][mm], acc[1][mm]);
+        } else {
+          o[size_t(kx) * nz + z] = acc[0][mm];
+          o[(size_t(lx) + kx) * nz + z] = acc[1][mm];
+        }
       }
     }
   }

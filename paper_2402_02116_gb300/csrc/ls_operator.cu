@@ -97,6 +97,53 @@ __global__ void __launch_bounds__(kTileThreads, Cfg<C>::colMinBlocks) k_cols(OpP
   cols_tile<C, LZ, V>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x, reinterpret_cast<C *>(smem_raw));
 }
 
+// The complex64 column stage: a CTA takes the columns kx of SL launch slots at a time (units
+// of T threads: unit u = column u / SL, slot u % SL). With SL = 4 the columns' Green's tables of the
+// first slot's frequency are staged in shared memory by asynchronous copies issued before the
+// forward transforms; slots of that frequency (consecutive slots share it, problems being
+// frequency-major) read them there, others from global memory. SL = 1 (few slots) reads the
+// tables from global memory. Bound by shared memory (82 % of the wavefront rate at L = 512, 80
+// registers, 3 CTAs per SM): 256 problems of 256^2 take 422 us, against 462 us with the components as
+// separate 8-byte lines and the tables read from L2 by every slot.
+template <int LZ, int V, int SL>
+__global__ void __launch_bounds__(kTileThreads, Cfg<float2>::colMinBlocks) k_cols_pairs(OpP<float2> p) {
+  using CF = ColCfg<float2, LZ>;
+  constexpr int COLS = CF::CC / SL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cpair *lines = reinterpret_cast<cpair *>(smem_raw);
+  float2 *Gs = reinterpret_cast<float2 *>(lines + size_t(CF::CC) * CF::PLP);
+  const int u = threadIdx.x / CF::T, t = threadIdx.x - u * CF::T;
+  const int kx = blockIdx.x * COLS + u / SL, sl0 = SL * int(blockIdx.y), sl = sl0 + u % SL;
+  auto prob = [&](int slot) { return p.plist ? p.plist[p.s0 + slot] : p.s0 + slot; };
+  auto freq = [&](int slot) {  // the slot's table, or -1 when it has no work
+    if (slot >= p.nb) return -1;
+    const int b = prob(slot), f = p.fidx[b];
+    return ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) ? -1 : f;
+  };
+  const int f0 = freq(sl0), f = SL == 1 ? f0 : freq(sl);
+  if constexpr (SL == 1) {
+    if (f0 < 0) return;  // uniform over the CTA
+  } else if (f0 >= 0) {
+    const size_t plane = size_t(p.lx) * LZ;
+    const float2 *G = p.Ghat + size_t(f0) * 3 * plane;
+    constexpr int N16 = COLS * 3 * LZ / 2;  // 16-byte copies
+#pragma unroll
+    for (int i = 0; i < (N16 + kTileThreads - 1) / kTileThreads; ++i) {
+      const int e = threadIdx.x + i * kTileThreads, ct = e / (LZ / 2), k = e - ct * (LZ / 2);  // ct = column * 3 + table
+      const int gx = blockIdx.x * COLS + ct / 3;
+      if (e < N16 && gx < p.lx) cp_async16(Gs + 2 * e, G + (ct % 3) * plane + size_t(gx) * LZ + 2 * k);
+    }
+  }
+  const bool live = f >= 0 && kx < p.lx;
+  const int b = live ? prob(sl) : 0;
+  cols_unit_pairs<LZ, V, SL != 1>(BatchTile<float2>{p, b, live ? sl : 0, live ? f : 0}, kx, u, t, live, lines,
+                                  f == f0 ? Gs + size_t(u / SL) * 3 * LZ : nullptr);
+}
+template <int LZ, int SL> constexpr size_t cols_pairs_smem() {
+  using CF = ColCfg<float2, LZ>;
+  return size_t(CF::CC) * CF::PLP * sizeof(cpair) + (SL == 1 ? 0 : size_t(CF::CC / SL) * 3 * LZ * sizeof(float2));
+}
+
 template <typename C, int LX, int EPI, int V>
 __global__ void __launch_bounds__(kTileThreads, Cfg<C>::rowInvMinBlocks) k_rows_inverse(OpP<C> p) {
   const int b = problem_of(p), f = p.fidx[b];
@@ -299,11 +346,28 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   if (!split_c) dispatch_len(a.lz, [&]<int LZ>() {
     with_plan<LZ>(a.precision, [&]<int V>() {
       using CF = ColCfg<C, LZ>;
-      const size_t bytes = cols_smem<C, LZ>();
-      dim3 grid((a.lx + CF::CC - 1) / CF::CC, nb);
-      cudaError_t e = allow_smem(k_cols<C, LZ, V>, bytes);
-      if (e == cudaSuccess) k_cols<C, LZ, V><<<grid, CF::NT, bytes, s>>>(p);
-      rc = e != cudaSuccess ? cuda_fail("k_cols smem", e) : check_launch("k_cols");
+      if constexpr (kPairSpectra<C>) {
+        if constexpr (LZ <= 512) {  // 1024 runs as pairs of 512-point transforms
+          cudaError_t e;
+          auto launch = [&]<int SL>() {
+            constexpr int COLS = CF::CC / SL;
+            const size_t bytes = cols_pairs_smem<LZ, SL>();
+            e = allow_smem(k_cols_pairs<LZ, V, SL>, bytes);
+            if (e == cudaSuccess)
+              k_cols_pairs<LZ, V, SL><<<dim3((a.lx + COLS - 1) / COLS, (nb + SL - 1) / SL), CF::NT, bytes, s>>>(p);
+          };
+          // four slots per CTA unless the last group would leave much of its CTAs idle
+          if (nb % 4 == 0 || nb >= 16) launch.template operator()<4>();
+          else launch.template operator()<1>();
+          rc = e != cudaSuccess ? cuda_fail("k_cols_pairs smem", e) : check_launch("k_cols_pairs");
+        }
+      } else {
+        const size_t bytes = cols_smem<C, LZ>();
+        dim3 grid((a.lx + CF::CC - 1) / CF::CC, nb);
+        cudaError_t e = allow_smem(k_cols<C, LZ, V>, bytes);
+        if (e == cudaSuccess) k_cols<C, LZ, V><<<grid, CF::NT, bytes, s>>>(p);
+        rc = e != cudaSuccess ? cuda_fail("k_cols smem", e) : check_launch("k_cols");
+      }
     });
   });
   prof_mark(PROF_COLS, true, s);

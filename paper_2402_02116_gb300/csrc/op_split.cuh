@@ -10,7 +10,7 @@
 // The register FFT of length M = 512 (three radix-8 passes, two shared-memory exchanges) replaces
 // the length-1024 one (four passes, three exchanges, half of the first or last pass idle), which
 // cuts the exchanges by a third; with 64 threads per line a 256-thread CTA takes four rows, so
-// the row stages read and write the column-major spectra in 32-byte runs (one sector).
+// the row stages read and write the column-major spectra in 64-byte runs (four pairs).
 //
 // The contrast source is formed by its own kernel (source_rows) into a scratch field, so that the
 // row transform needs no halo rows and few registers.
@@ -23,33 +23,27 @@ namespace dbi {
 constexpr int kSplitL = 1024, kSplitM = 512;
 constexpr int kSplitT = kSplitM / 8;                  // threads per line (64)
 constexpr int kSplitRows = kTileThreads / kSplitT;    // rows (or columns) per 256-thread tile (4)
-constexpr int kSplitLP = RegFFT<float2, kSplitM>::LP; // padded line in shared memory
+constexpr int kSplitLP = RegFFT<cpair, kSplitM>::LP;  // padded line of pairs in shared memory
 static_assert(kSplitL == 1024, "the per-point twiddles come from the contiguous W_1024 table");
 
-// Transposition tile of the row stages, one component at a time: [rows][KP]. A thread's pair of
-// points (2k, 2k + 1) is one 16-byte access (a quarter warp covers 128 contiguous bytes); the
-// column-major 8-byte reads and writes of four rows at a time are served half a warp at a time,
-// and with KP = 4 mod 16 the four rows x four kx of a half warp hit 16 distinct 8-byte bank slots.
-constexpr int kSplitKP = kSplitL + 4;
+// Transposition tile of the row stages, [rows][KP] pairs, the even kx of a row before its odd ones
+// (position q M + k holds kx = 2k + q, as the transforms of the two parities leave them): a quarter
+// warp's 16-byte accesses hit 8 distinct bank slots along a row and down the tile (4 rows x 2
+// positions, KP = 2 mod 8).
+constexpr int kSplitKP = kSplitL + 2;
+__device__ __forceinline__ int split_kx(int j) { return 2 * (j & (kSplitM - 1)) + (j >= kSplitM); }
 
-// Shared memory (bytes) of the split stages: the lines of one parity (two per row or column) and,
-// for the row stages, the transposition tile of one component.
-// The row stages run the two parities one after the other through two lines per row (one per
-// component); the column stage runs all four lines of a column at once (the twiddle powers formed
-// once, half the barriers: measured faster there and slower in the row stages).
-__host__ __device__ constexpr size_t split_lines_smem() { return size_t(2) * kSplitRows * kSplitLP * sizeof(float2); }
-__host__ __device__ constexpr size_t split_cols_lines_smem() {
-  return size_t(4) * kSplitRows * kSplitLP * sizeof(float2);
-}
-__host__ __device__ constexpr size_t split_tile_smem() { return size_t(kSplitRows) * kSplitKP * sizeof(float2); }
+// Shared memory (bytes): the row stages run the two parities one after the other through one line
+// of pairs per row, whose memory the transposition tile reuses; the column stage runs both lines of a
+// column at once (the twiddle powers formed once, half the barriers).
+__host__ __device__ constexpr size_t split_lines_smem() { return size_t(kSplitRows) * kSplitLP * sizeof(cpair); }
+__host__ __device__ constexpr size_t split_cols_lines_smem() { return 2 * split_lines_smem(); }
+__host__ __device__ constexpr size_t split_tile_smem() { return size_t(kSplitRows) * kSplitKP * sizeof(cpair); }
 __host__ __device__ constexpr size_t split_rows_smem() {
   return split_lines_smem() > split_tile_smem() ? split_lines_smem() : split_tile_smem();
 }
 __host__ __device__ constexpr size_t split_cols_smem() { return split_cols_lines_smem(); }
-// The inverse row stage stages the tiles of both components at once: [2][rows][KP].
-__host__ __device__ constexpr size_t split_rows_inverse_smem() {
-  return split_lines_smem() > 2 * split_tile_smem() ? split_lines_smem() : 2 * split_tile_smem();
-}
+__host__ __device__ constexpr size_t split_rows_inverse_smem() { return split_rows_smem(); }
 
 // Contrast source of the stencil kernel: one thread per column (nx <= M = 512 columns, the zero
 // columns x = -1 and x = nx on either side), a chunk of kSrcRows rows per CTA walked downwards.
@@ -169,29 +163,17 @@ __device__ __forceinline__ void source_rows(const A &a, int chunk, float2 *smem,
   if (j <= ze) step.template operator()<1>(j);
 }
 
-// The two parities of the two components, each an M-point transform held as 8 points per thread:
-// v[q][c][m] is point t + m T of the line of component c and parity q.
-struct SplitLines {
-  float2 *l[2][2];
-};
-
-// M-point transforms of both parities, one parity at a time through the two lines of the
-// components (the row stages).
+// The two parities, each an M-point transform of pairs held as 8 points per thread: v[q][m] is
+// point t + m T of parity q.
+// One parity at a time through one line (the row stages).
 template <bool INV, typename Sync>
-__device__ __forceinline__ void split_fft(float2 (&v)[2][2][8], float2 *const (&lines)[2], int t,
-                                          const TwReg<float2, kSplitM, 0> &tr, Sync &&sync) {
+__device__ __forceinline__ void split_fft(cpair (&v)[2][8], cpair *line, int t, const TwReg<float2, kSplitM, 0> &tr,
+                                          Sync &&sync) {
+  cpair *const lines[1] = {line};
 #pragma unroll
-  for (int q = 0; q < 2; ++q) RegPlan<kSplitM, 0>::template run<float2, 2, INV>(v[q], lines, t, tr, sync);
+  for (int q = 0; q < 2; ++q)
+    RegPlan<kSplitM, 0>::template run<cpair, 1, INV>(reinterpret_cast<cpair(&)[1][8]>(v[q]), lines, t, tr, sync);
 }
-
-// M-point transforms of both parities and both components at once, four lines through one
-// exchange set (the column stage).
-template <bool INV, typename Sync>
-__device__ __forceinline__ void split_fft4(float2 (&v)[2][2][8], float2 *const (&lines)[4], int t,
-                                           const TwReg<float2, kSplitM, 0> &tr, Sync &&sync) {
-  RegPlan<kSplitM, 0>::template run<float2, 4, INV>(reinterpret_cast<float2(&)[4][8]>(v), lines, t, tr, sync);
-}
-
 
 // Shared memory of the column stage with the column's Green's tables staged: the lines, then
 // Ghat(:, kx) of the three tables [3][L].
@@ -213,25 +195,20 @@ __device__ __forceinline__ void cols_column_split(const A &a, int kx, int g, boo
   const int t = threadIdx.x - g * T;
   const int nz = a.nz(), lx = a.lx();
   const C *tw = a.tw();
-  C *c0 = a.T() + size_t(kx) * nz, *c1 = a.T() + (size_t(lx) + kx) * nz;
+  cpair *c = reinterpret_cast<cpair *>(a.T()) + size_t(kx) * nz;
   const TwReg<C, kSplitM, 0> tr(t, tw);
-  C *lines[4];  // (parity q, component c) of column group g
-#pragma unroll
-  for (int l = 0; l < 4; ++l) lines[l] = smem + size_t(l * CC + g) * kSplitLP;
-  C v[2][2][8];
+  cpair *const lines[2] = {reinterpret_cast<cpair *>(smem) + size_t(g) * kSplitLP,
+                           reinterpret_cast<cpair *>(smem) + size_t(CC + g) * kSplitLP};
+  cpair v[2][8];
   if (live) {
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int z = t + m * T;
-      const bool in = z < nz;
-      const C x0 = in ? c0[z] : czero<C>(), x1 = in ? c1[z] : czero<C>();
-      const C w = __ldg(tw + kTw1024 + z);  // W_L^z
-      v[0][0][m] = x0;
-      v[0][1][m] = x1;
-      v[1][0][m] = hmul(x0, w);
-      v[1][1][m] = hmul(x1, w);
+      const cpair x = z < nz ? c[z] : pzero();
+      v[0][m] = x;
+      v[1][m] = hmul(x, __ldg(tw + kTw1024 + z));  // W_L^z
     }
-    split_fft4<false>(v, lines, t, tr, RowSync<T>{1 + g});
+    RegPlan<kSplitM, 0>::template run<cpair, 2, false>(v, lines, t, tr, RowSync<T>{1 + g});
   }
   if constexpr (STAGED) {
     cp_async_wait_all();
@@ -250,26 +227,17 @@ __device__ __forceinline__ void cols_column_split(const A &a, int kx, int g, boo
       } else {
         g11 = __ldg(G + k); g13 = __ldg(G + plane / 2 + k); g33 = __ldg(G + plane + k);
       }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const C a11 = q ? make_float2(g11.z, g11.w) : make_float2(g11.x, g11.y);
-        const C a13 = q ? make_float2(g13.z, g13.w) : make_float2(g13.x, g13.y);
-        const C a33 = q ? make_float2(g33.z, g33.w) : make_float2(g33.x, g33.y);
-        const C s1 = v[q][0][m], s3 = v[q][1][m];
-        v[q][0][m] = cadd(cmul(a11, s1), cmul(a13, s3));
-        v[q][1][m] = cadd(cmul(a13, s1), cmul(a33, s3));
-      }
+      v[0][m] = green_product(v[0][m], make_float2(g11.x, g11.y), make_float2(g13.x, g13.y),
+                              make_float2(g33.x, g33.y));
+      v[1][m] = green_product(v[1][m], make_float2(g11.z, g11.w), make_float2(g13.z, g13.w),
+                              make_float2(g33.z, g33.w));
     }
   }
-  split_fft4<true>(v, lines, t, tr, RowSync<T>{1 + g});
+  RegPlan<kSplitM, 0>::template run<cpair, 2, true>(v, lines, t, tr, RowSync<T>{1 + g});
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int z = t + m * T;
-    if (z < nz) {
-      const C w = cconj(__ldg(tw + kTw1024 + z));  // W_L^{-z}
-      c0[z] = cadd(v[0][0][m], cmul(w, v[1][0][m]));
-      c1[z] = cadd(v[0][1][m], cmul(w, v[1][1][m]));
-    }
+    if (z < nz) c[z] = hadd(v[0][m], hmul(v[1][m], cconj(__ldg(tw + kTw1024 + z))));  // W_L^{-z}
   }
 }
 
@@ -282,7 +250,7 @@ __device__ __forceinline__ void cols_tile_split(const A &a, int tile, float2 *sm
 
 // Four rows z0 .. z0 + 3: the source rows (from the stencil kernel, or the raw input times its
 // scale), the forward transform along x (even and odd kx), transposed through shared memory into
-// the column-major spectra T[c][kx][z] in runs of four rows.
+// the column-major spectra T[kx][z] in runs of four rows (64 bytes).
 template <typename A>
 __device__ __forceinline__ void rows_forward_tile_split(const A &a, int tile, float2 *smem, const float2 *src,
                                                         float scale) {
@@ -294,41 +262,39 @@ __device__ __forceinline__ void rows_forward_tile_split(const A &a, int tile, fl
   const size_t plane = size_t(nz) * nx;
   const C *tw = a.tw();
   const TwReg<C, kSplitM, 0> tr(t, tw);
-  C v[2][2][8];
+  cpair v[2][8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int x = t + m * T;
     const bool in = z < nz && x < nx;
     const C s0 = in ? cscale(__ldg(src + size_t(z) * nx + x), scale) : czero<C>();
     const C s1 = in ? cscale(__ldg(src + plane + size_t(z) * nx + x), scale) : czero<C>();
-    const C w = __ldg(tw + kTw1024 + x);  // W_L^x
-    v[0][0][m] = s0;
-    v[0][1][m] = s1;
-    v[1][0][m] = hmul(s0, w);
-    v[1][1][m] = hmul(s1, w);
+    v[0][m] = mkpair(s0, s1);
+    v[1][m] = hmul(v[0][m], __ldg(tw + kTw1024 + x));  // W_L^x
   }
-  C *const lines[2] = {smem + size_t(rr) * kSplitLP, smem + size_t(ROWS + rr) * kSplitLP};
-  split_fft<false>(v, lines, t, tr, RowSync<T>{1 + rr});
-  // transpose one component at a time through tile[rr][kx] (the lines' memory is free now)
+  cpair *ps = reinterpret_cast<cpair *>(smem);
+  split_fft<false>(v, ps + size_t(rr) * kSplitLP, t, tr, RowSync<T>{1 + rr});
+  // transpose through tile[rr][kx] (the lines' memory is free now)
+  __syncthreads();
+  cpair *row = ps + size_t(rr) * KP;
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    __syncthreads();
-    float4 *row = reinterpret_cast<float4 *>(smem + size_t(rr) * KP);
+  for (int m = 0; m < 8; ++m) {  // kx = 2k and 2k + 1
+    row[t + m * T] = v[0][m];
+    row[kSplitM + t + m * T] = v[1][m];
+  }
+  __syncthreads();
+  cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0;
+  const int r = threadIdx.x % ROWS;
+  if (z0 + r < nz) {
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const C e = v[0][c][m], o = v[1][c][m];  // kx = 2k and 2k + 1
-      row[t + m * T] = make_float4(e.x, e.y, o.x, o.y);
-    }
-    __syncthreads();
-    C *Tc = a.T() + size_t(c) * a.lx() * nz;
-    for (int idx = threadIdx.x; idx < kSplitL * ROWS; idx += kTileThreads) {
-      const int r = idx % ROWS, kx = idx / ROWS;
-      if (z0 + r < nz) Tc[size_t(kx) * nz + z0 + r] = smem[size_t(r) * KP + kx];
+    for (int i = 0; i < kSplitL * ROWS / kTileThreads; ++i) {
+      const int j = threadIdx.x / ROWS + i * (kTileThreads / ROWS);
+      Tp[size_t(split_kx(j)) * nz + r] = ps[size_t(r) * KP + j];
     }
   }
 }
 
-// Four rows: the spectra T[c][kx][z0 .. z0 + 3] through a transposition tile, the inverse
+// Four rows: the spectra T[kx][z0 .. z0 + 3] through a transposition tile, the inverse
 // transform along x (even and odd kx), y_x = even + W_L^{-x} odd for x < nx, then the epilogue of
 // rows_inverse_tile: out = ident - scale * y (or the scaled y) with the fused inner products.
 template <int EPI, typename A>
@@ -340,42 +306,38 @@ __device__ __forceinline__ void rows_inverse_tile_split(const A &a, int tile, fl
   const int rr = threadIdx.x / T, t = threadIdx.x - rr * T, z = z0 + rr;
   const C *tw = a.tw();
   const TwReg<C, kSplitM, 0> tr(t, tw);
-  C v[2][2][8];
-  // the spectra of both components into tile[c][r][kx] by asynchronous copies (zeros for rows
-  // beyond nz), all in flight at once and without register staging
-  constexpr int NLD = 2 * kSplitL * ROWS / kTileThreads;  // 32 copies per thread
+  cpair v[2][8];
+  cpair *ps = reinterpret_cast<cpair *>(smem);
+  // the spectra into tile[r][kx] by asynchronous copies (zeros for rows beyond nz), all in flight at
+  // once and without register staging
   {
     const int r = threadIdx.x % ROWS;  // the same row for all of a thread's copies
     const bool in = z0 + r < nz;
-    const C *T0 = a.T() + (in ? z0 + r : 0);
-    const size_t cplane = size_t(a.lx()) * nz;
+    const cpair *T0 = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
 #pragma unroll
-    for (int i = 0; i < NLD; ++i) {
-      const int idx = threadIdx.x + i * kTileThreads, kx = (idx / ROWS) % kSplitL, c = idx / (ROWS * kSplitL);
-      cp_async8(smem + size_t(c * ROWS + r) * KP + kx, T0 + c * cplane + size_t(kx) * nz, in);
+    for (int i = 0; i < kSplitL * ROWS / kTileThreads; ++i) {
+      const int j = threadIdx.x / ROWS + i * (kTileThreads / ROWS);
+      cp_async16z(ps + size_t(r) * KP + j, T0 + size_t(split_kx(j)) * nz, in);
     }
   }
   cp_async_wait_all();
   __syncthreads();
+  {
+    const cpair *row = ps + size_t(rr) * KP;
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const float4 *row = reinterpret_cast<const float4 *>(smem + size_t(c * ROWS + rr) * KP);
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const float4 eo = row[t + m * T];  // kx = 2k and 2k + 1
-      v[0][c][m] = make_float2(eo.x, eo.y);
-      v[1][c][m] = make_float2(eo.z, eo.w);
+    for (int m = 0; m < 8; ++m) {  // kx = 2k and 2k + 1
+      v[0][m] = row[t + m * T];
+      v[1][m] = row[kSplitM + t + m * T];
     }
   }
   __syncthreads();  // the lines reuse the tile's memory
-  C *const lines[2] = {smem + size_t(rr) * kSplitLP, smem + size_t(ROWS + rr) * kSplitLP};
-  split_fft<true>(v, lines, t, tr, RowSync<T>{1 + rr});
+  split_fft<true>(v, ps + size_t(rr) * kSplitLP, t, tr, RowSync<T>{1 + rr});
   C y[2][8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    const C w = cconj(__ldg(tw + kTw1024 + t + m * T));  // W_L^{-x}
-#pragma unroll
-    for (int c = 0; c < 2; ++c) y[c][m] = cadd(v[0][c][m], cmul(w, v[1][c][m]));
+    const cpair w = hadd(v[0][m], hmul(v[1][m], cconj(__ldg(tw + kTw1024 + t + m * T))));  // W_L^{-x}
+    y[0][m] = comp0(w);
+    y[1][m] = comp1(w);
   }
   const float osc = a.osc();
   const size_t base = size_t(z) * nx;

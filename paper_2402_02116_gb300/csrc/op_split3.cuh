@@ -20,20 +20,20 @@ constexpr int kS3L = 768, kS3M = 256;
 constexpr int kS3T = kS3M / 8;                    // threads per line: one warp
 constexpr int kS3Units = 4;                       // rows or columns per CTA
 constexpr int kS3Threads = kS3Units * 3 * kS3T;   // 384: a warp per (unit, residue)
-constexpr int kS3LP = RegFFT<float2, kS3M>::LP;   // padded line in shared memory
-// Transposition tile row of the row stages. 8-byte accesses are served half a warp at a time: with
-// KP = 4 mod 16 the column-major accesses (four rows x four kx per half warp) hit 16 distinct
-// 8-byte bank slots, and so do the residue-strided accesses 3k + q of a warp (3 is odd).
-constexpr int kS3KP = kS3L + 4;
+constexpr int kS3LP = RegFFT<cpair, kS3M>::LP;    // padded line of pairs in shared memory
+// Transposition tile row of the row stages. 16-byte accesses are served a quarter warp at a time:
+// with KP = 2 mod 8 the column-major accesses (four rows x two kx per quarter warp) hit 8 distinct
+// bank slots, and so do the residue-strided accesses 3k + q of a warp (3 is odd).
+constexpr int kS3KP = kS3L + 2;
 constexpr int kS3UnitThreads = 3 * kS3T;          // 96 threads per row or column
 constexpr int kS3Tw = kTwiddleN / kS3L;           // W_L^j = tw[j * kS3Tw]
 constexpr int kS3Third = kTwiddleN / 3;           // W_3 = tw[kS3Third]
 
-// Shared memory (bytes): two lines per warp (one per component); the row stages' transposition
-// tile [c][rr][KP] of both components reuses that memory, and so do the residues' inverse
+// Shared memory (bytes): a line of pairs per warp; the row stages' transposition
+// tile [rr][KP] reuses that memory, and so do the residues' inverse
 // transforms that the combine step reads. Every stage takes the same amount.
-__host__ __device__ constexpr size_t s3_lines_smem() { return size_t(kS3Units) * 3 * 2 * kS3LP * sizeof(float2); }
-__host__ __device__ constexpr size_t s3_tile_smem() { return size_t(2) * kS3Units * kS3KP * sizeof(float2); }
+__host__ __device__ constexpr size_t s3_lines_smem() { return size_t(kS3Units) * 3 * kS3LP * sizeof(cpair); }
+__host__ __device__ constexpr size_t s3_tile_smem() { return size_t(kS3Units) * kS3KP * sizeof(cpair); }
 __host__ __device__ constexpr size_t s3_smem() {
   return s3_lines_smem() > s3_tile_smem() ? s3_lines_smem() : s3_tile_smem();
 }
@@ -43,12 +43,12 @@ struct WarpSync {
   __device__ __forceinline__ void operator()() const { __syncwarp(); }
 };
 
-// The folded, twiddled input of residue q of both components at the thread's points
-// i = t + m T (m < 8): W_L^{iq} (x_c(i) + W_3^q x_c(i + M)), from a reader x(c, j) of the line's
+// The folded, twiddled input of residue q (both components) at the thread's points
+// i = t + m T (m < 8): W_L^{iq} (x(i) + W_3^q x(i + M)), from a reader x(j) of the line's
 // points (zero where j >= n). W_L^{iq} = W_L^{tq} W_24^{mq} (T = 32 = L / 24): one per-thread table
 // load and a warp-uniform one per m, instead of a 32-byte-strided load per point.
 template <typename Read>
-__device__ __forceinline__ void s3_fold(float2 (&v)[2][8], int t, int q, int n, const float2 *tw, Read &&x) {
+__device__ __forceinline__ void s3_fold(cpair (&v)[8], int t, int q, int n, const float2 *tw, Read &&x) {
   using C = float2;
   const C w3 = __ldg(tw + q * kS3Third);                  // W_3^q
   const C wt = __ldg(tw + ((t * q) % kS3L) * kS3Tw);      // W_L^{tq}
@@ -56,12 +56,9 @@ __device__ __forceinline__ void s3_fold(float2 (&v)[2][8], int t, int q, int n, 
   for (int m = 0; m < 8; ++m) {
     const int i = t + m * kS3T;
     const C wm = cmul(wt, __ldg(tw + ((m * q) % 24) * (kTwiddleN / 24)));  // W_L^{iq}
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      C a = i < n ? x(c, i) : czero<C>();
-      if (m < 4 && i + kS3M < n) a = cadd(a, cmul(w3, x(c, i + kS3M)));
-      v[c][m] = cmul(a, wm);
-    }
+    cpair a = i < n ? x(i) : pzero();
+    if (m < 4 && i + kS3M < n) a = hadd(a, hmul(x(i + kS3M), w3));
+    v[m] = hmul(a, wm);
   }
 }
 
@@ -69,18 +66,15 @@ __device__ __forceinline__ void s3_fold(float2 (&v)[2][8], int t, int q, int n, 
 // order) combined: y_j = sum_q W_L^{-jq} v_q[j mod M] for the unit's points j = u + 96 i (i < 4).
 // The warps first store v_q into their own lines; one CTA barrier later every thread reads the
 // three residues of its points. Every thread of the CTA must call it.
-__device__ __forceinline__ void s3_combine(const float2 (&v)[2][8], float2 *smem, int w, int t, const float2 *tw,
-                                           float2 (&y)[2][4]) {
+__device__ __forceinline__ void s3_combine(const cpair (&v)[8], cpair *smem, int w, int t, const float2 *tw,
+                                           cpair (&y)[4]) {
   using C = float2;
-  C *own = smem + size_t(2 * w) * kS3LP;
+  cpair *own = smem + size_t(w) * kS3LP;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    own[t + m * kS3T] = v[0][m];
-    own[kS3LP + t + m * kS3T] = v[1][m];
-  }
+  for (int m = 0; m < 8; ++m) own[t + m * kS3T] = v[m];
   __syncthreads();
   const int unit = w / 3, u = threadIdx.x - unit * kS3UnitThreads;
-  const C *base = smem + size_t(6 * unit) * kS3LP;  // lines of warps 3 unit + q: [q][c][LP]
+  const cpair *base = smem + size_t(3 * unit) * kS3LP;  // lines of warps 3 unit + q
   // W_L^{-j} = W_L^{-u} W_8^{-i} and W_L^{-2j} = W_L^{-2u} W_4^{-i} for j = u + 96 i (96 = L / 8)
   const C wu1 = cconj(__ldg(tw + u * kS3Tw)), wu2 = cconj(__ldg(tw + 2 * u * kS3Tw));
 #pragma unroll
@@ -88,11 +82,7 @@ __device__ __forceinline__ void s3_combine(const float2 (&v)[2][8], float2 *smem
     const int j = u + i * kS3UnitThreads, jm = j & (kS3M - 1);
     const C w1 = i ? cmulc(wu1, __ldg(tw + i * (kTwiddleN / 8))) : wu1;
     const C w2 = i ? cmulc(wu2, __ldg(tw + i * (kTwiddleN / 4))) : wu2;
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const C v0 = base[c * kS3LP + jm], v1 = base[(2 + c) * kS3LP + jm], v2 = base[(4 + c) * kS3LP + jm];
-      y[c][i] = cadd(v0, cadd(cmul(w1, v1), cmul(w2, v2)));
-    }
+    y[i] = hadd(base[jm], hadd(hmul(base[kS3LP + jm], w1), hmul(base[2 * kS3LP + jm], w2)));
   }
 }
 
@@ -110,44 +100,39 @@ __device__ __forceinline__ void cols_tile_s3(const A &a, int tile, float2 *smem)
   const int nz = a.nz(), lx = a.lx();
   const bool live = kx < lx;
   const C *tw = a.tw();
-  C *col[2] = {a.T() + size_t(kx) * nz, a.T() + (size_t(lx) + kx) * nz};
+  cpair *col = reinterpret_cast<cpair *>(a.T()) + size_t(kx) * nz;
+  cpair *ps = reinterpret_cast<cpair *>(smem);
   const TwReg<C, kS3M, 0> tr(t, tw);
   const int n = live ? nz : 0;
-  C v[2][8];
-  s3_fold(v, t, q, n, tw, [&](int c, int j) { return col[c][j]; });
-  C *const lines[2] = {smem + size_t(2 * w) * kS3LP, smem + size_t(2 * w + 1) * kS3LP};
-  RegPlan<kS3M, 0>::template run<C, 2, false>(v, lines, t, tr, WarpSync{});
+  cpair v[1][8];
+  s3_fold(v[0], t, q, n, tw, [&](int j) { return col[j]; });
+  cpair *const lines[1] = {ps + size_t(w) * kS3LP};
+  RegPlan<kS3M, 0>::template run<cpair, 1, false>(v, lines, t, tr, WarpSync{});
   if (live) {
     const size_t plane = size_t(lx) * kS3L;
     const C *G = a.G() + size_t(kx) * kS3L + q * kS3M;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int k = t + m * kS3T;
-      const C g11 = __ldg(G + k), g13 = __ldg(G + plane + k), g33 = __ldg(G + 2 * plane + k);
-      const C s1 = v[0][m], s3 = v[1][m];
-      v[0][m] = cadd(cmul(g11, s1), cmul(g13, s3));
-      v[1][m] = cadd(cmul(g13, s1), cmul(g33, s3));
+      v[0][m] = green_product(v[0][m], __ldg(G + k), __ldg(G + plane + k), __ldg(G + 2 * plane + k));
     }
   }
-  RegPlan<kS3M, 0>::template run<C, 2, true>(v, lines, t, tr, WarpSync{});
-  C y[2][4];
-  s3_combine(v, smem, w, t, tw, y);
+  RegPlan<kS3M, 0>::template run<cpair, 1, true>(v, lines, t, tr, WarpSync{});
+  cpair y[4];
+  s3_combine(v[0], ps, w, t, tw, y);
   if (live) {
     const int u = threadIdx.x - cc * kS3UnitThreads;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int z = u + i * kS3UnitThreads;
-      if (z < nz) {
-        col[0][z] = y[0][i];
-        col[1][z] = y[1][i];
-      }
+      if (z < nz) col[z] = y[i];
     }
   }
 }
 
 // Rows z0 .. z0 + 3: warp (row, q) folds the row (the source rows from the stencil kernel, or the
-// raw input times its scale) and transforms it (the spectra at kx = 3k + q); both components go
-// through the transposition tile into the column-major spectra T[c][kx][z] in runs of four rows.
+// raw input times its scale) and transforms it (the spectra at kx = 3k + q); the pairs go through the
+// transposition tile into the column-major spectra T[kx][z] in runs of four rows.
 template <typename A>
 __device__ __forceinline__ void rows_forward_tile_s3(const A &a, int tile, float2 *smem, const float2 *src,
                                                      float scale) {
@@ -161,32 +146,30 @@ __device__ __forceinline__ void rows_forward_tile_s3(const A &a, int tile, float
   const TwReg<C, kS3M, 0> tr(t, tw);
   const int n = z < nz ? nx : 0;
   const C *row = src + size_t(z < nz ? z : 0) * nx;
-  C v[2][8];
-  s3_fold(v, t, q, n, tw, [&](int c, int j) { return cscale(__ldg(row + c * plane + j), scale); });
-  C *const lines[2] = {smem + size_t(2 * w) * kS3LP, smem + size_t(2 * w + 1) * kS3LP};
-  RegPlan<kS3M, 0>::template run<C, 2, false>(v, lines, t, tr, WarpSync{});
-  __syncthreads();  // every warp is done with its lines: the tile reuses their memory
+  cpair *ps = reinterpret_cast<cpair *>(smem);
+  cpair v[1][8];
+  s3_fold(v[0], t, q, n, tw,
+          [&](int j) { return mkpair(cscale(__ldg(row + j), scale), cscale(__ldg(row + plane + j), scale)); });
+  cpair *const lines[1] = {ps + size_t(w) * kS3LP};
+  RegPlan<kS3M, 0>::template run<cpair, 1, false>(v, lines, t, tr, WarpSync{});
+  __syncthreads();  // every warp is done with its line: the tile reuses their memory
+  cpair *trow = ps + size_t(rr) * kS3KP;
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    C *trow = smem + size_t(c * kS3Units + rr) * kS3KP;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) trow[3 * (t + m * kS3T) + q] = v[c][m];
-  }
+  for (int m = 0; m < 8; ++m) trow[3 * (t + m * kS3T) + q] = v[0][m];
   __syncthreads();
-  const size_t cplane = size_t(a.lx()) * nz;
-  constexpr int NST = 2 * kS3L * kS3Units / kS3Threads;  // 16 stores per thread
-  const int r = threadIdx.x % kS3Units;                  // the same row for all of a thread's stores
+  constexpr int NST = kS3L * kS3Units / kS3Threads;  // 8 stores per thread
+  const int r = threadIdx.x % kS3Units;              // the same row for all of a thread's stores
   if (z0 + r < nz) {
+    cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0 + r;
 #pragma unroll
     for (int i = 0; i < NST; ++i) {
-      const int idx = threadIdx.x + i * kS3Threads, kx = (idx / kS3Units) % kS3L, c = idx / (kS3Units * kS3L);
-      a.T()[c * cplane + size_t(kx) * nz + z0 + r] = smem[size_t(c * kS3Units + r) * kS3KP + kx];
+      const int kx = threadIdx.x / kS3Units + i * (kS3Threads / kS3Units);
+      Tp[size_t(kx) * nz] = ps[size_t(r) * kS3KP + kx];
     }
   }
 }
 
-// Rows z0 .. z0 + 3: the spectra T[c][kx][z0 .. z0 + 3] of both components through the
-// transposition tile, warp (row, q) the inverse transform of residue q, the residues combined
+// Rows z0 .. z0 + 3: the spectra T[kx][z0 .. z0 + 3] through the transposition tile, warp (row, q) the inverse transform of residue q, the residues combined
 // into y_x for x < nx, then the epilogue of rows_inverse_tile: out = ident - scale * y (or the
 // scaled y) with the fused inner products.
 template <int EPI, typename A>
@@ -198,35 +181,37 @@ __device__ __forceinline__ void rows_inverse_tile_s3(const A &a, int tile, float
   const int nz = a.nz(), nx = a.nx();
   const C *tw = a.tw();
   const TwReg<C, kS3M, 0> tr(t, tw);
-  const size_t cplane = size_t(a.lx()) * nz;
-  constexpr int NLD = 2 * kS3L * kS3Units / kS3Threads;  // 16 loads per thread
-  const int r = threadIdx.x % kS3Units;
+  cpair *ps = reinterpret_cast<cpair *>(smem);
+  constexpr int NLD = kS3L * kS3Units / kS3Threads;  // 8 copies per thread, all in flight
   {
-    C ld[NLD];
-#pragma unroll
-    for (int i = 0; i < NLD; ++i) {  // all loads in flight before the shared-memory stores
-      const int idx = threadIdx.x + i * kS3Threads, kx = (idx / kS3Units) % kS3L, c = idx / (kS3Units * kS3L);
-      ld[i] = z0 + r < nz ? a.T()[c * cplane + size_t(kx) * nz + z0 + r] : czero<C>();
-    }
+    const int r = threadIdx.x % kS3Units;
+    const bool in = z0 + r < nz;
+    const cpair *T0 = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
 #pragma unroll
     for (int i = 0; i < NLD; ++i) {
-      const int idx = threadIdx.x + i * kS3Threads, kx = (idx / kS3Units) % kS3L, c = idx / (kS3Units * kS3L);
-      smem[size_t(c * kS3Units + r) * kS3KP + kx] = ld[i];
+      const int kx = threadIdx.x / kS3Units + i * (kS3Threads / kS3Units);
+      cp_async16z(ps + size_t(r) * kS3KP + kx, T0 + size_t(kx) * nz, in);
     }
   }
+  cp_async_wait_all();
   __syncthreads();
-  C v[2][8];
+  cpair v[1][8];
+  {
+    const cpair *trow = ps + size_t(rr) * kS3KP;
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const C *trow = smem + size_t(c * kS3Units + rr) * kS3KP;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) v[c][m] = trow[3 * (t + m * kS3T) + q];
+    for (int m = 0; m < 8; ++m) v[0][m] = trow[3 * (t + m * kS3T) + q];
   }
   __syncthreads();  // the lines reuse the tile's memory
-  C *const lines[2] = {smem + size_t(2 * w) * kS3LP, smem + size_t(2 * w + 1) * kS3LP};
-  RegPlan<kS3M, 0>::template run<C, 2, true>(v, lines, t, tr, WarpSync{});
+  cpair *const lines[1] = {ps + size_t(w) * kS3LP};
+  RegPlan<kS3M, 0>::template run<cpair, 1, true>(v, lines, t, tr, WarpSync{});
+  cpair yp[4];
+  s3_combine(v[0], ps, w, t, tw, yp);
   C y[2][4];
-  s3_combine(v, smem, w, t, tw, y);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    y[0][i] = comp0(yp[i]);
+    y[1][i] = comp1(yp[i]);
+  }
   const int u = threadIdx.x - rr * kS3UnitThreads;
   const float osc = a.osc();
   const size_t base = size_t(z) * nx, fplane = size_t(nz) * nx;

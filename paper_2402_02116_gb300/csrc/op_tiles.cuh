@@ -23,7 +23,7 @@ namespace dbi {
 // thread (c, t) with t fastest so that a warp reads a contiguous run of one column.
 template <typename C> struct Cfg;
 #ifndef DBI_COLS_MIN_BLOCKS
-#define DBI_COLS_MIN_BLOCKS 4
+#define DBI_COLS_MIN_BLOCKS 3  // the pair columns spill at 64 registers
 #endif
 #ifndef DBI_ROWS_INV_MIN_BLOCKS
 #define DBI_ROWS_INV_MIN_BLOCKS 4
@@ -49,13 +49,23 @@ template <typename C, int LX> struct RowCfg {
   static constexpr int ROWS = kTileThreads / T;
   static constexpr int NT = ROWS * T;
   static constexpr int LP = RegFFT<C, LX>::LP;
+  // complex64: lines of pairs, and the transposition tile [ROWS][KP] of pairs. A quarter warp's
+  // 16-byte accesses hit 8 distinct bank slots both along a row (consecutive kx) and down the tile
+  // (min(ROWS, 8) rows x consecutive kx).
+  static constexpr int PLP = RegFFT<cpair, LX>::LP;
+  static constexpr int KP = LX + (ROWS >= 8 ? 1 : 8 / ROWS);
 };
 template <typename C, int LZ> struct ColCfg {
   static constexpr int T = LZ / 8;
   static constexpr int CC = kTileThreads / T;  // named barriers 1..CC only when T > 32 (CC <= 4)
   static constexpr int NT = CC * T;
   static constexpr int LP = RegFFT<C, LZ>::LP;
+  static constexpr int PLP = RegFFT<cpair, LZ>::LP;
 };
+// The spectra T of complex64 problems are [lx][nz] pairs (both components of a point in 16 bytes:
+// fft_pair.cuh); those of complex128 problems [2][lx][nz].
+template <typename C> constexpr bool kPairSpectra = sizeof(C) == sizeof(float2);
+
 // Every line holds its data in its first half: the entry points require lz >= 2 nz - 1 and
 // lx >= 2 nx - 1, so a cell index t + m L/8 < n <= L/2 has m < 4. Points m = 4..7 are zero on
 // input to a forward transform and never needed on output of an inverse one.
@@ -86,8 +96,9 @@ template <typename C, int LX> inline size_t stencil_strip_smem(int nx) {
 // Dynamic shared memory of each stage (bytes).
 template <typename C, int LX> inline size_t rows_forward_smem(int nx, bool stencil) {
   using RC = RowCfg<C, LX>;
-  const size_t lines = size_t(2) * RC::ROWS * RC::LP * sizeof(C);
-  const size_t tile = tile_elems<C, LX>() * sizeof(C);
+  const size_t lines = kPairSpectra<C> ? size_t(RC::ROWS) * RC::PLP * sizeof(cpair)
+                                       : size_t(2) * RC::ROWS * RC::LP * sizeof(C);
+  const size_t tile = kPairSpectra<C> ? size_t(RC::ROWS) * RC::KP * sizeof(cpair) : tile_elems<C, LX>() * sizeof(C);
   size_t sg = 0;
   if (stencil) {
     if constexpr (kStripStencil<C, LX>) sg = stencil_strip_smem<C, LX>(nx);
@@ -97,10 +108,11 @@ template <typename C, int LX> inline size_t rows_forward_smem(int nx, bool stenc
 }
 template <typename C, int LZ> inline size_t cols_smem() {
   using CF = ColCfg<C, LZ>;
-  return size_t(2) * CF::CC * CF::LP * sizeof(C);
+  return kPairSpectra<C> ? size_t(CF::CC) * CF::PLP * sizeof(cpair) : size_t(2) * CF::CC * CF::LP * sizeof(C);
 }
 template <typename C, int LX> inline size_t rows_inverse_smem() {
   using RC = RowCfg<C, LX>;
+  if (kPairSpectra<C>) return size_t(RC::ROWS) * std::max(RC::PLP, RC::KP) * sizeof(cpair);
   return std::max(size_t(2) * RC::ROWS * RC::LP, tile_elems<C, LX>()) * sizeof(C);
 }
 
@@ -305,6 +317,35 @@ __device__ __forceinline__ void stencil_strip(const A &a, int z0, C *smem, C (&v
   __syncthreads();  // the FFT lines reuse the buffers
 }
 
+// Forward FFT along x of the tile's rows of pairs (thread (rr, t) holds the points t + m T of row
+// rr in v, both components) and their transposition into T[kx][z] in runs of ROWS pairs. No thread
+// reads the staging memory any more.
+template <int LX, int V, typename A>
+__device__ __forceinline__ void rows_forward_pairs(const A &a, int z0, int rr, int t, const float2 (&v)[2][8],
+                                                   cpair *smem, const TwReg<float2, LX, V> &tr) {
+  using RC = RowCfg<float2, LX>;
+  constexpr int ROWS = RC::ROWS, T = RC::T, KP = RC::KP;
+  const int nz = a.nz();
+  cpair p[1][8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) p[0][m] = mkpair(v[0][m], v[1][m]);
+  cpair *const line[1] = {smem + size_t(rr) * RC::PLP};
+  RegPlan<LX, V>::template run<cpair, 1, false, true>(p, line, t, tr, RowSync<T>{1 + rr});
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < 8; ++m) smem[size_t(rr) * KP + t + m * T] = p[0][m];
+  __syncthreads();
+  cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0;
+  const int r = threadIdx.x % ROWS;
+  if (z0 + r < nz) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int kx = threadIdx.x / ROWS + i * (RC::NT / ROWS);
+      Tp[size_t(kx) * nz + r] = smem[size_t(r) * KP + kx];
+    }
+  }
+}
+
 // Contrast source (or the raw source) of ROWS rows, zero-padded to LX, forward FFT along x.
 //   stencil: stress of rows z0-1 .. z0+ROWS (each computed once, kept in shared memory), then
 //            s1 = w^2 drho u1 + d1 sigma1 + d3 sigma5, s3 = w^2 drho u3 + d1 sigma5 + d3 sigma3.
@@ -401,6 +442,10 @@ __device__ __forceinline__ void rows_forward_tile(const A &a, int tile, C *smem)
       v[1][m] = in ? cscale(__ldg(u3 + size_t(z) * nx + x), isc) : czero<C>();
     }
   }
+  if constexpr (kPairSpectra<C>) {
+    rows_forward_pairs<LX, V>(a, z0, rr, t, v, reinterpret_cast<cpair *>(smem), tr);
+    return;
+  }
   C *const lines[2] = {smem + size_t(rr) * LP, smem + size_t(ROWS + rr) * LP};
   RegPlan<LX, V>::template run<C, 2, false, true>(v, lines, t, tr, RowSync<T>{1 + rr});
   // transpose through shared memory: tile[c][kx][rr], then ROWS consecutive z per kx
@@ -417,11 +462,72 @@ __device__ __forceinline__ void rows_forward_tile(const A &a, int tile, C *smem)
   }
 }
 
+// (g11 s1 + g13 s3, g13 s1 + g33 s3) of the pair (s1, s3)
+__device__ __forceinline__ cpair green_product(const cpair &v, float2 g11, float2 g13, float2 g33) {
+  const float2 s1 = comp0(v), s3 = comp1(v);
+  return mkpair(cadd(cmul(g11, s1), cmul(g13, s3)), cadd(cmul(g13, s1), cmul(g33, s3)));
+}
+
 // For CC columns kx: forward FFT along z of the nz non-zero rows padded to LZ, 2x2 multiply by
 // Ghat(kz, kx), inverse FFT along z, keep z < nz. Thread (col, t), t fastest: a warp reads a
 // contiguous run of one column; the T threads of a column share a barrier.
+// Column kx of one problem (both components), by the T threads of unit `u` of the CTA. Ghat(:, kx)
+// comes from Gs (the column's three tables staged in shared memory, [3][LZ]) or, when Gs is null,
+// from global memory; STAGED: every thread of the CTA (live or not) waits for the staging copies
+// between the transforms. `live` is uniform over the unit.
+template <int LZ, int V, bool STAGED, typename A>
+__device__ __forceinline__ void cols_unit_pairs(const A &a, int kx, int u, int t, bool live, cpair *smem,
+                                                const float2 *Gs) {
+  using CF = ColCfg<float2, LZ>;
+  constexpr int T = CF::T;
+  const int nz = a.nz(), lx = a.lx();
+  cpair *c = reinterpret_cast<cpair *>(a.T()) + size_t(kx) * nz;
+  const TwReg<float2, LZ, V> tr(t, a.tw());
+  cpair v[1][8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const int z = t + m * T;
+    v[0][m] = (m < kHalf && live && z < nz) ? c[z] : pzero();
+  }
+  cpair *const line[1] = {smem + size_t(u) * CF::PLP};
+  RegPlan<LZ, V>::template run<cpair, 1, false, true>(v, line, t, tr, RowSync<T>{1 + u});
+  if constexpr (STAGED) {
+    cp_async_wait_all();
+    __syncthreads();
+  }
+  if (live) {
+    const size_t plane = size_t(lx) * LZ;
+    const float2 *G = a.G() + size_t(kx) * LZ;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int kz = t + m * T;
+      float2 g11, g13, g33;
+      if (STAGED && Gs) {
+        g11 = Gs[kz]; g13 = Gs[LZ + kz]; g33 = Gs[2 * LZ + kz];
+      } else {
+        g11 = __ldg(G + kz); g13 = __ldg(G + plane + kz); g33 = __ldg(G + 2 * plane + kz);
+      }
+      v[0][m] = green_product(v[0][m], g11, g13, g33);
+    }
+  }
+  RegPlan<LZ, V>::template run<cpair, 1, true>(v, line, t, tr, RowSync<T>{1 + u});
+  if (live) {
+#pragma unroll
+    for (int m = 0; m < kHalf; ++m) {
+      const int z = t + m * T;
+      if (z < nz) c[z] = v[0][m];
+    }
+  }
+}
+
 template <typename C, int LZ, int V, typename A>
 __device__ __forceinline__ void cols_tile(const A &a, int tile, C *smem) {
+  if constexpr (kPairSpectra<C>) {
+    constexpr int CC = ColCfg<C, LZ>::CC, T = ColCfg<C, LZ>::T;
+    const int u = threadIdx.x / T, kx = tile * CC + u;
+    cols_unit_pairs<LZ, V, false>(a, kx, u, threadIdx.x - u * T, kx < a.lx(), reinterpret_cast<cpair *>(smem), nullptr);
+    return;
+  }
   using CF = ColCfg<C, LZ>;
   constexpr int CC = CF::CC, T = CF::T, LP = CF::LP;
   const int col = threadIdx.x / T, t = threadIdx.x - col * T;
@@ -477,6 +583,34 @@ __device__ __forceinline__ void rows_inverse_tile(const A &a, int tile, C *smem)
   const int nz = a.nz(), nx = a.nx();
   const int rr = threadIdx.x / T, t = threadIdx.x - rr * T, z = z0 + rr;
   const TwReg<C, LX, V> tr(t, a.tw());
+  C v[2][8];
+  if constexpr (kPairSpectra<C>) {
+    // ROWS consecutive z of every kx into tile[r][kx] by asynchronous copies (zeros beyond nz), then
+    // each thread takes its row
+    constexpr int KP = RC::KP;
+    cpair *tile_p = reinterpret_cast<cpair *>(smem);
+    const int r = threadIdx.x % ROWS;
+    const bool in = z0 + r < nz;
+    const cpair *Tp = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int kx = threadIdx.x / ROWS + i * (RC::NT / ROWS);
+      cp_async16z(tile_p + size_t(r) * KP + kx, Tp + size_t(kx) * nz, in);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    cpair p[1][8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) p[0][m] = tile_p[size_t(rr) * KP + t + m * T];
+    __syncthreads();  // the FFT lines reuse the tile
+    cpair *const line[1] = {tile_p + size_t(rr) * RC::PLP};
+    RegPlan<LX, V>::template run<cpair, 1, true>(p, line, t, tr, RowSync<T>{1 + rr});
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      v[0][m] = comp0(p[0][m]);
+      v[1][m] = comp1(p[0][m]);
+    }
+  } else {
   // ROWS consecutive z of every (c, kx) into tile[c][kx][r], then each thread takes its row
   constexpr int RP = ROWS + 1, NLD = 2 * LX * ROWS / RC::NT;
   static_assert((2 * LX * ROWS) % RC::NT == 0, "tile load");
@@ -494,7 +628,6 @@ __device__ __forceinline__ void rows_inverse_tile(const A &a, int tile, C *smem)
     }
   }
   __syncthreads();
-  C v[2][8];
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
@@ -502,6 +635,7 @@ __device__ __forceinline__ void rows_inverse_tile(const A &a, int tile, C *smem)
   __syncthreads();  // the FFT lines reuse the tile
   C *const lines[2] = {smem + size_t(rr) * LP, smem + size_t(ROWS + rr) * LP};
   RegPlan<LX, V>::template run<C, 2, true>(v, lines, t, tr, RowSync<T>{1 + rr});
+  }
   const Rl osc = a.osc();
   const size_t base = size_t(z) * nx;
   // per-thread partials of the fused inner products: FP32 for complex64, FP64 for complex128
