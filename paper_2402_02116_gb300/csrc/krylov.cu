@@ -4,21 +4,26 @@
 // Per iteration i (van der Vorst's BiCGSTAB, <a, b> = sum conj(a) b):
 //   p = r + beta (p - omega v)                  k_update_p      (beta from the previous k_check)
 //   v = A p, partials of <rhat, v>              operator (inner product in k_rows_inverse)
-//   alpha = rho / <rhat, v>                     k_alpha         (one warp per problem)
+//   alpha = rho / <rhat, v>                     the last CTA of each problem's k_rows_inverse (k_alpha
+//                                               for uneven batches and the paper-literal form)
 //   s = r - alpha v                             k_update_s      (+ partials of ||s||^2)
 //   t = A s, partials of <t, s>, <t, t>         operator (inner products in k_rows_inverse)
-//   omega = <t,s>/<t,t>                         k_omega         (one warp per problem)
+//   omega = <t,s>/<t,t>                         likewise (k_omega)
 //   x += alpha p + omega s, r = s - omega t     k_update_xr     (+ partials of <rhat, r>, ||r||^2)
-//   convergence, breakdown, beta = (rho_new / rho)(alpha / omega)  k_check
+//   convergence, breakdown, beta = (rho_new / rho)(alpha / omega)  the last CTA of each problem's k_update_xr
+// The scalar steps as kernels of their own took 4.8 to 6.7 us each (one warp gathering 64 partials
+// behind a launch), 13 % of a 45 x 180 solve's iteration.
 // Every scalar lives on the device in FP64. Each reduction is two-stage and deterministic: each
 // thread sums its elements, the CTA sums its threads in a fixed tree, and every consumer sums the
-// kRedBlocks CTA partials of its problem in the same fixed order. Converged problems drop out
+// CTA partials of its problem in the same fixed order. Converged problems drop out
 // (their CTAs return at once); the host polls an active-problem counter every check_every
 // iterations. A breakdown (rho or omega vanishing) restarts the problem from its iterate.
 #include <cmath>
+#include <type_traits>
 
 #include "group.cuh"
 #include "krylov.cuh"
+#include "krylov_finish.cuh"
 #include "reduce.cuh"
 #include "vec.cuh"
 
@@ -38,14 +43,23 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_absmax(Span sp, const T *x, double *part) {
   const int b = blockIdx.y;
   decltype(absmax(T{})) m = 0;
-  DBI_PROBLEM_LOOP(sp) m = fmax(m, absmax(x[off + i]));
-  block_max_store(double(m), part + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
+  if constexpr (std::is_same_v<T, float2>) {
+    problem_loop_pairs<T>(sp, b, [&]<int N>(size_t o) {
+      T v[N];
+      ldN(x + o, v);
+#pragma unroll
+      for (int n = 0; n < N; ++n) m = max_of(m, absmax(v[n]));
+    });
+  } else {
+    DBI_PROBLEM_LOOP(sp) m = max_of(m, absmax(x[off + i]));
+  }
+  block_max_store(m, part + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
 }
 
 // Power-of-two scale per problem that brings max |rhs| into [1, 2); the solver iterates on the
 // scaled system (exact in any precision) and unscales the solution at the end.
-__global__ void k_scale(KState *st, const double *part) {
-  const double m = gather_max(part + size_t(blockIdx.x) * kRedBlocks * kRedSlots, kRedBlocks);
+__global__ void k_scale(KState *st, const double *part, int nblk) {
+  const double m = gather_max(part + size_t(blockIdx.x) * kRedBlocks * kRedSlots, nblk);
   if (threadIdx.x == 0) st[blockIdx.x].scale = pow2_below(m);
 }
 
@@ -54,8 +68,13 @@ template <typename C>
 __global__ void k_scale_x(Span sp, const KState *st, C *x, int inverse) {
   const int b = blockIdx.y;
   using R = typename RealOf<C>::type;
-  const double sc = st[blockIdx.y].scale;
-  const R f = R(inverse ? 1.0 / sc : sc);
+  __shared__ R sf;  // one FP64 division per CTA, not per thread
+  if (threadIdx.x == 0) {
+    const double sc = st[blockIdx.y].scale;
+    sf = R(inverse ? 1.0 / sc : sc);
+  }
+  __syncthreads();
+  const R f = sf;
   DBI_PROBLEM_LOOP(sp) x[off + i] = cscale(x[off + i], f);
 }
 
@@ -85,12 +104,13 @@ __global__ void __launch_bounds__(kRedThreads) k_init(Span sp, const KState *st,
   block_sum_store<2>(acc, part + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
 }
 
-__global__ void k_init_state(KState *st, int *active, int *counters, const double *part, double tol,
-                             int max_iter) {
+__global__ void k_init_state(KState *st, int *active, int *counters, int *arrived, const double *part, int nblk,
+                             double tol, int max_iter) {
   const int b = blockIdx.x;
   double s[2];
-  gather_n<2>(part + size_t(b) * kRedBlocks * kRedSlots, kRedBlocks, s);
+  gather_n<2>(part + size_t(b) * kRedBlocks * kRedSlots, nblk, s);
   if (threadIdx.x == 0) {
+    arrived[b] = 0;
     KState k{};
     k.scale = st[b].scale;
     k.bnorm2 = s[0];
@@ -103,6 +123,7 @@ __global__ void k_init_state(KState *st, int *active, int *counters, const doubl
     const bool bad = !finite_value(s[0]) || !finite_value(s[1]);  // NaN or infinity in the right-hand side or x0
     const bool conv = !bad && (k.zero_rhs || s[1] <= tol * tol * s[0]);
     k.code = bad ? DBI_NONFINITE : conv ? DBI_CONVERGED : DBI_NOT_CONVERGED;
+    round_state(k);
     st[b] = k;
     const int act = (!bad && !conv && max_iter > 0) ? 1 : 0;
     active[b] = act;
@@ -125,7 +146,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_p(Span sp, const int *pl
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) counters[parity] = 0;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
-  const KState k = st[b];
+  const KState &k = st[b];
   if (k.restart) {
     problem_loop_pairs<C>(sp, b, [&]<int N>(size_t o) {
       C ri[N];
@@ -135,8 +156,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_p(Span sp, const int *pl
     });
     return;
   }
-  const C be = from_z<C>(make_double2(k.beta_re, k.beta_im));
-  const C om = from_z<C>(make_double2(k.om_re, k.om_im));
+  const C be = state_beta<C>(k), om = state_omega<C>(k);
   problem_loop_pairs<C>(sp, b, [&]<int N>(size_t o) {
     C pi[N], vi[N], ri[N];
     ldN(p + o, pi);
@@ -148,21 +168,11 @@ __global__ void __launch_bounds__(kRedThreads) k_update_p(Span sp, const int *pl
   });
 }
 
-// alpha = rho / <rhat, A p> of every active problem, from the operator's fused partials, once
-// per problem (one warp each) so that the s update starts streaming at once.
+// alpha of every active problem (one warp each): the paths whose operator does not finish it.
 __global__ void k_alpha(const int *plist, KState *st, const int *active, int nparts, const double *partA) {
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
-  double sg[2];
-  gather_n<2>(partA + size_t(b) * nparts * kRedSlots, nparts, sg);
-  if (threadIdx.x == 0) {
-    const double2 sigma = make_double2(sg[0], sg[1]);
-    const double2 alpha = (sigma.x == 0.0 && sigma.y == 0.0)
-                              ? make_double2(0.0, 0.0)
-                              : zdiv(make_double2(st[b].rho_re, st[b].rho_im), sigma);
-    st[b].alpha_re = alpha.x;
-    st[b].alpha_im = alpha.y;
-  }
+  finish_alpha(st, b, partA + size_t(b) * nparts * kRedSlots, nparts);
 }
 
 template <typename C>
@@ -173,7 +183,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_s(Span sp, const int *pl
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
-  const C al = from_z<C>(make_double2(st[b].alpha_re, st[b].alpha_im));
+  const C al = state_alpha<C>(st[b]);
   A ss = 0;
   problem_loop_pairs<C>(sp, b, [&]<int N>(size_t o) {
     C ri[N], vi[N];
@@ -190,38 +200,26 @@ __global__ void __launch_bounds__(kRedThreads) k_update_s(Span sp, const int *pl
   block_sum_store<1>(acc, partS + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
 }
 
-// omega = <t, s> / ||t||^2 (zero when the half step already met tol) of every active problem,
-// once per problem (one warp each), from the second operator pass's partials and ||s||^2.
+// omega of every active problem (one warp each), likewise.
 __global__ void k_omega(const int *plist, KState *st, const int *active, int nparts, const double *partB,
-                        const double *partS, double tol) {
+                        const double *partS, int nS, double tol) {
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
-  double q[3], sn[1];
-  gather_n<3>(partB + size_t(b) * nparts * kRedSlots, nparts, q);
-  gather_n<1>(partS + size_t(b) * kRedBlocks * kRedSlots, kRedBlocks, sn);
-  if (threadIdx.x == 0) {
-    const int half = sn[0] <= tol * tol * st[b].bnorm2;
-    const double2 om = (half || q[2] == 0.0) ? make_double2(0.0, 0.0)
-                                             : make_double2(q[0] / q[2], q[1] / q[2]);
-    st[b].om_re = om.x;
-    st[b].om_im = om.y;
-    st[b].half = half;
-    st[b].snorm2 = sn[0];
-  }
+  finish_omega(st, b, partB + size_t(b) * nparts * kRedSlots, nparts, partS + size_t(b) * kRedBlocks * kRedSlots, nS,
+               tol);
 }
 
 template <typename C>
-__global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *plist, const KState *st,
-                                                           const int *active, const C *__restrict__ p,
+__global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *plist, KState *st, int *active,
+                                                           int *counters, int parity, int *arrived, double tol,
+                                                           int max_iter, const C *__restrict__ p,
                                                            const C *__restrict__ s, const C *__restrict__ t,
                                                            const C *__restrict__ rhat, C *__restrict__ x,
                                                            C *__restrict__ r, double *partC) {
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
-  const KState k = st[b];
-  const C al = from_z<C>(make_double2(k.alpha_re, k.alpha_im));
-  const C o = from_z<C>(make_double2(k.om_re, k.om_im));
+  const C al = state_alpha<C>(st[b]), o = state_omega<C>(st[b]);
   A re = 0, im = 0, rr = 0;
   problem_loop_pairs<C>(sp, b, [&]<int N>(size_t e) {
     C si[N], xi[N], pi[N], ti[N], hi[N];
@@ -243,20 +241,17 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *p
     stN(r + e, si);
   });
   A acc[3] = {re, im, rr};
-  block_sum_store<3>(acc, partC + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
-}
-
-// Convergence test, breakdown restart and beta for the next iteration (one CTA per problem;
-// the decision itself is bicgstab_decide in krylov.cuh).
-__global__ void k_check(const int *plist, KState *st, int *active, int *counters, int parity,
-                        const double *partC, double tol, int max_iter) {
-  const int b = problem_at(plist, blockIdx.x);
-  if (!active[b]) return;
+  double *pb = partC + size_t(b) * kRedBlocks * kRedSlots;
+  block_sum_store<3>(acc, pb + size_t(blockIdx.x) * kRedSlots);
+  // convergence test, breakdown restart and beta for the next iteration, by the problem's last CTA
+  // (the decision itself is bicgstab_decide in krylov.cuh)
+  if (!last_cta(arrived + b, gridDim.x)) return;
   double q[3];
-  gather_n<3>(partC + size_t(b) * kRedBlocks * kRedSlots, kRedBlocks, q);
+  gather_n<3>(pb, gridDim.x, q);
   if (threadIdx.x != 0) return;
   KState k = st[b];
   const int act = bicgstab_decide(k, q, tol, max_iter);
+  round_state(k);
   st[b] = k;
   active[b] = act;
   atomicAdd(&counters[parity], act);
@@ -306,8 +301,8 @@ __global__ void k_finalize(int B, const KState *st, int *iters, double *relres, 
 // ---------------------------------------------------------------------------------------------
 // power-of-two normalisers
 // ---------------------------------------------------------------------------------------------
-__global__ void k_pow2(const double *part, double *scale, double *inv, const double *extra) {
-  const double m = gather_max(part + size_t(blockIdx.x) * kRedBlocks * kRedSlots, kRedBlocks);
+__global__ void k_pow2(const double *part, int nblk, double *scale, double *inv, const double *extra) {
+  const double m = gather_max(part + size_t(blockIdx.x) * kRedBlocks * kRedSlots, nblk);
   if (threadIdx.x == 0) {
     const double sc = pow2_below(m);
     scale[blockIdx.x] = sc;
@@ -317,7 +312,8 @@ __global__ void k_pow2(const double *part, double *scale, double *inv, const dou
 
 int pow2_scales(const void *x, int precision, bool real, int B, size_t n, double *part, double *scale,
                 double *inv, const double *extra, cudaStream_t s, const long long *offs) {
-  const dim3 grid(kRedBlocks, B);
+  const int nblk = offs ? kRedBlocks : red_blocks(n, B, precision);
+  const dim3 grid(nblk, B);
   const Span sp{n, offs};
   if (precision == DBI_C64) {
     if (real) k_absmax<float><<<grid, kRedThreads, 0, s>>>(sp, static_cast<const float *>(x), part);
@@ -328,7 +324,7 @@ int pow2_scales(const void *x, int precision, bool real, int B, size_t n, double
   }
   int rc;
   if ((rc = check_launch("k_absmax"))) return rc;
-  k_pow2<<<B, 32, 0, s>>>(part, scale, inv, extra);
+  k_pow2<<<B, 32, 0, s>>>(part, nblk, scale, inv, extra);
   return check_launch("k_pow2");
 }
 
@@ -352,6 +348,9 @@ SolverBufs carve_solver_fields(Arena &ar, size_t f, int B) {
   sb.partS = static_cast<double *>(ar.take(bytes_partials(B)));
   sb.partB = static_cast<double *>(ar.take(bytes_partials(B)));
   sb.partC = static_cast<double *>(ar.take(bytes_partials(B)));
+  // partC uses kRedBlocks of the kMaxParts partials per problem that its carve holds
+  static_assert(kMaxParts >= 2 * kRedBlocks, "room for the CTA counters");
+  if (sb.partC) sb.arrived = reinterpret_cast<int *>(sb.partC + size_t(B) * kRedBlocks * kRedSlots);
   return sb;
 }
 SolverBufs carve_solver(Arena &ar, const dbi_grid *g, int B, int precision) {
@@ -388,18 +387,23 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   C *x = static_cast<C *>(x_);
   C *r = static_cast<C *>(sb.r), *rhat = static_cast<C *>(sb.rhat), *p = static_cast<C *>(sb.p);
   C *v = static_cast<C *>(sb.v), *sv = static_cast<C *>(sb.s), *t = static_cast<C *>(sb.t);
-  const dim3 grid(kRedBlocks, B);
+  const int nblk = group ? kRedBlocks : red_blocks(sp.n, B, op.precision);  // CTAs per problem of the vector kernels
+  const dim3 grid(nblk, B);
   int rc;
   cudaError_t e = cudaMemsetAsync(sb.counters, 0, 3 * sizeof(int), s);
   if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync(counters)", e);
   const int nparts = group    ? group_parts(op.group)
                      : op.Dhat ? operator_parts_k(op.nz, op.lx, op.precision)
-                               : operator_parts(op.nz, op.lx, op.precision);
+                               : operator_parts(op.B, op.nz, op.lx, op.precision);
+  // the single-grid operator finishes alpha and omega in its last kernel
+  const bool fused = !group && !op.Dhat;
+  const KrylovFinish fin{sb.st, sb.arrived, sb.partS, nblk, o.tol};
+  if (fused) op.finish = &fin;
   op.stencil = true;
   op.active = nullptr;
   k_absmax<C><<<grid, kRedThreads, 0, s>>>(sp, rhs, sb.partA);
   if ((rc = check_launch("k_absmax"))) return rc;
-  k_scale<<<B, 32, 0, s>>>(sb.st, sb.partA);
+  k_scale<<<B, 32, 0, s>>>(sb.st, sb.partA, nblk);
   if ((rc = check_launch("k_scale"))) return rc;
   if (!x_zero) {  // x0 into the scaled system, v = A x0
     k_scale_x<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, x, 0);
@@ -409,7 +413,7 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   }
   k_init<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, rhs, v, r, rhat, p, x, x_zero ? 1 : 0, sb.partA);
   if ((rc = check_launch("k_init"))) return rc;
-  k_init_state<<<B, 32, 0, s>>>(sb.st, sb.active, sb.counters, sb.partA, o.tol, o.max_iter);
+  k_init_state<<<B, 32, 0, s>>>(sb.st, sb.active, sb.counters, sb.arrived, sb.partA, nblk, o.tol, o.max_iter);
   if ((rc = check_launch("k_init_state"))) return rc;
   if (!x_zero) {
     k_zero_flagged<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, x);
@@ -440,7 +444,7 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   // One BiCGSTAB iteration of every active problem on stream `st`.
   auto iterate = [&](int it, cudaStream_t st) -> int {
     const int parity = it & 1;
-    const dim3 g2(kRedBlocks, nrun);
+    const dim3 g2(nblk, nrun);
     int rc2;
     op.plist = plist;
     op.nb = nrun;
@@ -448,18 +452,21 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
     if ((rc2 = check_launch("k_update_p"))) return rc2;
     op.epi = 1; op.in = p; op.ident = p; op.out = v; op.part_out = sb.partA;
     if ((rc2 = run_operator(op, st))) return rc2;
-    k_alpha<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, nparts, sb.partA);
-    if ((rc2 = check_launch("k_alpha"))) return rc2;
+    if (!fused) {
+      k_alpha<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, nparts, sb.partA);
+      if ((rc2 = check_launch("k_alpha"))) return rc2;
+    }
     k_update_s<C><<<g2, kRedThreads, 0, st>>>(sp, plist, sb.st, sb.active, r, v, sv, sb.partS);
     if ((rc2 = check_launch("k_update_s"))) return rc2;
     op.epi = 2; op.in = sv; op.ident = sv; op.out = t; op.part_out = sb.partB;
     if ((rc2 = run_operator(op, st))) return rc2;
-    k_omega<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, nparts, sb.partB, sb.partS, o.tol);
-    if ((rc2 = check_launch("k_omega"))) return rc2;
-    k_update_xr<C><<<g2, kRedThreads, 0, st>>>(sp, plist, sb.st, sb.active, p, sv, t, rhat, x, r, sb.partC);
-    if ((rc2 = check_launch("k_update_xr"))) return rc2;
-    k_check<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, sb.counters, parity, sb.partC, o.tol, o.max_iter);
-    return check_launch("k_check");
+    if (!fused) {
+      k_omega<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, nparts, sb.partB, sb.partS, nblk, o.tol);
+      if ((rc2 = check_launch("k_omega"))) return rc2;
+    }
+    k_update_xr<C><<<g2, kRedThreads, 0, st>>>(sp, plist, sb.st, sb.active, sb.counters, parity, sb.arrived, o.tol,
+                                               o.max_iter, p, sv, t, rhat, x, r, sb.partC);
+    return check_launch("k_update_xr");
   };
   const int K = o.check_every;
   if (group && use_graph && K > 0) {

@@ -17,6 +17,10 @@ struct KState {
   double scale;                              // power of two applied to rhs and x
   int iters, code, restart, half;
   int zero_rhs, restarts, pad[2];  // restarts: breakdown restarts so far
+  // alpha, omega and beta rounded to FP32 where they are set, for the complex64 vector updates: an
+  // FP64 conversion per thread costs a warp 16 cycles of the SM's FP64 pipe, more than the update
+  // of the few elements a thread has on a small grid.
+  float al_f[2], om_f[2], be_f[2];
 };
 
 // A value that is neither NaN nor infinite (host and device).
@@ -72,6 +76,17 @@ __host__ __device__ inline int bicgstab_decide(KState &k, const double q[3], dou
   return 1;
 }
 
+// Once per problem, by the last CTA to finish the launch that made the partials: alpha = rho /
+// <rhat, A p> (part: the first operator pass's partials), omega = <t, s> / ||t||^2 (zero when the half
+// step already met tol; part: the second pass's, partS: ||s||^2).
+struct KrylovFinish {
+  KState *st;         // [B], or NULL: nothing to do (the solver runs kernels of its own for them)
+  int *arrived;       // [B] CTA counters, zero between launches
+  const double *partS;
+  int nS;             // partials of ||s||^2 per problem
+  double tol;
+};
+
 struct SolverBufs {
   void *r, *rhat, *p, *v, *s, *t;  // [B][2][nz][nx] complex
   KState *st;                      // [B]
@@ -79,6 +94,8 @@ struct SolverBufs {
   int *counters;                   // [4]: active counts by iteration parity, compaction count
   int *plist;                      // [B] active problems, compacted
   double *partA, *partS, *partB, *partC;  // [B][kRedBlocks][kRedSlots]
+  int *arrived;                    // [B] CTA counters of the fused scalar steps (in the unused tail of
+                                   // partC's carve)
 };
 
 size_t bytes_solver(const dbi_grid *g, int B, int precision);

@@ -8,6 +8,7 @@
 #include <algorithm>
 
 #include "group.cuh"
+#include "krylov_finish.cuh"
 #include "op_split.cuh"
 #include "op_split3.cuh"
 #include "op_tiles.cuh"
@@ -38,6 +39,7 @@ template <typename C> struct OpP {
   const C *krhat;
   double *part_out;
   int part_count;
+  KrylovFinish fin;  // the solver's scalar steps, done by the last inverse row tile of a problem
   C *S;  // [slots][2][nz][nx] contrast-source scratch of the split row stages (L = 1024, 768), or NULL
 };
 
@@ -80,21 +82,21 @@ template <typename C> struct BatchTile {
   __device__ __forceinline__ Rl ms() const { return p.m_scale ? Rl(p.m_scale[0]) : Rl(1); }
 };
 
-template <typename C, int LX, bool STENCIL, int V>
-__global__ void __launch_bounds__(kTileThreads, Cfg<C>::rowFwdMinBlocks(LX)) k_rows_forward(OpP<C> p) {
+template <typename C, int LX, bool STENCIL, int V, int NTT>
+__global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowFwdMinBlocks(LX) : 1) k_rows_forward(OpP<C> p) {
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rows_forward_tile<C, LX, STENCIL, V>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x,
+  rows_forward_tile<C, LX, STENCIL, V, NTT>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x,
                                        reinterpret_cast<C *>(smem_raw));
 }
 
-template <typename C, int LZ, int V>
-__global__ void __launch_bounds__(kTileThreads, Cfg<C>::colMinBlocks) k_cols(OpP<C> p) {
+template <typename C, int LZ, int V, int NTT>
+__global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::colMinBlocks : 1) k_cols(OpP<C> p) {
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cols_tile<C, LZ, V>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x, reinterpret_cast<C *>(smem_raw));
+  cols_tile<C, LZ, V, NTT>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x, reinterpret_cast<C *>(smem_raw));
 }
 
 // The complex64 column stage: a CTA takes the columns kx of SL launch slots at a time (units
@@ -144,13 +146,14 @@ template <int LZ, int SL> constexpr size_t cols_pairs_smem() {
   return size_t(CF::CC) * CF::PLP * sizeof(cpair) + (SL == 1 ? 0 : size_t(CF::CC / SL) * 3 * LZ * sizeof(float2));
 }
 
-template <typename C, int LX, int EPI, int V>
-__global__ void __launch_bounds__(kTileThreads, Cfg<C>::rowInvMinBlocks) k_rows_inverse(OpP<C> p) {
+template <typename C, int LX, int EPI, int V, int NTT>
+__global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowInvMinBlocks : 1) k_rows_inverse(OpP<C> p) {
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rows_inverse_tile<C, LX, EPI, V>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x,
-                                   reinterpret_cast<C *>(smem_raw));
+  const BatchTile<C> a{p, b, int(blockIdx.y), f};
+  rows_inverse_tile<C, LX, EPI, V, NTT>(a, blockIdx.x, reinterpret_cast<C *>(smem_raw));
+  if constexpr (EPI != 0) finish_tile<EPI>(p.fin, b, a.part(), gridDim.x);
 }
 
 // Stages of the L = 1024 complex64 operator as pairs of 512-point transforms (op_split.cuh).
@@ -210,8 +213,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_rows_inverse_split(OpP<floa
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rows_inverse_tile_split<EPI>(BatchTile<float2>{p, b, int(blockIdx.y), f}, blockIdx.x,
-                               reinterpret_cast<float2 *>(smem_raw));
+  const BatchTile<float2> a{p, b, int(blockIdx.y), f};
+  rows_inverse_tile_split<EPI>(a, blockIdx.x, reinterpret_cast<float2 *>(smem_raw));
+  if constexpr (EPI != 0) finish_tile<EPI>(p.fin, b, a.part(), gridDim.x);
 }
 
 // Stages of the L = 768 complex64 operator as triples of 256-point transforms (op_split3.cuh);
@@ -239,8 +243,27 @@ __global__ void __launch_bounds__(kS3Threads, 2) k_rows_inverse_s3(OpP<float2> p
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rows_inverse_tile_s3<EPI>(BatchTile<float2>{p, b, int(blockIdx.y), f}, blockIdx.x,
-                            reinterpret_cast<float2 *>(smem_raw));
+  const BatchTile<float2> a{p, b, int(blockIdx.y), f};
+  rows_inverse_tile_s3<EPI>(a, blockIdx.x, reinterpret_cast<float2 *>(smem_raw));
+  if constexpr (EPI != 0) finish_tile<EPI>(p.fin, b, a.part(), gridDim.x);
+}
+
+// Threads per CTA of the ordinary stages: 256, or for complex128 batches too small to give every SM a
+// 256-thread tile, as few as hold whole lines and warps. FP64 runs at two lanes a cycle and SM, so
+// what counts there is the number of SMs: a 32 x 32 grid of one problem was one row tile and two
+// column tiles (68, 40 and 24 us for the three stages).
+template <int L> constexpr int kSmallThreads = L / 8 > 32 ? L / 8 : 32;
+inline bool small_tiles(int B, int nz, int lx, int precision) {
+  return precision == DBI_C128 && lx <= 1024 && size_t(B) * ((size_t(nz) * lx + 2047) / 2048) < 2 * 152;
+}
+template <typename C, int L, typename F> inline void with_tile(bool small, F &&f) {
+  if constexpr (sizeof(C) == sizeof(double2)) {
+    if (small) {
+      f.template operator()<kSmallThreads<L>>();
+      return;
+    }
+  }
+  f.template operator()<kTileThreads>();
 }
 
 // Calls f.template operator()<V>() with the radix plan chosen for length L (plans differ only
@@ -274,12 +297,14 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   p.in_scale = a.in_scale;
   p.m_scale = a.m_scale;
   p.out_scale = a.out_scale;
-  p.part_count = operator_parts(a.nz, a.lx, a.precision);
+  p.part_count = operator_parts(a.B, a.nz, a.lx, a.precision);
+  p.fin = KrylovFinish{};
+  if (a.finish && a.epi != 0) p.fin = *a.finish;
   p.krhat = static_cast<const C *>(a.krhat);
   p.part_out = a.part_out;
   p.S = nullptr;
   int rc = DBI_OK;
-  const bool stencil = a.stencil;
+  const bool stencil = a.stencil, small = small_tiles(a.B, a.nz, a.lx, a.precision);
   const int kr = split_kind(a.lx, a.precision), kc = split_kind(a.lz, a.precision);
   const bool split_r = kr != 0, split_c = kc != 0;
   if (split_r) p.S = p.T + size_t(cap) * 2 * a.lx * a.nz;  // after the chunk's spectra
@@ -312,16 +337,18 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   }
   if (!split_r) dispatch_len(a.lx, [&]<int LX>() {
     with_plan<LX>(a.precision, [&]<int V>() {
-      using RC = RowCfg<C, LX>;
-      const size_t bytes = rows_forward_smem<C, LX>(a.nx, stencil);
-      dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
       cudaError_t e;
-      auto launch = [&](auto kernel) {
-        e = allow_smem(kernel, bytes);
-        if (e == cudaSuccess) kernel<<<grid, RC::NT, bytes, s>>>(p);
-      };
-      if (stencil) launch(k_rows_forward<C, LX, true, V>);
-      else launch(k_rows_forward<C, LX, false, V>);
+      with_tile<C, LX>(small, [&]<int NTT>() {
+        using RC = RowCfg<C, LX, NTT>;
+        const size_t bytes = rows_forward_smem<C, LX, NTT>(a.nx, stencil);
+        dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
+        auto launch = [&](auto kernel) {
+          e = allow_smem(kernel, bytes);
+          if (e == cudaSuccess) kernel<<<grid, RC::NT, bytes, s>>>(p);
+        };
+        if (stencil) launch(k_rows_forward<C, LX, true, V, NTT>);
+        else launch(k_rows_forward<C, LX, false, V, NTT>);
+      });
       rc = e != cudaSuccess ? cuda_fail("k_rows_forward smem", e) : check_launch("k_rows_forward");
     });
   });
@@ -362,10 +389,14 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           rc = e != cudaSuccess ? cuda_fail("k_cols_pairs smem", e) : check_launch("k_cols_pairs");
         }
       } else {
-        const size_t bytes = cols_smem<C, LZ>();
-        dim3 grid((a.lx + CF::CC - 1) / CF::CC, nb);
-        cudaError_t e = allow_smem(k_cols<C, LZ, V>, bytes);
-        if (e == cudaSuccess) k_cols<C, LZ, V><<<grid, CF::NT, bytes, s>>>(p);
+        cudaError_t e;
+        with_tile<C, LZ>(small, [&]<int NTT>() {
+          using CN = ColCfg<C, LZ, NTT>;
+          const size_t bytes = cols_smem<C, LZ, NTT>();
+          dim3 grid((a.lx + CN::CC - 1) / CN::CC, nb);
+          e = allow_smem(k_cols<C, LZ, V, NTT>, bytes);
+          if (e == cudaSuccess) k_cols<C, LZ, V, NTT><<<grid, CN::NT, bytes, s>>>(p);
+        });
         rc = e != cudaSuccess ? cuda_fail("k_cols smem", e) : check_launch("k_cols");
       }
     });
@@ -392,17 +423,19 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   }
   if (!split_r) dispatch_len(a.lx, [&]<int LX>() {
     with_plan<LX>(a.precision, [&]<int V>() {
-      using RC = RowCfg<C, LX>;
-      const size_t bytes = rows_inverse_smem<C, LX>();
-      dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
       cudaError_t e;
-      auto launch = [&](auto kernel) {
-        e = allow_smem(kernel, bytes);
-        if (e == cudaSuccess) kernel<<<grid, RC::NT, bytes, s>>>(p);
-      };
-      if (a.epi == 1) launch(k_rows_inverse<C, LX, 1, V>);
-      else if (a.epi == 2) launch(k_rows_inverse<C, LX, 2, V>);
-      else launch(k_rows_inverse<C, LX, 0, V>);
+      with_tile<C, LX>(small, [&]<int NTT>() {
+        using RC = RowCfg<C, LX, NTT>;
+        const size_t bytes = rows_inverse_smem<C, LX, NTT>();
+        dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
+        auto launch = [&](auto kernel) {
+          e = allow_smem(kernel, bytes);
+          if (e == cudaSuccess) kernel<<<grid, RC::NT, bytes, s>>>(p);
+        };
+        if (a.epi == 1) launch(k_rows_inverse<C, LX, 1, V, NTT>);
+        else if (a.epi == 2) launch(k_rows_inverse<C, LX, 2, V, NTT>);
+        else launch(k_rows_inverse<C, LX, 0, V, NTT>);
+      });
       rc = e != cudaSuccess ? cuda_fail("k_rows_inverse smem", e) : check_launch("k_rows_inverse");
     });
   });
@@ -423,9 +456,14 @@ template <typename C> static int run_typed(const OpArgs &a, cudaStream_t s) {
   return rc;
 }
 
-int operator_parts(int nz, int lx, int precision) {
+int operator_parts(int B, int nz, int lx, int precision) {
   static_assert(kS3Units == kSplitRows, "split row tiles hold the same number of rows");
   if (split_rows(lx, precision)) return (nz + kSplitRows - 1) / kSplitRows;
+  if (small_tiles(B, nz, lx, precision)) {
+    int rows = 1;
+    dispatch_len(lx, [&]<int LX>() { rows = RowCfg<double2, LX, kSmallThreads<LX>>::ROWS; });
+    return (nz + rows - 1) / rows;
+  }
   return operator_parts_k(nz, lx, precision);
 }
 

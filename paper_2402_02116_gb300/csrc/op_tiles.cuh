@@ -44,9 +44,9 @@ template <> struct Cfg<double2> {
 };
 constexpr int kTileThreads = 256;
 
-template <typename C, int LX> struct RowCfg {
+template <typename C, int LX, int NTT = kTileThreads> struct RowCfg {
   static constexpr int T = LX / 8;
-  static constexpr int ROWS = kTileThreads / T;
+  static constexpr int ROWS = NTT / T;
   static constexpr int NT = ROWS * T;
   static constexpr int LP = RegFFT<C, LX>::LP;
   // complex64: lines of pairs, and the transposition tile [ROWS][KP] of pairs. A quarter warp's
@@ -55,9 +55,9 @@ template <typename C, int LX> struct RowCfg {
   static constexpr int PLP = RegFFT<cpair, LX>::LP;
   static constexpr int KP = LX + (ROWS >= 8 ? 1 : 8 / ROWS);
 };
-template <typename C, int LZ> struct ColCfg {
+template <typename C, int LZ, int NTT = kTileThreads> struct ColCfg {
   static constexpr int T = LZ / 8;
-  static constexpr int CC = kTileThreads / T;  // named barriers 1..CC only when T > 32 (CC <= 4)
+  static constexpr int CC = NTT / T;  // named barriers 1..CC only when T > 32 (CC <= 4)
   static constexpr int NT = CC * T;
   static constexpr int LP = RegFFT<C, LZ>::LP;
   static constexpr int PLP = RegFFT<cpair, LZ>::LP;
@@ -72,8 +72,8 @@ template <typename C> constexpr bool kPairSpectra = sizeof(C) == sizeof(float2);
 constexpr int kHalf = 4;
 
 // Transposition tile of the rows kernels: [2][LX][ROWS + 1] (padded against bank conflicts).
-template <typename C, int LX> constexpr size_t tile_elems() {
-  return size_t(2) * LX * (RowCfg<C, LX>::ROWS + 1);
+template <typename C, int LX, int NTT = kTileThreads> constexpr size_t tile_elems() {
+  return size_t(2) * LX * (RowCfg<C, LX, NTT>::ROWS + 1);
 }
 
 // Lengths whose stencil uses the strip form (one column per thread, few rows per tile).
@@ -83,8 +83,8 @@ template <typename C, int LX> constexpr size_t tile_elems() {
 #ifndef DBI_STRIP_1024
 #define DBI_STRIP_1024 1
 #endif
-template <typename C, int LX>
-constexpr bool kStripStencil = LX == 512 || (LX == 1024 && DBI_STRIP_1024 && sizeof(C) == 8) ||
+template <typename C, int LX, int NTT = kTileThreads>
+constexpr bool kStripStencil = NTT != kTileThreads ? false : LX == 512 || (LX == 1024 && DBI_STRIP_1024 && sizeof(C) == 8) ||
                                (LX == 256 && DBI_STRIP_256);  // complex128 at 1024 would spill
 
 // Shared memory of the strip stencil (bytes): u at ROWS + 2 rows, sigma1 and sigma5 at ROWS rows.
@@ -94,26 +94,26 @@ template <typename C, int LX> inline size_t stencil_strip_smem(int nx) {
 }
 
 // Dynamic shared memory of each stage (bytes).
-template <typename C, int LX> inline size_t rows_forward_smem(int nx, bool stencil) {
-  using RC = RowCfg<C, LX>;
+template <typename C, int LX, int NTT = kTileThreads> inline size_t rows_forward_smem(int nx, bool stencil) {
+  using RC = RowCfg<C, LX, NTT>;
   const size_t lines = kPairSpectra<C> ? size_t(RC::ROWS) * RC::PLP * sizeof(cpair)
                                        : size_t(2) * RC::ROWS * RC::LP * sizeof(C);
-  const size_t tile = kPairSpectra<C> ? size_t(RC::ROWS) * RC::KP * sizeof(cpair) : tile_elems<C, LX>() * sizeof(C);
+  const size_t tile = kPairSpectra<C> ? size_t(RC::ROWS) * RC::KP * sizeof(cpair) : tile_elems<C, LX, NTT>() * sizeof(C);
   size_t sg = 0;
   if (stencil) {
-    if constexpr (kStripStencil<C, LX>) sg = stencil_strip_smem<C, LX>(nx);
+    if constexpr (kStripStencil<C, LX, NTT>) sg = stencil_strip_smem<C, LX>(nx);
     else sg = (size_t(3) * (RC::ROWS + 2) + size_t(2) * (RC::ROWS + 4)) * (nx + 2) * sizeof(C);
   }
   return std::max(std::max(lines, tile), sg);
 }
-template <typename C, int LZ> inline size_t cols_smem() {
-  using CF = ColCfg<C, LZ>;
+template <typename C, int LZ, int NTT = kTileThreads> inline size_t cols_smem() {
+  using CF = ColCfg<C, LZ, NTT>;
   return kPairSpectra<C> ? size_t(CF::CC) * CF::PLP * sizeof(cpair) : size_t(2) * CF::CC * CF::LP * sizeof(C);
 }
-template <typename C, int LX> inline size_t rows_inverse_smem() {
-  using RC = RowCfg<C, LX>;
+template <typename C, int LX, int NTT = kTileThreads> inline size_t rows_inverse_smem() {
+  using RC = RowCfg<C, LX, NTT>;
   if (kPairSpectra<C>) return size_t(RC::ROWS) * std::max(RC::PLP, RC::KP) * sizeof(cpair);
-  return std::max(size_t(2) * RC::ROWS * RC::LP, tile_elems<C, LX>()) * sizeof(C);
+  return std::max(size_t(2) * RC::ROWS * RC::LP, tile_elems<C, LX, NTT>()) * sizeof(C);
 }
 
 // Barrier over the threads that share a line: the T threads of one row or column.
@@ -349,10 +349,10 @@ __device__ __forceinline__ void rows_forward_pairs(const A &a, int z0, int rr, i
 // Contrast source (or the raw source) of ROWS rows, zero-padded to LX, forward FFT along x.
 //   stencil: stress of rows z0-1 .. z0+ROWS (each computed once, kept in shared memory), then
 //            s1 = w^2 drho u1 + d1 sigma1 + d3 sigma5, s3 = w^2 drho u3 + d1 sigma5 + d3 sigma3.
-template <typename C, int LX, bool STENCIL, int V, typename A>
+template <typename C, int LX, bool STENCIL, int V, int NTT = kTileThreads, typename A>
 __device__ __forceinline__ void rows_forward_tile(const A &a, int tile, C *smem) {
   using Rl = typename RealOf<C>::type;
-  using RC = RowCfg<C, LX>;
+  using RC = RowCfg<C, LX, NTT>;
   constexpr int ROWS = RC::ROWS, T = RC::T, LP = RC::LP;
   const int z0 = tile * ROWS;
   const int nz = a.nz(), nx = a.nx();
@@ -363,7 +363,7 @@ __device__ __forceinline__ void rows_forward_tile(const A &a, int tile, C *smem)
   const TwReg<C, LX, V> tr(t, a.tw());
   C v[2][8];
 
-  if constexpr (STENCIL && kStripStencil<C, LX>) {
+  if constexpr (STENCIL && kStripStencil<C, LX, NTT>) {
     stencil_strip<C, LX>(a, z0, smem, v);
   } else if constexpr (STENCIL) {
     const int W = nx + 2;          // rows with one zero column on each side
@@ -520,7 +520,7 @@ __device__ __forceinline__ void cols_unit_pairs(const A &a, int kx, int u, int t
   }
 }
 
-template <typename C, int LZ, int V, typename A>
+template <typename C, int LZ, int V, int NTT = kTileThreads, typename A>
 __device__ __forceinline__ void cols_tile(const A &a, int tile, C *smem) {
   if constexpr (kPairSpectra<C>) {
     constexpr int CC = ColCfg<C, LZ>::CC, T = ColCfg<C, LZ>::T;
@@ -528,7 +528,7 @@ __device__ __forceinline__ void cols_tile(const A &a, int tile, C *smem) {
     cols_unit_pairs<LZ, V, false>(a, kx, u, threadIdx.x - u * T, kx < a.lx(), reinterpret_cast<cpair *>(smem), nullptr);
     return;
   }
-  using CF = ColCfg<C, LZ>;
+  using CF = ColCfg<C, LZ, NTT>;
   constexpr int CC = CF::CC, T = CF::T, LP = CF::LP;
   const int col = threadIdx.x / T, t = threadIdx.x - col * T;
   const int kx = tile * CC + col;
@@ -574,10 +574,10 @@ __device__ __forceinline__ void cols_tile(const A &a, int tile, C *smem) {
 
 // Inverse FFT along x of ROWS rows, keep x < nx, out = ident - osc * result (or the scaled
 // result when there is no identity term).
-template <typename C, int LX, int EPI, int V, typename A>
+template <typename C, int LX, int EPI, int V, int NTT = kTileThreads, typename A>
 __device__ __forceinline__ void rows_inverse_tile(const A &a, int tile, C *smem) {
   using Rl = typename RealOf<C>::type;
-  using RC = RowCfg<C, LX>;
+  using RC = RowCfg<C, LX, NTT>;
   constexpr int ROWS = RC::ROWS, T = RC::T, LP = RC::LP;
   const int z0 = tile * ROWS;
   const int nz = a.nz(), nx = a.nx();

@@ -17,6 +17,7 @@ struct Span {
   }
 };
 
+struct KrylovFinish;  // scalar steps of the solver fused into the operator's last kernel (krylov.cuh)
 struct GroupLaunch;  // launch description of an uneven batch (group.cuh)
 
 // One batched pass  out = ident - K(src)  or  out = K(src), where K(src) = h^2 G * src and src
@@ -54,6 +55,7 @@ struct OpArgs {
   int epi;
   const void *krhat;
   double *part_out;
+  const KrylovFinish *finish;  // single-grid divergence form only; or NULL
   // Uneven batch: problems on different grids (nz, nx, lz, lx, m, Ghat, omega, ref above are then
   // unused and come from the group's member descriptors). offs: field offsets per problem.
   const GroupLaunch *group;
@@ -67,7 +69,7 @@ struct OpArgs {
 // Partials per problem written by the operator kernels (one per CTA row block): the single-grid
 // divergence form (operator_parts) and the paper-literal form (operator_parts_k, whose row stages
 // keep 2048 / L rows per tile at every length).
-int operator_parts(int nz, int lx, int precision);
+int operator_parts(int B, int nz, int lx, int precision);
 int operator_parts_k(int nz, int lx, int precision);
 
 int run_operator(const OpArgs &a, cudaStream_t s);

@@ -34,6 +34,24 @@ template <int NS, typename T> __device__ __forceinline__ void block_sum_store(T 
   __syncthreads();
 }
 
+// True in every thread of the last of a problem's `n` CTAs to arrive (each CTA must call it once,
+// with every thread, after its partials are stored); `arrived` counts them and is zero again when
+// the last one has left. The last CTA sees the partials of all the others.
+__device__ __forceinline__ bool last_cta(int *arrived, int n) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(arrived, 1) == n - 1;
+    if (last) {
+      *arrived = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last != 0;
+}
+
 // Sum slot k (k < NS) of `count` partials of one problem in a fixed order; every thread of the
 // CTA gets the sums. Every thread of the CTA must call it.
 template <int NS> __device__ __forceinline__ void gather_n(const double *part, int count, double (&out)[NS]) {
@@ -43,7 +61,7 @@ template <int NS> __device__ __forceinline__ void gather_n(const double *part, i
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
       double a = 0.0;
-      for (int i = lane; i < count; i += 32) a += part[i * kRedSlots + k];
+      for (int i = lane; i < count; i += 32) a += __ldcg(part + i * kRedSlots + k);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
       if (lane == 0) sh[k] = a;
@@ -55,18 +73,22 @@ template <int NS> __device__ __forceinline__ void gather_n(const double *part, i
   __syncthreads();
 }
 
-// Maximum of v over the CTA; thread 0 stores it to out[0]. Every thread of the CTA must call it.
-__device__ __forceinline__ void block_max_store(double v, double *out) {
-  __shared__ double sh[32];
+__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
+
+// Maximum of v over the CTA, compared in its own type; thread 0 stores it to out[0]. Every thread of
+// the CTA must call it.
+template <typename T> __device__ __forceinline__ void block_max_store(T v, double *out) {
+  __shared__ T sh[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, off));
+  for (int off = 16; off > 0; off >>= 1) v = max_of(v, __shfl_down_sync(0xffffffffu, v, off));
   if (lane == 0) sh[warp] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double a = 0.0;
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) a = fmax(a, sh[w]);
-    out[0] = a;
+    T a = 0;
+    for (int w = 0; w < int(blockDim.x >> 5); ++w) a = max_of(a, sh[w]);
+    out[0] = double(a);
   }
   __syncthreads();
 }
