@@ -92,6 +92,7 @@ template <typename C, int LX> inline size_t kk_rows_forward_smem(int nx) {
 // forward FFT along x, transposed into T5[slot][c][kx][z].
 template <typename C, int LX>
 __global__ void __launch_bounds__(kTileThreads) kk_rows_forward(KP<C> p) {
+  pdl_begin();
   using Rl = typename RealOf<C>::type;
   using RC = RowCfg<C, LX>;
   constexpr int ROWS = RC::ROWS, T = RC::T, LP = RC::LP, RG = ROWS + 2, RP = ROWS + 1;
@@ -175,6 +176,7 @@ template <typename C> constexpr int kKColsLines = sizeof(C) == 8 ? DBI_KCOLS_LIN
 
 template <typename C, int LZ>
 __global__ void __launch_bounds__(kTileThreads, sizeof(C) == 8 ? 2 : 1) kk_cols(KP<C> p) {
+  pdl_begin();
   using CF = ColCfg<C, LZ>;
   constexpr int CC = CF::CC, T = CF::T, LP = CF::LP;
   const int b = kproblem(p), f = p.fidx[b], slot = blockIdx.y;
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(C) == 8 ? 2 : 1) kk_cols(
 
 template <typename C, int LX, int EPI>
 __global__ void __launch_bounds__(kTileThreads) kk_rows_inverse(KP<C> p) {
+  pdl_begin();
   const int b = kproblem(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -305,7 +308,7 @@ template <typename C> static int run_k_typed(const OpArgs &a, cudaStream_t s) {
     const size_t bytes = kk_rows_forward_smem<C, LX>(a.nx);
     const dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
     cudaError_t e = allow_smem(kk_rows_forward<C, LX>, bytes);
-    if (e == cudaSuccess) kk_rows_forward<C, LX><<<grid, kTileThreads, bytes, s>>>(p);
+    if (e == cudaSuccess) launch_pdl(kk_rows_forward<C, LX>, grid, kTileThreads, bytes, s, p);
     rc = e != cudaSuccess ? cuda_fail("kk_rows_forward smem", e) : check_launch("kk_rows_forward");
   });
   prof_mark(PROF_ROWS_FORWARD, true, s);
@@ -316,7 +319,7 @@ template <typename C> static int run_k_typed(const OpArgs &a, cudaStream_t s) {
     const size_t bytes = cols_smem<C, LZ>();
     const dim3 grid((a.lx + CF::CC - 1) / CF::CC, nb);
     cudaError_t e = allow_smem(kk_cols<C, LZ>, bytes);
-    if (e == cudaSuccess) kk_cols<C, LZ><<<grid, kTileThreads, bytes, s>>>(p);
+    if (e == cudaSuccess) launch_pdl(kk_cols<C, LZ>, grid, kTileThreads, bytes, s, p);
     rc = e != cudaSuccess ? cuda_fail("kk_cols smem", e) : check_launch("kk_cols");
   });
   prof_mark(PROF_COLS, true, s);
@@ -329,7 +332,7 @@ template <typename C> static int run_k_typed(const OpArgs &a, cudaStream_t s) {
     cudaError_t e;
     auto launch = [&](auto kernel) {
       e = allow_smem(kernel, bytes);
-      if (e == cudaSuccess) kernel<<<grid, kTileThreads, bytes, s>>>(p);
+      if (e == cudaSuccess) launch_pdl(kernel, grid, kTileThreads, bytes, s, p);
     };
     if (a.epi == 1) launch(kk_rows_inverse<C, LX, 1>);
     else if (a.epi == 2) launch(kk_rows_inverse<C, LX, 2>);

@@ -98,6 +98,7 @@ static GmresBufs carve_gmres(Arena &ar, size_t f, int B, int m) {
 // x *= scale (inverse = 0) or x /= scale (inverse = 1)
 template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_gm_scale_x(Span sp, const double *scale, C *x, int inverse) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int b = blockIdx.y;
   const R f = R(inverse ? 1.0 / scale[b] : scale[b]);
@@ -111,6 +112,7 @@ template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_gm_residual(Span sp, const int *live, const double *scale,
                                                              const C *__restrict__ rhs, C *__restrict__ v0,
                                                              int have_ax, C *__restrict__ x0z, double *part) {
+  pdl_begin();
   using A = typename Acc<C>::type;
   using R = typename RealOf<C>::type;
   const int b = blockIdx.y;
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_residual(Span sp, const int 
 // g = beta e_1. On the first cycle every problem is initialised; later only active ones restart.
 __global__ void k_gm_begin(GState *st, int *active, double2 *g, const double *part, double tol, int max_iter,
                            int first, int m) {
+  pdl_begin();
   const int b = blockIdx.x;
   if (!first && !active[b]) return;
   double s[2];
@@ -168,6 +171,7 @@ __global__ void k_gm_begin(GState *st, int *active, double2 *g, const double *pa
 
 template <typename C>
 __global__ void k_gm_zero_flagged(Span sp, const GState *st, C *x) {
+  pdl_begin();
   const int b = blockIdx.y;
   if (!st[b].zero_rhs) return;
   DBI_PROBLEM_LOOP(sp) x[off + i] = czero<C>();
@@ -177,6 +181,7 @@ __global__ void k_gm_zero_flagged(Span sp, const GState *st, C *x) {
 template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_gm_scale_v(Span sp, const int *plist, const int *active,
                                                             const GState *st, C *v) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
@@ -191,6 +196,7 @@ template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_gm_dots(Span sp, const int *plist, const int *active,
                                                          const GState *st, const C *__restrict__ V,
                                                          size_t vstride, int j, int round, double *partD) {
+  pdl_begin();
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b] || (round == 1 && !st[b].need2)) return;
@@ -250,6 +256,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_dots(Span sp, const int *pli
 // the first pass also stores ||K v_j||^2. One CTA of 2 kGmresMaxRestart + 32 threads per problem.
 __global__ void k_gm_hsum(const int *plist, const int *active, GState *st, const double *partD, double2 *hc,
                           double2 *H, int j, int round, int m) {
+  pdl_begin();
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b] || (round == 1 && !st[b].need2)) return;
   const int t = threadIdx.x;
@@ -281,6 +288,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_update(Span sp, const int *p
                                                            const GState *st, C *__restrict__ V, size_t vstride,
                                                            int j, int round, const double2 *hc, int m,
                                                            double *partN) {
+  pdl_begin();
   using A = typename Acc<C>::type;
   __shared__ C h[kGmresMaxRestart + kDotGroup];
   const int b = problem_at(plist, blockIdx.y);
@@ -336,6 +344,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_update(Span sp, const int *p
 
 // After the first round: re-orthogonalise when ||w'||^2 < 0.49 ||w||^2 (one CTA per problem).
 __global__ void k_gm_need2(const int *plist, const int *active, GState *st, const double *partN) {
+  pdl_begin();
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
   double s[1];
@@ -349,6 +358,7 @@ __global__ void k_gm_need2(const int *plist, const int *active, GState *st, cons
 // vanishes (the solution lies in the space built so far), or at the iteration limit.
 __global__ void k_gm_close(const int *plist, int *active, GState *st, double2 *H, double2 *g, double *cs,
                            double2 *sn, const double *partN, int j, int m, double tol, int max_iter) {
+  pdl_begin();
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
   double s[1];
@@ -408,6 +418,7 @@ __global__ void k_gm_close(const int *plist, int *active, GState *st, double2 *H
 
 // End of a cycle: y from R y = g by back substitution for every problem that ran this cycle.
 __global__ void k_gm_solve_y(int B, GState *st, const double2 *H, const double2 *g, double2 *y, int m) {
+  pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   GState k = st[b];
@@ -433,6 +444,7 @@ template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_gm_update_x(Span sp, const GState *st, const C *__restrict__ V,
                                                              size_t vstride, const double2 *y, int m,
                                                              C *__restrict__ x) {
+  pdl_begin();
   __shared__ C c[kGmresMaxRestart + kDotGroup];
   const int b = blockIdx.y;
   const int kx = st[b].kx;
@@ -454,6 +466,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_update_x(Span sp, const GSta
 }
 
 __global__ void k_gm_finalize(int B, const GState *st, int *iters, double *relres, int *code) {
+  pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const GState k = st[b];
@@ -488,7 +501,7 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
   op.nb = B;
   if ((rc = pow2_scales(rhs, op.precision, false, B, n, gb.partN, gb.scale, nullptr, nullptr, s))) return rc;
   if (!x_zero) {
-    k_gm_scale_x<C><<<all, kRedThreads, 0, s>>>(sp, gb.scale, x, 0);
+    launch_pdl(k_gm_scale_x<C>, all, kRedThreads, 0, s, sp, gb.scale, x, 0);
     if ((rc = check_launch("k_gm_scale_x"))) return rc;
   }
   int nact = B, nrun = B;
@@ -504,26 +517,26 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
   for (bool first = true;; first = false) {
     // residual of the problems that (re)start a cycle
     if (first && x_zero) {
-      k_gm_residual<C><<<all, kRedThreads, 0, s>>>(sp, nullptr, gb.scale, rhs, Vj(0), 0, x, gb.partN);
+      launch_pdl(k_gm_residual<C>, all, kRedThreads, 0, s, sp, nullptr, gb.scale, rhs, Vj(0), 0, x, gb.partN);
     } else {
       op.plist = first ? nullptr : plist;
       op.nb = first ? B : nrun;
       op.active = first ? nullptr : gb.active;
       op.in = x; op.ident = x; op.out = Vj(0);
       if ((rc = run_operator(op, s))) return rc;
-      k_gm_residual<C><<<all, kRedThreads, 0, s>>>(sp, first ? nullptr : gb.active, gb.scale, rhs, Vj(0), 1,
+      launch_pdl(k_gm_residual<C>, all, kRedThreads, 0, s, sp, first ? nullptr : gb.active, gb.scale, rhs, Vj(0), 1,
                                                    static_cast<C *>(nullptr), gb.partN);
     }
     if ((rc = check_launch("k_gm_residual"))) return rc;
-    k_gm_begin<<<B, 32, 0, s>>>(gb.st, gb.active, gb.g, gb.partN, o.tol, o.max_iter, first ? 1 : 0, m);
+    launch_pdl(k_gm_begin, B, 32, 0, s, gb.st, gb.active, gb.g, gb.partN, o.tol, o.max_iter, first ? 1 : 0, m);
     if ((rc = check_launch("k_gm_begin"))) return rc;
     if (first && !x_zero) {
-      k_gm_zero_flagged<C><<<all, kRedThreads, 0, s>>>(sp, gb.st, x);
+      launch_pdl(k_gm_zero_flagged<C>, all, kRedThreads, 0, s, sp, gb.st, x);
       if ((rc = check_launch("k_gm_zero_flagged"))) return rc;
     }
     if ((rc = compact())) return rc;
     if (nact == 0) break;
-    k_gm_scale_v<C><<<dim3(kRedBlocks, nrun), kRedThreads, 0, s>>>(sp, plist, gb.active, gb.st, Vj(0));
+    launch_pdl(k_gm_scale_v<C>, dim3(kRedBlocks, nrun), kRedThreads, 0, s, sp, plist, gb.active, gb.st, Vj(0));
     if ((rc = check_launch("k_gm_scale_v"))) return rc;
     for (int j = 0; j < m; ++j) {
       const dim3 g2(kRedBlocks, nrun);
@@ -532,24 +545,24 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
       if ((rc = run_operator(op, s))) return rc;
       for (int round = 0; round < 2; ++round) {
         if (round == 1) {
-          k_gm_need2<<<nrun, 32, 0, s>>>(plist, gb.active, gb.st, gb.partN);
+          launch_pdl(k_gm_need2, nrun, 32, 0, s, plist, gb.active, gb.st, gb.partN);
           if ((rc = check_launch("k_gm_need2"))) return rc;
         }
         const dim3 g3(kRedBlocks, nrun, (j + 1 + kDotGroup - 1) / kDotGroup);
-        k_gm_dots<C><<<g3, kRedThreads, 0, s>>>(sp, plist, gb.active, gb.st, V, vstride, j, round, gb.partD);
+        launch_pdl(k_gm_dots<C>, g3, kRedThreads, 0, s, sp, plist, gb.active, gb.st, V, vstride, j, round, gb.partD);
         if ((rc = check_launch("k_gm_dots"))) return rc;
-        k_gm_hsum<<<nrun, 2 * kGmresMaxRestart + 32, 0, s>>>(plist, gb.active, gb.st, gb.partD, gb.hc, gb.H, j,
+        launch_pdl(k_gm_hsum, nrun, 2 * kGmresMaxRestart + 32, 0, s, plist, gb.active, gb.st, gb.partD, gb.hc, gb.H, j,
                                                              round, m);
         if ((rc = check_launch("k_gm_hsum"))) return rc;
-        k_gm_update<C><<<g2, kRedThreads, 0, s>>>(sp, plist, gb.active, gb.st, V, vstride, j, round, gb.hc, m,
+        launch_pdl(k_gm_update<C>, g2, kRedThreads, 0, s, sp, plist, gb.active, gb.st, V, vstride, j, round, gb.hc, m,
                                                   gb.partN);
         if ((rc = check_launch("k_gm_update"))) return rc;
       }
-      k_gm_close<<<nrun, 32, 0, s>>>(plist, gb.active, gb.st, gb.H, gb.g, gb.cs, gb.sn, gb.partN, j, m, o.tol,
+      launch_pdl(k_gm_close, nrun, 32, 0, s, plist, gb.active, gb.st, gb.H, gb.g, gb.cs, gb.sn, gb.partN, j, m, o.tol,
                                      o.max_iter);
       if ((rc = check_launch("k_gm_close"))) return rc;
       if (j + 1 < m) {
-        k_gm_scale_v<C><<<g2, kRedThreads, 0, s>>>(sp, plist, gb.active, gb.st, Vj(j + 1));
+        launch_pdl(k_gm_scale_v<C>, g2, kRedThreads, 0, s, sp, plist, gb.active, gb.st, Vj(j + 1));
         if ((rc = check_launch("k_gm_scale_v"))) return rc;
       }
       if (j + 1 == m || (K > 0 && (j + 1) % K == 0)) {
@@ -557,16 +570,16 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
         if (nact == 0) break;
       }
     }
-    k_gm_solve_y<<<(B + 127) / 128, 128, 0, s>>>(B, gb.st, gb.H, gb.g, gb.y, m);
+    launch_pdl(k_gm_solve_y, (B + 127) / 128, 128, 0, s, B, gb.st, gb.H, gb.g, gb.y, m);
     if ((rc = check_launch("k_gm_solve_y"))) return rc;
-    k_gm_update_x<C><<<all, kRedThreads, 0, s>>>(sp, gb.st, V, vstride, gb.y, m, x);
+    launch_pdl(k_gm_update_x<C>, all, kRedThreads, 0, s, sp, gb.st, V, vstride, gb.y, m, x);
     if ((rc = check_launch("k_gm_update_x"))) return rc;
     if (nact == 0) break;
   }
-  k_gm_scale_x<C><<<all, kRedThreads, 0, s>>>(sp, gb.scale, x, 1);
+  launch_pdl(k_gm_scale_x<C>, all, kRedThreads, 0, s, sp, gb.scale, x, 1);
   if ((rc = check_launch("k_gm_scale_x"))) return rc;
   if (status) {
-    k_gm_finalize<<<(B + 127) / 128, 128, 0, s>>>(B, gb.st, status->iters, status->relres, status->code);
+    launch_pdl(k_gm_finalize, (B + 127) / 128, 128, 0, s, B, gb.st, status->iters, status->relres, status->code);
     if ((rc = check_launch("k_gm_finalize"))) return rc;
   }
   return DBI_OK;

@@ -41,6 +41,7 @@ __device__ __forceinline__ double absmax(double2 v) { return fmax(fabs(v.x), fab
 
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_absmax(Span sp, const T *x, double *part) {
+  pdl_begin();
   const int b = blockIdx.y;
   decltype(absmax(T{})) m = 0;
   if constexpr (std::is_same_v<T, float2>) {
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(kRedThreads) k_absmax(Span sp, const T *x, dou
 // Power-of-two scale per problem that brings max |rhs| into [1, 2); the solver iterates on the
 // scaled system (exact in any precision) and unscales the solution at the end.
 __global__ void k_scale(KState *st, const double *part, int nblk) {
+  pdl_begin();
   const double m = gather_max(part + size_t(blockIdx.x) * kRedBlocks * kRedSlots, nblk);
   if (threadIdx.x == 0) st[blockIdx.x].scale = pow2_below(m);
 }
@@ -66,6 +68,7 @@ __global__ void k_scale(KState *st, const double *part, int nblk) {
 // x *= scale (inverse = 0) or x /= scale (inverse = 1)
 template <typename C>
 __global__ void k_scale_x(Span sp, const KState *st, C *x, int inverse) {
+  pdl_begin();
   const int b = blockIdx.y;
   using R = typename RealOf<C>::type;
   __shared__ R sf;  // one FP64 division per CTA, not per thread
@@ -83,6 +86,7 @@ __global__ void __launch_bounds__(kRedThreads) k_init(Span sp, const KState *st,
                                                       C *__restrict__ v, C *__restrict__ r,
                                                       C *__restrict__ rhat, C *__restrict__ p,
                                                       C *__restrict__ x, int x_zero, double *part) {
+  pdl_begin();
   const int b = blockIdx.y;
   using A = typename Acc<C>::type;
   using R = typename RealOf<C>::type;
@@ -106,6 +110,7 @@ __global__ void __launch_bounds__(kRedThreads) k_init(Span sp, const KState *st,
 
 __global__ void k_init_state(KState *st, int *active, int *counters, int *arrived, const double *part, int nblk,
                              double tol, int max_iter) {
+  pdl_begin();
   const int b = blockIdx.x;
   double s[2];
   gather_n<2>(part + size_t(b) * kRedBlocks * kRedSlots, nblk, s);
@@ -133,6 +138,7 @@ __global__ void k_init_state(KState *st, int *active, int *counters, int *arrive
 
 template <typename C>
 __global__ void k_zero_flagged(Span sp, const KState *st, C *x) {
+  pdl_begin();
   const int b = blockIdx.y;
   if (!st[blockIdx.y].zero_rhs) return;
   DBI_PROBLEM_LOOP(sp) x[off + i] = czero<C>();
@@ -143,6 +149,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_p(Span sp, const int *pl
                                                           const int *active, int *counters, int parity,
                                                           const C *__restrict__ r, C *__restrict__ rhat,
                                                           C *__restrict__ p, const C *__restrict__ v) {
+  pdl_begin();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) counters[parity] = 0;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
@@ -170,6 +177,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_p(Span sp, const int *pl
 
 // alpha of every active problem (one warp each): the paths whose operator does not finish it.
 __global__ void k_alpha(const int *plist, KState *st, const int *active, int nparts, const double *partA) {
+  pdl_begin();
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
   finish_alpha(st, b, partA + size_t(b) * nparts * kRedSlots, nparts);
@@ -180,6 +188,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_s(Span sp, const int *pl
                                                           const int *active, const C *__restrict__ r,
                                                           const C *__restrict__ v, C *__restrict__ s,
                                                           double *partS) {
+  pdl_begin();
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
@@ -203,6 +212,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_s(Span sp, const int *pl
 // omega of every active problem (one warp each), likewise.
 __global__ void k_omega(const int *plist, KState *st, const int *active, int nparts, const double *partB,
                         const double *partS, int nS, double tol) {
+  pdl_begin();
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
   finish_omega(st, b, partB + size_t(b) * nparts * kRedSlots, nparts, partS + size_t(b) * kRedBlocks * kRedSlots, nS,
@@ -216,6 +226,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *p
                                                            const C *__restrict__ s, const C *__restrict__ t,
                                                            const C *__restrict__ rhat, C *__restrict__ x,
                                                            C *__restrict__ r, double *partC) {
+  pdl_begin();
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, blockIdx.y);
   if (!active[b]) return;
@@ -259,6 +270,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *p
 
 // plist = the active problems in ascending order, count = how many (one CTA of 1024 threads).
 __global__ void __launch_bounds__(1024) k_compact(int B, const int *active, int *plist, int *count) {
+  pdl_begin();
   __shared__ int warp_tot[32];
   __shared__ int base;
   if (threadIdx.x == 0) base = 0;
@@ -285,11 +297,12 @@ __global__ void __launch_bounds__(1024) k_compact(int B, const int *active, int 
 }
 
 int compact_active(int B, const int *active, int *plist, int *count, cudaStream_t s) {
-  k_compact<<<1, 1024, 0, s>>>(B, active, plist, count);
+  launch_pdl(k_compact, 1, 1024, 0, s, B, active, plist, count);
   return check_launch("k_compact");
 }
 
 __global__ void k_finalize(int B, const KState *st, int *iters, double *relres, int *code) {
+  pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const KState k = st[b];
@@ -302,6 +315,7 @@ __global__ void k_finalize(int B, const KState *st, int *iters, double *relres, 
 // power-of-two normalisers
 // ---------------------------------------------------------------------------------------------
 __global__ void k_pow2(const double *part, int nblk, double *scale, double *inv, const double *extra) {
+  pdl_begin();
   const double m = gather_max(part + size_t(blockIdx.x) * kRedBlocks * kRedSlots, nblk);
   if (threadIdx.x == 0) {
     const double sc = pow2_below(m);
@@ -316,15 +330,15 @@ int pow2_scales(const void *x, int precision, bool real, int B, size_t n, double
   const dim3 grid(nblk, B);
   const Span sp{n, offs};
   if (precision == DBI_C64) {
-    if (real) k_absmax<float><<<grid, kRedThreads, 0, s>>>(sp, static_cast<const float *>(x), part);
-    else k_absmax<float2><<<grid, kRedThreads, 0, s>>>(sp, static_cast<const float2 *>(x), part);
+    if (real) launch_pdl(k_absmax<float>, grid, kRedThreads, 0, s, sp, static_cast<const float *>(x), part);
+    else launch_pdl(k_absmax<float2>, grid, kRedThreads, 0, s, sp, static_cast<const float2 *>(x), part);
   } else {
-    if (real) k_absmax<double><<<grid, kRedThreads, 0, s>>>(sp, static_cast<const double *>(x), part);
-    else k_absmax<double2><<<grid, kRedThreads, 0, s>>>(sp, static_cast<const double2 *>(x), part);
+    if (real) launch_pdl(k_absmax<double>, grid, kRedThreads, 0, s, sp, static_cast<const double *>(x), part);
+    else launch_pdl(k_absmax<double2>, grid, kRedThreads, 0, s, sp, static_cast<const double2 *>(x), part);
   }
   int rc;
   if ((rc = check_launch("k_absmax"))) return rc;
-  k_pow2<<<B, 32, 0, s>>>(part, nblk, scale, inv, extra);
+  launch_pdl(k_pow2, B, 32, 0, s, part, nblk, scale, inv, extra);
   return check_launch("k_pow2");
 }
 
@@ -401,22 +415,22 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   if (fused) op.finish = &fin;
   op.stencil = true;
   op.active = nullptr;
-  k_absmax<C><<<grid, kRedThreads, 0, s>>>(sp, rhs, sb.partA);
+  launch_pdl(k_absmax<C>, grid, kRedThreads, 0, s, sp, rhs, sb.partA);
   if ((rc = check_launch("k_absmax"))) return rc;
-  k_scale<<<B, 32, 0, s>>>(sb.st, sb.partA, nblk);
+  launch_pdl(k_scale, B, 32, 0, s, sb.st, sb.partA, nblk);
   if ((rc = check_launch("k_scale"))) return rc;
   if (!x_zero) {  // x0 into the scaled system, v = A x0
-    k_scale_x<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, x, 0);
+    launch_pdl(k_scale_x<C>, grid, kRedThreads, 0, s, sp, sb.st, x, 0);
     if ((rc = check_launch("k_scale_x"))) return rc;
     op.in = x; op.ident = x; op.out = v;
     if ((rc = run_operator(op, s))) return rc;
   }
-  k_init<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, rhs, v, r, rhat, p, x, x_zero ? 1 : 0, sb.partA);
+  launch_pdl(k_init<C>, grid, kRedThreads, 0, s, sp, sb.st, rhs, v, r, rhat, p, x, x_zero ? 1 : 0, sb.partA);
   if ((rc = check_launch("k_init"))) return rc;
-  k_init_state<<<B, 32, 0, s>>>(sb.st, sb.active, sb.counters, sb.arrived, sb.partA, nblk, o.tol, o.max_iter);
+  launch_pdl(k_init_state, B, 32, 0, s, sb.st, sb.active, sb.counters, sb.arrived, sb.partA, nblk, o.tol, o.max_iter);
   if ((rc = check_launch("k_init_state"))) return rc;
   if (!x_zero) {
-    k_zero_flagged<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, x);
+    launch_pdl(k_zero_flagged<C>, grid, kRedThreads, 0, s, sp, sb.st, x);
     if ((rc = check_launch("k_zero_flagged"))) return rc;
   }
   // Batches on one grid run their launches over the problems still active: at every host check
@@ -426,7 +440,7 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   int nrun = B;   // launch slots: the compacted active problems, or every problem of an uneven batch
   const int *plist = nullptr;
   auto compact = [&]() -> int {
-    k_compact<<<1, 1024, 0, s>>>(B, sb.active, sb.plist, sb.counters + 2);
+    launch_pdl(k_compact, 1, 1024, 0, s, B, sb.active, sb.plist, sb.counters + 2);
     int e2 = check_launch("k_compact");
     if (e2 == DBI_OK) e2 = read_counter(sb.counters + 2, s, &nact);
     plist = sb.plist;
@@ -448,23 +462,23 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
     int rc2;
     op.plist = plist;
     op.nb = nrun;
-    k_update_p<C><<<g2, kRedThreads, 0, st>>>(sp, plist, sb.st, sb.active, sb.counters, parity, r, rhat, p, v);
+    launch_pdl(k_update_p<C>, g2, kRedThreads, 0, st, sp, plist, sb.st, sb.active, sb.counters, parity, r, rhat, p, v);
     if ((rc2 = check_launch("k_update_p"))) return rc2;
     op.epi = 1; op.in = p; op.ident = p; op.out = v; op.part_out = sb.partA;
     if ((rc2 = run_operator(op, st))) return rc2;
     if (!fused) {
-      k_alpha<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, nparts, sb.partA);
+      launch_pdl(k_alpha, nrun, 32, 0, st, plist, sb.st, sb.active, nparts, sb.partA);
       if ((rc2 = check_launch("k_alpha"))) return rc2;
     }
-    k_update_s<C><<<g2, kRedThreads, 0, st>>>(sp, plist, sb.st, sb.active, r, v, sv, sb.partS);
+    launch_pdl(k_update_s<C>, g2, kRedThreads, 0, st, sp, plist, sb.st, sb.active, r, v, sv, sb.partS);
     if ((rc2 = check_launch("k_update_s"))) return rc2;
     op.epi = 2; op.in = sv; op.ident = sv; op.out = t; op.part_out = sb.partB;
     if ((rc2 = run_operator(op, st))) return rc2;
     if (!fused) {
-      k_omega<<<nrun, 32, 0, st>>>(plist, sb.st, sb.active, nparts, sb.partB, sb.partS, nblk, o.tol);
+      launch_pdl(k_omega, nrun, 32, 0, st, plist, sb.st, sb.active, nparts, sb.partB, sb.partS, nblk, o.tol);
       if ((rc2 = check_launch("k_omega"))) return rc2;
     }
-    k_update_xr<C><<<g2, kRedThreads, 0, st>>>(sp, plist, sb.st, sb.active, sb.counters, parity, sb.arrived, o.tol,
+    launch_pdl(k_update_xr<C>, g2, kRedThreads, 0, st, sp, plist, sb.st, sb.active, sb.counters, parity, sb.arrived, o.tol,
                                                o.max_iter, p, sv, t, rhat, x, r, sb.partC);
     return check_launch("k_update_xr");
   };
@@ -504,11 +518,11 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   }
   op.plist = nullptr;
   if (unscale) {
-    k_scale_x<C><<<grid, kRedThreads, 0, s>>>(sp, sb.st, x, 1);
+    launch_pdl(k_scale_x<C>, grid, kRedThreads, 0, s, sp, sb.st, x, 1);
     if ((rc = check_launch("k_scale_x"))) return rc;
   }
   if (status) {
-    k_finalize<<<(B + 127) / 128, 128, 0, s>>>(B, sb.st, status->iters, status->relres, status->code);
+    launch_pdl(k_finalize, (B + 127) / 128, 128, 0, s, B, sb.st, status->iters, status->relres, status->code);
     if ((rc = check_launch("k_finalize"))) return rc;
   }
   return DBI_OK;

@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(128) k3_stress(int nz, int ny, int nx, typenam
                                                  const typename RealOf<C>::type *m, Ref6 ref,
                                                  const C *u, const double *in_scale, const int *plist,
                                                  const int *active, C *sig) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int zy = blockIdx.y, z = zy / ny, y = zy - z * ny, slot = blockIdx.z;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(128) k3_source(int nz, int ny, int nx, int ly,
                                                  Ref6 ref, const C *u, const double *in_scale,
                                                  const double *omega, const int *fidx, const int *plist,
                                                  const int *active, const C *sig, C *T) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int zy = blockIdx.y, z = zy / ny, y = zy - z * ny, slot = blockIdx.z;
@@ -119,6 +121,7 @@ template <typename C>
 __global__ void __launch_bounds__(128) k3_copy_source(int nz, int ny, int nx, int ly, int lx, const C *u,
                                                       const double *in_scale, const int *plist, const int *active,
                                                       C *T) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int zy = blockIdx.y, z = zy / ny, y = zy - z * ny, slot = blockIdx.z;
@@ -136,6 +139,7 @@ __global__ void __launch_bounds__(128) k3_copy_source(int nz, int ny, int nx, in
 template <typename C, int LX>
 __global__ void __launch_bounds__(256) k3_fft_x(int nb, int nz, int ny, int nx, int ly, const int *plist,
                                                 const int *active, const C *tw, C *T) {
+  pdl_begin();
   constexpr int NL = 2048 / LX, LS = LX + 1, NT = NL * LX / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *s = reinterpret_cast<C *>(smem_raw);
@@ -181,6 +185,7 @@ __global__ void __launch_bounds__(kTileThreads) k3_fft_x_reg(int nb, int nz, int
                                                              const int *active, const float2 *tw, float2 *T,
                                                              const float2 *ident, const double *out_scale,
                                                              float2 *out) {
+  pdl_begin();
   using C = float2;
   using X = XRegCfg<LX>;
   constexpr int TX = X::T;
@@ -237,6 +242,7 @@ template <typename C, int LY> struct YCfg {
 template <typename C, int LY, bool INV>
 __global__ void __launch_bounds__(256) k3_fft_y(int nz, int ny, int lx, const int *plist, const int *active,
                                                 const C *tw, C *T) {
+  pdl_begin();
   constexpr int CC = YCfg<C, LY>::CC, LS = YCfg<C, LY>::LS, NT = YCfg<C, LY>::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *s = reinterpret_cast<C *>(smem_raw);
@@ -273,6 +279,7 @@ template <int LY> struct YRegCfg {
 template <int LY, bool INV>
 __global__ void __launch_bounds__(kTileThreads, 4) k3_fft_y_reg(int nz, int ny, int lx, const int *plist,
                                                                const int *active, const float2 *tw, float2 *T) {
+  pdl_begin();
   using C = float2;
   using Y = YRegCfg<LY>;
   constexpr int TY = Y::T, CC = Y::CC, LP = Y::LP, NT = Y::NT;
@@ -334,6 +341,7 @@ template <typename C, int LZ>
 __global__ void __launch_bounds__(ZCfg<C, LZ>::NT, ZCfg<C, LZ>::MIN_BLOCKS) k3_fft_z_mul(int nb, int nz, int nf, size_t plane, const int *plist,
                                                                 const int *active, const int *fidx, const C *Ghat,
                                                                 const C *tw, C *T) {
+  pdl_begin();
   using Z = ZCfg<C, LZ>;
   constexpr int CC = Z::CC, NL = Z::NL, LS = Z::LS, NT = Z::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -397,6 +405,7 @@ template <int LZ>
 __global__ void __launch_bounds__(kTileThreads, DBI_3D_ZREG_MINB) k3_fft_z_reg(int nb, int nz, int nf, size_t plane, const int *plist,
                                                                const int *active, const int *fidx, const float2 *Ghat,
                                                                const float2 *tw, float2 *T) {
+  pdl_begin();
   using C = float2;
   using Z = ZRegCfg<LZ>;
   constexpr int TZ = Z::T, CC = Z::CC, LP = Z::LP, NT = Z::NT, NL = Z::NL;
@@ -466,6 +475,7 @@ template <typename C, int LX>
 __global__ void __launch_bounds__(256) k3_fft_x_epi(int nb, int nz, int ny, int nx, int ly, const int *plist,
                                                     const int *active, const C *tw, const C *T, const C *ident,
                                                     const double *out_scale, C *out) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   constexpr int NL = 2048 / LX, LS = LX + 1, NT = NL * LX / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -512,13 +522,13 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
   prof_mark(PROF_OPERATOR, false, s);
   const dim3 cg((a.nx + 127) / 128, a.nz * a.ny, nb);
   if (a.stencil) {
-    k3_stress<C><<<cg, 128, 0, s>>>(a.nz, a.ny, a.nx, inv2h, m, ref, in, a.in_scale, a.plist, a.active, sig);
+    launch_pdl(k3_stress<C>, cg, 128, 0, s, a.nz, a.ny, a.nx, inv2h, m, ref, in, a.in_scale, a.plist, a.active, sig);
     if ((rc = check_launch("k3_stress"))) return rc;
-    k3_source<C><<<cg, 128, 0, s>>>(a.nz, a.ny, a.nx, a.ly, a.lx, a.nf, inv2h, m, ref, in, a.in_scale, a.omega,
+    launch_pdl(k3_source<C>, cg, 128, 0, s, a.nz, a.ny, a.nx, a.ly, a.lx, a.nf, inv2h, m, ref, in, a.in_scale, a.omega,
                                     a.fidx, a.plist, a.active, sig, T);
     if ((rc = check_launch("k3_source"))) return rc;
   } else {
-    k3_copy_source<C><<<cg, 128, 0, s>>>(a.nz, a.ny, a.nx, a.ly, a.lx, in, a.in_scale, a.plist, a.active, T);
+    launch_pdl(k3_copy_source<C>, cg, 128, 0, s, a.nz, a.ny, a.nx, a.ly, a.lx, in, a.in_scale, a.plist, a.active, T);
     if ((rc = check_launch("k3_copy_source"))) return rc;
   }
   rc = DBI_ERR_UNSUPPORTED;
@@ -532,8 +542,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
         const long rows = long(nb) * 3 * a.nz * a.ny;
         cudaError_t e = allow_smem(k3_fft_x_reg<LX, EPI>, X::smem);
         if (e == cudaSuccess)
-          k3_fft_x_reg<LX, EPI><<<unsigned((rows + X::ROWS - 1) / X::ROWS), kTileThreads, X::smem, s>>>(
-              nb, a.nz, a.ny, a.nx, a.ly, a.plist, a.active, reinterpret_cast<const float2 *>(tw),
+          launch_pdl(k3_fft_x_reg<LX, EPI>, unsigned((rows + X::ROWS - 1) / X::ROWS), kTileThreads, X::smem, s, nb, a.nz, a.ny, a.nx, a.ly, a.plist, a.active, reinterpret_cast<const float2 *>(tw),
               reinterpret_cast<float2 *>(T), static_cast<const float2 *>(a.ident), a.out_scale,
               static_cast<float2 *>(a.out));
         rc = e != cudaSuccess ? cuda_fail("k3_fft_x_reg smem", e) : check_launch("k3_fft_x_reg");
@@ -548,7 +557,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
     const long rows = long(nb) * 3 * a.nz * a.ny;
     cudaError_t e = allow_smem(k3_fft_x<C, LX>, bytes);
     if (e == cudaSuccess)
-      k3_fft_x<C, LX><<<unsigned((rows + NL - 1) / NL), NT, bytes, s>>>(nb, a.nz, a.ny, a.nx, a.ly, a.plist,
+      launch_pdl(k3_fft_x<C, LX>, unsigned((rows + NL - 1) / NL), NT, bytes, s, nb, a.nz, a.ny, a.nx, a.ly, a.plist,
                                                                        a.active, tw, T);
     rc = e != cudaSuccess ? cuda_fail("k3_fft_x smem", e) : check_launch("k3_fft_x");
   });
@@ -562,7 +571,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
         cudaError_t e = allow_smem(k3_fft_y_reg<LY, INV>, Y::smem);
         const dim3 grid((a.lx + Y::CC - 1) / Y::CC, nb * 3 * a.nz);
         if (e == cudaSuccess)
-          k3_fft_y_reg<LY, INV><<<grid, Y::NT, Y::smem, s>>>(a.nz, a.ny, a.lx, a.plist, a.active,
+          launch_pdl(k3_fft_y_reg<LY, INV>, grid, Y::NT, Y::smem, s, a.nz, a.ny, a.lx, a.plist, a.active,
                                                              reinterpret_cast<const float2 *>(tw),
                                                              reinterpret_cast<float2 *>(T));
         rc = e != cudaSuccess ? cuda_fail("k3_fft_y_reg smem", e) : check_launch("k3_fft_y_reg");
@@ -572,7 +581,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
       const size_t bytes = size_t(CC) * (LY + 1) * sizeof(C);
       cudaError_t e = allow_smem(k3_fft_y<C, LY, INV>, bytes);
       const dim3 grid((a.lx + CC - 1) / CC, nb * 3 * a.nz);
-      if (e == cudaSuccess) k3_fft_y<C, LY, INV><<<grid, NT, bytes, s>>>(a.nz, a.ny, a.lx, a.plist, a.active, tw, T);
+      if (e == cudaSuccess) launch_pdl(k3_fft_y<C, LY, INV>, grid, NT, bytes, s, a.nz, a.ny, a.lx, a.plist, a.active, tw, T);
       rc = e != cudaSuccess ? cuda_fail("k3_fft_y smem", e) : check_launch("k3_fft_y");
     });
     return rc;
@@ -592,8 +601,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
       }
       cudaError_t e = allow_smem(k3_fft_z_reg<LZ>, Z::smem);
       if (e == cudaSuccess)
-        k3_fft_z_reg<LZ><<<unsigned(blocks), Z::NT, Z::smem, s>>>(
-            nb, a.nz, a.nf, plane, a.plist, a.active, a.fidx, static_cast<const float2 *>(a.Ghat),
+        launch_pdl(k3_fft_z_reg<LZ>, unsigned(blocks), Z::NT, Z::smem, s, nb, a.nz, a.nf, plane, a.plist, a.active, a.fidx, static_cast<const float2 *>(a.Ghat),
             reinterpret_cast<const float2 *>(tw), reinterpret_cast<float2 *>(T));
       rc = e != cudaSuccess ? cuda_fail("k3_fft_z_reg smem", e) : check_launch("k3_fft_z_reg");
       return;
@@ -609,7 +617,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
       return;
     }
     if (e == cudaSuccess)
-      k3_fft_z_mul<C, LZ><<<unsigned(blocks), Z::NT, bytes, s>>>(nb, a.nz, a.nf, plane, a.plist, a.active, a.fidx,
+      launch_pdl(k3_fft_z_mul<C, LZ>, unsigned(blocks), Z::NT, bytes, s, nb, a.nz, a.nf, plane, a.plist, a.active, a.fidx,
                                                      static_cast<const C *>(a.Ghat), tw, T);
     rc = e != cudaSuccess ? cuda_fail("k3_fft_z_mul smem", e) : check_launch("k3_fft_z_mul");
   });
@@ -623,8 +631,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
     const long rows = long(nb) * 3 * a.nz * a.ny;
     cudaError_t e = allow_smem(k3_fft_x_epi<C, LX>, bytes);
     if (e == cudaSuccess)
-      k3_fft_x_epi<C, LX><<<unsigned((rows + NL - 1) / NL), NT, bytes, s>>>(
-          nb, a.nz, a.ny, a.nx, a.ly, a.plist, a.active, tw, T, static_cast<const C *>(a.ident), a.out_scale,
+      launch_pdl(k3_fft_x_epi<C, LX>, unsigned((rows + NL - 1) / NL), NT, bytes, s, nb, a.nz, a.ny, a.nx, a.ly, a.plist, a.active, tw, T, static_cast<const C *>(a.ident), a.out_scale,
           static_cast<C *>(a.out));
     rc = e != cudaSuccess ? cuda_fail("k3_fft_x_epi smem", e) : check_launch("k3_fft_x_epi");
   });
@@ -699,6 +706,7 @@ __device__ double2 green3_self(double h, double w, double alpha, double beta, do
 template <typename C>
 __global__ void k3_green_space(int nz, int ny, int nx, int lz, int ly, int lx, double h, const double *omega,
                                double rho, double alpha, double beta, double2 *W, C *Gspace) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int dx = blockIdx.x * blockDim.x + threadIdx.x;
   const int dzy = blockIdx.y, dz = dzy / ny, dy = dzy - dz * ny, f = blockIdx.z;
@@ -731,6 +739,7 @@ __global__ void k3_green_space(int nz, int ny, int nx, int lz, int ly, int lx, d
 
 template <typename C>
 __global__ void k3_scale_cast(const double2 *W, C *Ghat, size_t n, double scale) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
     Ghat[i] = mk<C>(R(W[i].x * scale), R(W[i].y * scale));
@@ -740,6 +749,7 @@ __global__ void k3_scale_cast(const double2 *W, C *Ghat, size_t n, double scale)
 template <typename C>
 __global__ void k3_incident(int nf, int nz, int ny, int nx, int lz, int ly, int lx, const int *fidx,
                             const C *Gspace, const int *src, const double *forces, C *u0) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int zy = blockIdx.y, z = zy / ny, y = zy - z * ny, b = blockIdx.z;
@@ -841,10 +851,10 @@ extern "C" int greens_tabulate_3d(const dbi_grid3 *g, const dbi_medium *ref, con
   if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync(3D Green table)", e);
   const dim3 grid((g->nx + 127) / 128, g->nz * g->ny, nf);
   if (precision == DBI_C64)
-    k3_green_space<float2><<<grid, 128, 0, s>>>(g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, g->h, omega, ref->rho0,
+    launch_pdl(k3_green_space<float2>, grid, 128, 0, s, g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, g->h, omega, ref->rho0,
                                                 ref->alpha0, ref->beta0, W, static_cast<float2 *>(Gspace));
   else
-    k3_green_space<double2><<<grid, 128, 0, s>>>(g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, g->h, omega,
+    launch_pdl(k3_green_space<double2>, grid, 128, 0, s, g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, g->h, omega,
                                                  ref->rho0, ref->alpha0, ref->beta0, W,
                                                  static_cast<double2 *>(Gspace));
   if ((rc = check_launch("k3_green_space"))) return rc;
@@ -854,8 +864,8 @@ extern "C" int greens_tabulate_3d(const dbi_grid3 *g, const dbi_medium *ref, con
   if ((rc = fft_cols_fp64(W, nf * 6, g->lz, g->ly * g->lx, tw, s))) return rc;
   const double scale = g->h * g->h * g->h / (double(g->lz) * g->ly * g->lx);
   const int blocks = int(std::min<size_t>((tab + 255) / 256, 8192));
-  if (precision == DBI_C64) k3_scale_cast<float2><<<blocks, 256, 0, s>>>(W, static_cast<float2 *>(Ghat), tab, scale);
-  else k3_scale_cast<double2><<<blocks, 256, 0, s>>>(W, static_cast<double2 *>(Ghat), tab, scale);
+  if (precision == DBI_C64) launch_pdl(k3_scale_cast<float2>, blocks, 256, 0, s, W, static_cast<float2 *>(Ghat), tab, scale);
+  else launch_pdl(k3_scale_cast<double2>, blocks, 256, 0, s, W, static_cast<double2 *>(Ghat), tab, scale);
   return check_launch("k3_scale_cast");
 }
 
@@ -870,11 +880,11 @@ extern "C" int incident_field_3d(const dbi_grid3 *g, const dbi_batch *batch, con
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const dim3 grid((g->nx + 127) / 128, g->nz * g->ny, batch->B);
   if (precision == DBI_C64)
-    k3_incident<float2><<<grid, 128, 0, s>>>(batch->nf, g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, batch->fidx,
+    launch_pdl(k3_incident<float2>, grid, 128, 0, s, batch->nf, g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, batch->fidx,
                                              static_cast<const float2 *>(Gspace), src_cells, forces,
                                              static_cast<float2 *>(u0));
   else
-    k3_incident<double2><<<grid, 128, 0, s>>>(batch->nf, g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, batch->fidx,
+    launch_pdl(k3_incident<double2>, grid, 128, 0, s, batch->nf, g->nz, g->ny, g->nx, g->lz, g->ly, g->lx, batch->fidx,
                                               static_cast<const double2 *>(Gspace), src_cells, forces,
                                               static_cast<double2 *>(u0));
   return check_launch("k3_incident");
@@ -978,6 +988,7 @@ namespace dbi {
 // d[b][r][c] = u[b][c] at receiver cell r (P u); out-of-range receivers give 0.
 template <typename C>
 __global__ void k3_sample(int B, int nz, int ny, int nx, int n_rec, const int *rec, const C *u, C *d) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * n_rec) return;
   const int b = i / n_rec, r = i - b * n_rec;
@@ -992,6 +1003,7 @@ __global__ void k3_sample(int B, int nz, int ny, int nx, int n_rec, const int *r
 // share a cell are summed).
 template <typename C>
 __global__ void k3_inject_conj(int B, int nz, int ny, int nx, int n_rec, const int *rec, const C *r, C *q) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * n_rec) return;
@@ -1013,6 +1025,7 @@ __global__ void k3_inject_conj(int B, int nz, int ny, int nx, int n_rec, const i
 template <typename C, typename GOut>
 __global__ void __launch_bounds__(128) k3_imaging(int B, int nf, int nz, int ny, int nx, double h, const double *omega,
                                                   const int *fidx, const C *ua, const C *ub, GOut *g) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int zy = blockIdx.y, z = zy / ny, y = zy - z * ny;
@@ -1101,10 +1114,10 @@ static int frechet3(const Ctx3 &c, const void *u_b, const int *rec, int n_rec, c
   if ((rc = run_operator(a, c.s)) || (rc = solve3(c, c.src, c.sol))) return rc;
   const int tot = B * n_rec;
   if (c.precision == DBI_C64)
-    k3_sample<float2><<<(tot + 127) / 128, 128, 0, c.s>>>(B, g->nz, g->ny, g->nx, n_rec, rec,
+    launch_pdl(k3_sample<float2>, (tot + 127) / 128, 128, 0, c.s, B, g->nz, g->ny, g->nx, n_rec, rec,
                                                           static_cast<const float2 *>(c.sol), static_cast<float2 *>(d));
   else
-    k3_sample<double2><<<(tot + 127) / 128, 128, 0, c.s>>>(B, g->nz, g->ny, g->nx, n_rec, rec,
+    launch_pdl(k3_sample<double2>, (tot + 127) / 128, 128, 0, c.s, B, g->nz, g->ny, g->nx, n_rec, rec,
                                                            static_cast<const double2 *>(c.sol),
                                                            static_cast<double2 *>(d));
   return check_launch("k3_sample");
@@ -1121,11 +1134,11 @@ static int adjoint3(const Ctx3 &c, const void *u_b, const int *rec, int n_rec, c
   cudaError_t e = cudaMemsetAsync(c.sol, 0, c.fbytes, c.s);
   if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync(adjoint source)", e);
   if (c.precision == DBI_C64)
-    k3_inject_conj<float2><<<(tot + 127) / 128, 128, 0, c.s>>>(B, g->nz, g->ny, g->nx, n_rec, rec,
+    launch_pdl(k3_inject_conj<float2>, (tot + 127) / 128, 128, 0, c.s, B, g->nz, g->ny, g->nx, n_rec, rec,
                                                                static_cast<const float2 *>(r),
                                                                static_cast<float2 *>(c.sol));
   else
-    k3_inject_conj<double2><<<(tot + 127) / 128, 128, 0, c.s>>>(B, g->nz, g->ny, g->nx, n_rec, rec,
+    launch_pdl(k3_inject_conj<double2>, (tot + 127) / 128, 128, 0, c.s, B, g->nz, g->ny, g->nx, n_rec, rec,
                                                                 static_cast<const double2 *>(r),
                                                                 static_cast<double2 *>(c.sol));
   if ((rc = check_launch("k3_inject_conj"))) return rc;
@@ -1137,11 +1150,11 @@ static int adjoint3(const Ctx3 &c, const void *u_b, const int *rec, int n_rec, c
   if ((rc = run_operator(a, c.s)) || (rc = solve3(c, c.src, c.sol))) return rc;
   const dim3 grid((g->nx + 127) / 128, g->nz * g->ny);
   if (c.precision == DBI_C64)
-    k3_imaging<float2, GOut><<<grid, 128, 0, c.s>>>(B, c.batch->nf, g->nz, g->ny, g->nx, g->h, c.batch->omega,
+    launch_pdl(k3_imaging<float2, GOut>, grid, 128, 0, c.s, B, c.batch->nf, g->nz, g->ny, g->nx, g->h, c.batch->omega,
                                                     c.batch->fidx, static_cast<const float2 *>(c.sol),
                                                     static_cast<const float2 *>(u_b), gout);
   else
-    k3_imaging<double2, GOut><<<grid, 128, 0, c.s>>>(B, c.batch->nf, g->nz, g->ny, g->nx, g->h, c.batch->omega,
+    launch_pdl(k3_imaging<double2, GOut>, grid, 128, 0, c.s, B, c.batch->nf, g->nz, g->ny, g->nx, g->h, c.batch->omega,
                                                      c.batch->fidx, static_cast<const double2 *>(c.sol),
                                                      static_cast<const double2 *>(u_b), gout);
   return check_launch("k3_imaging");
@@ -1229,6 +1242,7 @@ namespace dbi {
 template <typename TO>
 static __global__ void k3_mscale_norm(int np, size_t plane, const double *x, TO *y, MScale s, const double *sc,
                                       int invert) {
+  pdl_begin();
   const double f = invert ? (sc[S_INV] > 0.0 ? 1.0 / sc[S_INV] : 0.0) : sc[S_INV];
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np * plane; i += size_t(gridDim.x) * blockDim.x)
     y[i] = TO(x[i] * s.s[i / plane] * f);
@@ -1293,27 +1307,27 @@ extern "C" int normal_cg_3d(const dbi_model3 *background, const dbi_batch *batch
   const MScale one{{1, 1, 1, 1, 1, 1}};
   const int mblocks = int(std::min<size_t>((nm + 255) / 256, 4096));
   auto dot = [&](const double *a, const double *b) -> int {
-    k_mdot<<<kMBlocks, kMThreads, 0, s>>>(nm, a, b, part);
+    launch_pdl(k_mdot, kMBlocks, kMThreads, 0, s, nm, a, b, part);
     return check_launch("k_mdot");
   };
   auto scal = [&](int what, int k) -> int {
-    k_scalar<<<1, 32, 0, s>>>(what, part, sc, hist, k);
+    launch_pdl(k_scalar, 1, 32, 0, s, what, part, sc, hist, k);
     return check_launch("k_scalar");
   };
   auto H = [&](const double *pin, double *qout) -> int {  // S Re J^H J S p, applied to p / ||p||
     int e;
     if ((e = dot(pin, pin)) || (e = scal(3, 0))) return e;  // sc[S_INV] = 1 / ||p||
     if (precision == DBI_C64)
-      k3_mscale_norm<float><<<mblocks, 256, 0, s>>>(6, plane, pin, static_cast<float *>(dmt), MS, sc, 0);
-    else k3_mscale_norm<double><<<mblocks, 256, 0, s>>>(6, plane, pin, static_cast<double *>(dmt), MS, sc, 0);
+      launch_pdl(k3_mscale_norm<float>, mblocks, 256, 0, s, 6, plane, pin, static_cast<float *>(dmt), MS, sc, 0);
+    else launch_pdl(k3_mscale_norm<double>, mblocks, 256, 0, s, 6, plane, pin, static_cast<double *>(dmt), MS, sc, 0);
     if ((e = check_launch("k3_mscale_norm"))) return e;
     if ((e = frechet3(c, u_b, rec_cells, n_rec, dmt, dvec))) return e;
     if ((e = adjoint3<double>(c, u_b, rec_cells, n_rec, dvec, gd))) return e;
-    k3_mscale_norm<double><<<mblocks, 256, 0, s>>>(6, plane, gd, qout, MS, sc, 1);
+    launch_pdl(k3_mscale_norm<double>, mblocks, 256, 0, s, 6, plane, gd, qout, MS, sc, 1);
     return check_launch("k3_mscale_norm");
   };
   auto axpy = [&](int mode, const double *xx, double *yy, const double *qq, double *rr) -> int {
-    k_maxpy<<<mblocks, 256, 0, s>>>(nm, mode, sc, xx, yy, qq, rr);
+    launch_pdl(k_maxpy, mblocks, 256, 0, s, nm, mode, sc, xx, yy, qq, rr);
     return check_launch("k_maxpy");
   };
   double init_sc[16] = {0};
@@ -1323,8 +1337,8 @@ extern "C" int normal_cg_3d(const dbi_model3 *background, const dbi_batch *batch
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail("cudaMemcpyAsync(scalars)", e);
   if (!(cg->lambda > 0)) {  // lambda = lambda_rel x the Rayleigh quotient after power steps
-    if (precision == DBI_C64) k_mscale<float, double><<<mblocks, 256, 0, s>>>(6, plane, static_cast<const float *>(power_start), p, one);
-    else k_mscale<double, double><<<mblocks, 256, 0, s>>>(6, plane, static_cast<const double *>(power_start), p, one);
+    if (precision == DBI_C64) launch_pdl(k_mscale<float, double>, mblocks, 256, 0, s, 6, plane, static_cast<const float *>(power_start), p, one);
+    else launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 6, plane, static_cast<const double *>(power_start), p, one);
     if ((rc = check_launch("k_mscale"))) return rc;
     if ((rc = dot(p, p)) || (rc = scal(3, 0)) || (rc = axpy(2, p, p, nullptr, nullptr))) return rc;
     for (int it = 0; it < cg->power_iters; ++it)
@@ -1332,7 +1346,7 @@ extern "C" int normal_cg_3d(const dbi_model3 *background, const dbi_batch *batch
     if ((rc = H(p, q)) || (rc = dot(p, q)) || (rc = scal(4, 0))) return rc;
   }
   if ((rc = adjoint3<double>(c, u_b, rec_cells, n_rec, dd, gd))) return rc;  // r = p = S Re J^H dd, x = 0
-  k_mscale<double, double><<<mblocks, 256, 0, s>>>(6, plane, gd, r, MS);
+  launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 6, plane, gd, r, MS);
   if ((rc = check_launch("k_mscale"))) return rc;
   e = cudaMemsetAsync(x, 0, mb, s);
   if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync(x)", e);
@@ -1344,8 +1358,8 @@ extern "C" int normal_cg_3d(const dbi_model3 *background, const dbi_batch *batch
     if ((rc = dot(r, r)) || (rc = scal(2, k + 1))) return rc;
     if ((rc = axpy(1, r, p, nullptr, nullptr))) return rc;
   }
-  if (precision == DBI_C64) k_mscale<double, float><<<mblocks, 256, 0, s>>>(6, plane, x, static_cast<float *>(dm), MS);
-  else k_mscale<double, double><<<mblocks, 256, 0, s>>>(6, plane, x, static_cast<double *>(dm), MS);
+  if (precision == DBI_C64) launch_pdl(k_mscale<double, float>, mblocks, 256, 0, s, 6, plane, x, static_cast<float *>(dm), MS);
+  else launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 6, plane, x, static_cast<double *>(dm), MS);
   if ((rc = check_launch("k_mscale"))) return rc;
   double lam = 0.0;
   std::vector<double> h(size_t(cg->iters) + 1);
@@ -1369,10 +1383,10 @@ extern "C" int sample_3d(const dbi_grid3 *g, int B, const int *rec_cells, int n_
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int tot = B * n_rec;
   if (precision == DBI_C64)
-    k3_sample<float2><<<(tot + 127) / 128, 128, 0, s>>>(B, g->nz, g->ny, g->nx, n_rec, rec_cells,
+    launch_pdl(k3_sample<float2>, (tot + 127) / 128, 128, 0, s, B, g->nz, g->ny, g->nx, n_rec, rec_cells,
                                                         static_cast<const float2 *>(u), static_cast<float2 *>(d));
   else
-    k3_sample<double2><<<(tot + 127) / 128, 128, 0, s>>>(B, g->nz, g->ny, g->nx, n_rec, rec_cells,
+    launch_pdl(k3_sample<double2>, (tot + 127) / 128, 128, 0, s, B, g->nz, g->ny, g->nx, n_rec, rec_cells,
                                                          static_cast<const double2 *>(u), static_cast<double2 *>(d));
   return check_launch("k3_sample");
 }

@@ -84,6 +84,7 @@ template <typename C> struct BatchTile {
 
 template <typename C, int LX, bool STENCIL, int V, int NTT>
 __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowFwdMinBlocks(LX) : 1) k_rows_forward(OpP<C> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowFwdMinBl
 
 template <typename C, int LZ, int V, int NTT>
 __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::colMinBlocks : 1) k_cols(OpP<C> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -109,6 +111,7 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::colMinBlock
 // separate 8-byte lines and the tables read from L2 by every slot.
 template <int LZ, int V, int SL>
 __global__ void __launch_bounds__(kTileThreads, Cfg<float2>::colMinBlocks) k_cols_pairs(OpP<float2> p) {
+  pdl_begin();
   using CF = ColCfg<float2, LZ>;
   constexpr int COLS = CF::CC / SL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -148,6 +151,7 @@ template <int LZ, int SL> constexpr size_t cols_pairs_smem() {
 
 template <typename C, int LX, int EPI, int V, int NTT>
 __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowInvMinBlocks : 1) k_rows_inverse(OpP<C> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -158,6 +162,7 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowInvMinBl
 
 // Stages of the L = 1024 complex64 operator as pairs of 512-point transforms (op_split.cuh).
 __global__ void __launch_bounds__(kSrcThreads) k_source_split(OpP<float2> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -167,6 +172,7 @@ __global__ void __launch_bounds__(kSrcThreads) k_source_split(OpP<float2> p) {
 
 template <bool STENCIL>
 __global__ void __launch_bounds__(kTileThreads, 2) k_rows_forward_split(OpP<float2> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -182,6 +188,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_rows_forward_split(OpP<floa
 // that frequency (consecutive slots share it, problems being frequency-major) read them there,
 // others from global memory.
 __global__ void __launch_bounds__(kTileThreads, 2) k_cols_split(OpP<float2> p) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2 *smem = reinterpret_cast<float2 *>(smem_raw);
   float4 *Gs = reinterpret_cast<float4 *>(smem + split_cols_lines_smem() / sizeof(float2));
@@ -210,6 +217,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_cols_split(OpP<float2> p) {
 
 template <int EPI>
 __global__ void __launch_bounds__(kTileThreads, 2) k_rows_inverse_split(OpP<float2> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -222,6 +230,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_rows_inverse_split(OpP<floa
 // the contrast source comes from k_source_split.
 template <bool STENCIL>
 __global__ void __launch_bounds__(kS3Threads, 2) k_rows_forward_s3(OpP<float2> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -232,6 +241,7 @@ __global__ void __launch_bounds__(kS3Threads, 2) k_rows_forward_s3(OpP<float2> p
 }
 
 __global__ void __launch_bounds__(kS3Threads, 2) k_cols_s3(OpP<float2> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -240,6 +250,7 @@ __global__ void __launch_bounds__(kS3Threads, 2) k_cols_s3(OpP<float2> p) {
 
 template <int EPI>
 __global__ void __launch_bounds__(kS3Threads, 2) k_rows_inverse_s3(OpP<float2> p) {
+  pdl_begin();
   const int b = problem_of(p), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -316,7 +327,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
       if (stencil) {
         const int chunks = (a.nz + kSrcRows - 1) / kSrcRows;
         e = allow_smem(k_source_split, source_smem());
-        if (e == cudaSuccess) k_source_split<<<dim3(chunks, nb), kSrcThreads, source_smem(), s>>>(q);
+        if (e == cudaSuccess) launch_pdl(k_source_split, dim3(chunks, nb), kSrcThreads, source_smem(), s, q);
         rc = e != cudaSuccess ? cuda_fail("k_source_split smem", e) : check_launch("k_source_split");
         if (rc) return rc;
       }
@@ -324,13 +335,13 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
         const dim3 grid((a.nz + kSplitRows - 1) / kSplitRows, nb);
         auto kern = stencil ? k_rows_forward_split<true> : k_rows_forward_split<false>;
         e = allow_smem(kern, split_rows_smem());
-        if (e == cudaSuccess) kern<<<grid, kTileThreads, split_rows_smem(), s>>>(q);
+        if (e == cudaSuccess) launch_pdl(kern, grid, kTileThreads, split_rows_smem(), s, q);
         rc = e != cudaSuccess ? cuda_fail("k_rows_forward_split smem", e) : check_launch("k_rows_forward_split");
       } else {
         const dim3 grid((a.nz + kS3Units - 1) / kS3Units, nb);
         auto kern = stencil ? k_rows_forward_s3<true> : k_rows_forward_s3<false>;
         e = allow_smem(kern, s3_smem());
-        if (e == cudaSuccess) kern<<<grid, kS3Threads, s3_smem(), s>>>(q);
+        if (e == cudaSuccess) launch_pdl(kern, grid, kS3Threads, s3_smem(), s, q);
         rc = e != cudaSuccess ? cuda_fail("k_rows_forward_s3 smem", e) : check_launch("k_rows_forward_s3");
       }
     }
@@ -344,7 +355,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
         dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
         auto launch = [&](auto kernel) {
           e = allow_smem(kernel, bytes);
-          if (e == cudaSuccess) kernel<<<grid, RC::NT, bytes, s>>>(p);
+          if (e == cudaSuccess) launch_pdl(kernel, grid, RC::NT, bytes, s, p);
         };
         if (stencil) launch(k_rows_forward<C, LX, true, V, NTT>);
         else launch(k_rows_forward<C, LX, false, V, NTT>);
@@ -360,13 +371,13 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
       OpP<float2> &q = reinterpret_cast<OpP<float2> &>(p);
       const dim3 grid(a.lx, (nb + 3) / 4);
       cudaError_t e = allow_smem(k_cols_split, split_cols_staged_smem());
-      if (e == cudaSuccess) k_cols_split<<<grid, kTileThreads, split_cols_staged_smem(), s>>>(q);
+      if (e == cudaSuccess) launch_pdl(k_cols_split, grid, kTileThreads, split_cols_staged_smem(), s, q);
       rc = e != cudaSuccess ? cuda_fail("k_cols_split smem", e) : check_launch("k_cols_split");
     } else if (kc == kSplitTriple) {
       OpP<float2> &q = reinterpret_cast<OpP<float2> &>(p);
       const dim3 grid((a.lx + kS3Units - 1) / kS3Units, nb);
       cudaError_t e = allow_smem(k_cols_s3, s3_smem());
-      if (e == cudaSuccess) k_cols_s3<<<grid, kS3Threads, s3_smem(), s>>>(q);
+      if (e == cudaSuccess) launch_pdl(k_cols_s3, grid, kS3Threads, s3_smem(), s, q);
       rc = e != cudaSuccess ? cuda_fail("k_cols_s3 smem", e) : check_launch("k_cols_s3");
     }
   }
@@ -381,7 +392,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
             const size_t bytes = cols_pairs_smem<LZ, SL>();
             e = allow_smem(k_cols_pairs<LZ, V, SL>, bytes);
             if (e == cudaSuccess)
-              k_cols_pairs<LZ, V, SL><<<dim3((a.lx + COLS - 1) / COLS, (nb + SL - 1) / SL), CF::NT, bytes, s>>>(p);
+              launch_pdl(k_cols_pairs<LZ, V, SL>, dim3((a.lx + COLS - 1) / COLS, (nb + SL - 1) / SL), CF::NT, bytes, s, p);
           };
           // four slots per CTA unless the last group would leave much of its CTAs idle
           if (nb % 4 == 0 || nb >= 16) launch.template operator()<4>();
@@ -395,7 +406,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           const size_t bytes = cols_smem<C, LZ, NTT>();
           dim3 grid((a.lx + CN::CC - 1) / CN::CC, nb);
           e = allow_smem(k_cols<C, LZ, V, NTT>, bytes);
-          if (e == cudaSuccess) k_cols<C, LZ, V, NTT><<<grid, CN::NT, bytes, s>>>(p);
+          if (e == cudaSuccess) launch_pdl(k_cols<C, LZ, V, NTT>, grid, CN::NT, bytes, s, p);
         });
         rc = e != cudaSuccess ? cuda_fail("k_cols smem", e) : check_launch("k_cols");
       }
@@ -410,14 +421,14 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
       const dim3 grid((a.nz + kSplitRows - 1) / kSplitRows, nb);
       auto kern = a.epi == 1 ? k_rows_inverse_split<1> : a.epi == 2 ? k_rows_inverse_split<2> : k_rows_inverse_split<0>;
       cudaError_t e = allow_smem(kern, split_rows_inverse_smem());
-      if (e == cudaSuccess) kern<<<grid, kTileThreads, split_rows_inverse_smem(), s>>>(q);
+      if (e == cudaSuccess) launch_pdl(kern, grid, kTileThreads, split_rows_inverse_smem(), s, q);
       rc = e != cudaSuccess ? cuda_fail("k_rows_inverse_split smem", e) : check_launch("k_rows_inverse_split");
     } else if (kr == kSplitTriple) {
       OpP<float2> &q = reinterpret_cast<OpP<float2> &>(p);
       const dim3 grid((a.nz + kS3Units - 1) / kS3Units, nb);
       auto kern = a.epi == 1 ? k_rows_inverse_s3<1> : a.epi == 2 ? k_rows_inverse_s3<2> : k_rows_inverse_s3<0>;
       cudaError_t e = allow_smem(kern, s3_smem());
-      if (e == cudaSuccess) kern<<<grid, kS3Threads, s3_smem(), s>>>(q);
+      if (e == cudaSuccess) launch_pdl(kern, grid, kS3Threads, s3_smem(), s, q);
       rc = e != cudaSuccess ? cuda_fail("k_rows_inverse_s3 smem", e) : check_launch("k_rows_inverse_s3");
     }
   }
@@ -430,7 +441,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
         dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
         auto launch = [&](auto kernel) {
           e = allow_smem(kernel, bytes);
-          if (e == cudaSuccess) kernel<<<grid, RC::NT, bytes, s>>>(p);
+          if (e == cudaSuccess) launch_pdl(kernel, grid, RC::NT, bytes, s, p);
         };
         if (a.epi == 1) launch(k_rows_inverse<C, LX, 1, V, NTT>);
         else if (a.epi == 2) launch(k_rows_inverse<C, LX, 2, V, NTT>);

@@ -9,6 +9,7 @@ namespace dbi {
 constexpr int kMBlocks = 64, kMThreads = 256;
 
 static __global__ void k_mdot(size_t n, const double *a, const double *b, double *part) {
+  pdl_begin();
   __shared__ double sh[kMThreads / 32];
   double acc = 0.0;
   for (size_t i = size_t(blockIdx.x) * kMThreads + threadIdx.x; i < n; i += size_t(kMBlocks) * kMThreads)
@@ -34,6 +35,7 @@ static __device__ __forceinline__ double sum_parts(const double *part) {
 enum { S_RR = 0, S_ALPHA = 1, S_BETA = 2, S_LAMBDA = 3, S_INV = 4, S_LREL = 5 };
 
 static __global__ void k_scalar(int what, const double *part, double *sc, double *hist, int k) {
+  pdl_begin();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double s = sum_parts(part);
   switch (what) {
@@ -61,6 +63,7 @@ static __global__ void k_scalar(int what, const double *part, double *sc, double
 // y = alpha_sel * x + beta_sel * y elementwise with scalars picked from sc (or 1 / 0)
 static __global__ void k_maxpy(size_t n, int mode, const double *sc, const double *x, double *y,
                         const double *q, double *r) {
+  pdl_begin();
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     switch (mode) {
       case 0:  // x += alpha p (y = x, x = p); r -= alpha q
@@ -89,6 +92,7 @@ struct MScale {
 };
 template <typename TI, typename TO>
 static __global__ void k_mscale(int np, size_t plane, const TI *x, TO *y, MScale sc) {
+  pdl_begin();
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < np * plane; i += size_t(gridDim.x) * blockDim.x)
     y[i] = TO(double(x[i]) * sc.s[i / plane]);
 }

@@ -30,6 +30,7 @@ __device__ __forceinline__ bool rec_ok(const int *cells, int k, int nz, int nx, 
 // d = fac[b] * P u, the factor applied in FP64
 template <typename C>
 __global__ void k_sample(int B, int nrec, int nz, int nx, const int *cells, const C *u, const double *fac, C *d) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
@@ -46,6 +47,7 @@ __global__ void k_sample(int B, int nrec, int nz, int nx, const int *cells, cons
 
 template <typename C>
 __global__ void k_zero(size_t n, C *x) {
+  pdl_begin();
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
     x[i] = czero<C>();
 }
@@ -53,6 +55,7 @@ __global__ void k_zero(size_t n, C *x) {
 // q = P^T conj(r): one thread per (problem, component) adds the receivers in order.
 template <typename C>
 __global__ void k_inject_conj(int B, int nrec, int nz, int nx, const int *cells, const C *r, C *q) {
+  pdl_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * B) return;
   const int b = t >> 1, c = t & 1;
@@ -90,6 +93,7 @@ template <typename C>
 __global__ void k_imaging_part(int B, int pb, int nf, int nz, int nx, double h, const double *omega,
                                const int *fidx, const C *ua, const C *ub, const double *src_scale,
                                const KState *st, const double *ub_scale, double *part) {
+  pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int z = blockIdx.y;
@@ -131,6 +135,7 @@ __global__ void k_imaging_part(int B, int pb, int nf, int nz, int nx, double h, 
 // g = sum of the chunks' partial images, in chunk order.
 template <typename GOut>
 __global__ void k_imaging_sum(size_t n, int nch, const double *part, GOut *g) {
+  pdl_begin();
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     double a = 0.0;
     for (int c = 0; c < nch; ++c) a += part[size_t(c) * n + i];
@@ -144,6 +149,7 @@ __global__ void k_imaging_sum(size_t n, int nch, const double *part, GOut *g) {
 template <typename C>
 __global__ void k_residual(int B, int nrec, int nz, int nx, const int *cells, const C *u, const C *dobs,
                            C *r, double *phi) {
+  pdl_begin();
   __shared__ double sh[32];
   double acc = 0.0;
   const int total = B * nrec;
@@ -224,10 +230,10 @@ static int frechet_internal(const ProdCtx &c, const void *u_b, const dbi_receive
   if ((rc = solve_background(c, c.f1, c.f2, true))) return rc;
   dim3 grid((rec->n + 127) / 128, B);
   if (c.precision == DBI_C64)
-    k_sample<float2><<<grid, 128, 0, c.s>>>(B, rec->n, c.g->nz, c.g->nx, rec->cells,
+    launch_pdl(k_sample<float2>, grid, 128, 0, c.s, B, rec->n, c.g->nz, c.g->nx, rec->cells,
                                             static_cast<const float2 *>(c.f2), c.sc.inv, static_cast<float2 *>(d));
   else
-    k_sample<double2><<<grid, 128, 0, c.s>>>(B, rec->n, c.g->nz, c.g->nx, rec->cells,
+    launch_pdl(k_sample<double2>, grid, 128, 0, c.s, B, rec->n, c.g->nz, c.g->nx, rec->cells,
                                              static_cast<const double2 *>(c.f2), c.sc.inv, static_cast<double2 *>(d));
   return check_launch("k_sample");
 }
@@ -241,14 +247,14 @@ static int adjoint_internal(const ProdCtx &c, const void *u_b, const dbi_receive
   const int zb = int(std::min<size_t>((n + 255) / 256, 8192));
   // q = P^T conj(r) in f2, then f1 = K q, then f2 = A_b^{-1} f1
   if (c.precision == DBI_C64) {
-    k_zero<float2><<<zb, 256, 0, c.s>>>(n, static_cast<float2 *>(c.f2));
+    launch_pdl(k_zero<float2>, zb, 256, 0, c.s, n, static_cast<float2 *>(c.f2));
     if ((rc = check_launch("k_zero"))) return rc;
-    k_inject_conj<float2><<<(2 * B + 127) / 128, 128, 0, c.s>>>(B, rec->n, nz, nx, rec->cells,
+    launch_pdl(k_inject_conj<float2>, (2 * B + 127) / 128, 128, 0, c.s, B, rec->n, nz, nx, rec->cells,
                                                                 static_cast<const float2 *>(r), static_cast<float2 *>(c.f2));
   } else {
-    k_zero<double2><<<zb, 256, 0, c.s>>>(n, static_cast<double2 *>(c.f2));
+    launch_pdl(k_zero<double2>, zb, 256, 0, c.s, n, static_cast<double2 *>(c.f2));
     if ((rc = check_launch("k_zero"))) return rc;
-    k_inject_conj<double2><<<(2 * B + 127) / 128, 128, 0, c.s>>>(B, rec->n, nz, nx, rec->cells,
+    launch_pdl(k_inject_conj<double2>, (2 * B + 127) / 128, 128, 0, c.s, B, rec->n, nz, nx, rec->cells,
                                                                  static_cast<const double2 *>(r), static_cast<double2 *>(c.f2));
   }
   if ((rc = check_launch("k_inject_conj"))) return rc;
@@ -269,18 +275,18 @@ static int adjoint_internal(const ProdCtx &c, const void *u_b, const dbi_receive
   const int nch = imaging_chunks(B), pb = (B + nch - 1) / nch;
   dim3 grid((nx + 127) / 128, nz, nch);
   if (c.precision == DBI_C64)
-    k_imaging_part<float2><<<grid, 128, 0, c.s>>>(B, pb, c.batch->nf, nz, nx, c.g->h, c.batch->omega,
+    launch_pdl(k_imaging_part<float2>, grid, 128, 0, c.s, B, pb, c.batch->nf, nz, nx, c.g->h, c.batch->omega,
                                                   c.batch->fidx, static_cast<const float2 *>(c.f2),
                                                   static_cast<const float2 *>(u_b), c.sc.scale, c.sb.st,
                                                   c.sc.aux, c.img);
   else
-    k_imaging_part<double2><<<grid, 128, 0, c.s>>>(B, pb, c.batch->nf, nz, nx, c.g->h, c.batch->omega,
+    launch_pdl(k_imaging_part<double2>, grid, 128, 0, c.s, B, pb, c.batch->nf, nz, nx, c.g->h, c.batch->omega,
                                                    c.batch->fidx, static_cast<const double2 *>(c.f2),
                                                    static_cast<const double2 *>(u_b), c.sc.scale, c.sb.st,
                                                    c.sc.aux, c.img);
   if ((rc = check_launch("k_imaging_part"))) return rc;
   const size_t nm = size_t(5) * nz * nx;
-  k_imaging_sum<GOut><<<int(std::min<size_t>((nm + 255) / 256, 4096)), 256, 0, c.s>>>(nm, nch, c.img, g);
+  launch_pdl(k_imaging_sum<GOut>, int(std::min<size_t>((nm + 255) / 256, 4096)), 256, 0, c.s, nm, nch, c.img, g);
   return check_launch("k_imaging_sum");
 }
 
@@ -376,11 +382,11 @@ extern "C" int data_residual(const dbi_grid *g, const dbi_batch *batch, const db
   if (batch->B > 0 && rec->n > 0 && (!u || !d_obs || !r)) { set_error("NULL u, d_obs or r"); return DBI_ERR_ARG; }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (precision == DBI_C64)
-    k_residual<float2><<<1, 1024, 0, s>>>(batch->B, rec->n, g->nz, g->nx, rec->cells,
+    launch_pdl(k_residual<float2>, 1, 1024, 0, s, batch->B, rec->n, g->nz, g->nx, rec->cells,
                                           static_cast<const float2 *>(u), static_cast<const float2 *>(d_obs),
                                           static_cast<float2 *>(r), phi);
   else
-    k_residual<double2><<<1, 1024, 0, s>>>(batch->B, rec->n, g->nz, g->nx, rec->cells,
+    launch_pdl(k_residual<double2>, 1, 1024, 0, s, batch->B, rec->n, g->nz, g->nx, rec->cells,
                                            static_cast<const double2 *>(u), static_cast<const double2 *>(d_obs),
                                            static_cast<double2 *>(r), phi);
   return check_launch("k_residual");
@@ -427,24 +433,24 @@ extern "C" int normal_cg(const dbi_model *background, const dbi_batch *batch, co
   // q = S adjoint(frechet(S p)) in FP64 model space
   auto H = [&](const double *pin, double *qout) -> int {
     int e;
-    if (precision == DBI_C64) k_mscale<double, float><<<mblocks, 256, 0, s>>>(5, plane, pin, static_cast<float *>(dmt), MS);
-    else k_mscale<double, double><<<mblocks, 256, 0, s>>>(5, plane, pin, static_cast<double *>(dmt), MS);
+    if (precision == DBI_C64) launch_pdl(k_mscale<double, float>, mblocks, 256, 0, s, 5, plane, pin, static_cast<float *>(dmt), MS);
+    else launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 5, plane, pin, static_cast<double *>(dmt), MS);
     if ((e = check_launch("k_mscale"))) return e;
     if ((e = frechet_internal(c, u_b, rec, dmt, dvec))) return e;
     if ((e = adjoint_internal<double>(c, u_b, rec, dvec, gd))) return e;
-    k_mscale<double, double><<<mblocks, 256, 0, s>>>(5, plane, gd, qout, MS);
+    launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 5, plane, gd, qout, MS);
     return check_launch("k_mscale");
   };
   auto dot = [&](const double *a, const double *b) -> int {
-    k_mdot<<<kMBlocks, kMThreads, 0, s>>>(nm, a, b, part);
+    launch_pdl(k_mdot, kMBlocks, kMThreads, 0, s, nm, a, b, part);
     return check_launch("k_mdot");
   };
   auto scal = [&](int what, int k) -> int {
-    k_scalar<<<1, 32, 0, s>>>(what, part, sc, hist, k);
+    launch_pdl(k_scalar, 1, 32, 0, s, what, part, sc, hist, k);
     return check_launch("k_scalar");
   };
   auto axpy = [&](int mode, const double *xx, double *yy, const double *qq, double *rr) -> int {
-    k_maxpy<<<mblocks, 256, 0, s>>>(nm, mode, sc, xx, yy, qq, rr);
+    launch_pdl(k_maxpy, mblocks, 256, 0, s, nm, mode, sc, xx, yy, qq, rr);
     return check_launch("k_maxpy");
   };
 
@@ -457,8 +463,8 @@ extern "C" int normal_cg(const dbi_model *background, const dbi_batch *batch, co
 
   if (!(cg->lambda > 0)) {  // power iteration on Re J~^H J~
     const MScale one{{1, 1, 1, 1, 1, 1}};
-    if (precision == DBI_C64) k_mscale<float, double><<<mblocks, 256, 0, s>>>(5, plane, static_cast<const float *>(power_start), p, one);
-    else k_mscale<double, double><<<mblocks, 256, 0, s>>>(5, plane, static_cast<const double *>(power_start), p, one);
+    if (precision == DBI_C64) launch_pdl(k_mscale<float, double>, mblocks, 256, 0, s, 5, plane, static_cast<const float *>(power_start), p, one);
+    else launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 5, plane, static_cast<const double *>(power_start), p, one);
     if ((rc = check_launch("k_mscale"))) return rc;
     if ((rc = dot(p, p)) || (rc = scal(3, 0)) || (rc = axpy(2, p, p, nullptr, nullptr))) return rc;
     for (int it = 0; it < cg->power_iters; ++it) {
@@ -468,7 +474,7 @@ extern "C" int normal_cg(const dbi_model *background, const dbi_batch *batch, co
   }
   // CG from x = 0: r = p = S Re J^H dd
   if ((rc = adjoint_internal<double>(c, u_b, rec, dd, gd))) return rc;
-  k_mscale<double, double><<<mblocks, 256, 0, s>>>(5, plane, gd, r, MS);
+  launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 5, plane, gd, r, MS);
   if ((rc = check_launch("k_mscale"))) return rc;
   e = cudaMemsetAsync(x, 0, mb, s);
   if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync(x)", e);
@@ -480,8 +486,8 @@ extern "C" int normal_cg(const dbi_model *background, const dbi_batch *batch, co
     if ((rc = dot(r, r)) || (rc = scal(2, k + 1))) return rc;                  // beta, hist
     if ((rc = axpy(1, r, p, nullptr, nullptr))) return rc;                     // p
   }
-  if (precision == DBI_C64) k_mscale<double, float><<<mblocks, 256, 0, s>>>(5, plane, x, static_cast<float *>(dm), MS);
-  else k_mscale<double, double><<<mblocks, 256, 0, s>>>(5, plane, x, static_cast<double *>(dm), MS);
+  if (precision == DBI_C64) launch_pdl(k_mscale<double, float>, mblocks, 256, 0, s, 5, plane, x, static_cast<float *>(dm), MS);
+  else launch_pdl(k_mscale<double, double>, mblocks, 256, 0, s, 5, plane, x, static_cast<double *>(dm), MS);
   if ((rc = check_launch("k_mscale"))) return rc;
   double lam = 0.0;
   std::vector<double> h(size_t(cg->iters) + 1);
