@@ -7,6 +7,7 @@
 //   k_rows_inverse : inverse FFT along x of a few rows, out = ident - result (or the result)
 #include <algorithm>
 
+#include "fft16.cuh"
 #include "group.cuh"
 #include "krylov_finish.cuh"
 #include "op_split.cuh"
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::colMinBlock
   cols_tile<C, LZ, V, NTT>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x, reinterpret_cast<C *>(smem_raw));
 }
 
-// The complex64 column stage: a CTA takes the columns kx of SL launch slots at a time (units
+// The complex64 column stage of length 512: a CTA takes the columns kx of SL launch slots at a time (units
 // of T threads: unit u = column u / SL, slot u % SL). With SL = 4 the columns' Green's tables of the
 // first slot's frequency are staged in shared memory by asynchronous copies issued before the
 // forward transforms; slots of that frequency (consecutive slots share it, problems being
@@ -147,6 +148,61 @@ __global__ void __launch_bounds__(kTileThreads, Cfg<float2>::colMinBlocks) k_col
 template <int LZ, int SL> constexpr size_t cols_pairs_smem() {
   using CF = ColCfg<float2, LZ>;
   return size_t(CF::CC) * CF::PLP * sizeof(cpair) + (SL == 1 ? 0 : size_t(CF::CC / SL) * 3 * LZ * sizeof(float2));
+}
+
+// The complex64 column stage of lengths 32 to 256 with 16 points per thread (fft16.cuh): T lanes of one
+// warp take one column of one slot, every exchange stays inside them, and the CTA meets at no
+// barrier. SL slots of a column sit side by side, so that their warp or CTA finds the column's Green's
+// tables in L1. 168 registers, 3 CTAs per SM (128 spill). 45 problems of 45 x 180 (lz = 128): 17.2 us
+// against 24 us with 8 points per thread; 120^2 x 256 problems (lz = 256) 91 us. At length 512
+// (two 256-point transforms per half-pruned one, the two half warps combining by lane exchanges) the
+// same form took 408 to 444 us for 256 problems of 256^2 with more rounding error or more table loads,
+// against 422 us of the 8-point form above, which stays there.
+constexpr int kCols16Threads = 128;
+template <int LZ> constexpr size_t kCols16Smem = size_t(kCols16Threads / (LZ / 16)) * Fft16<LZ>::LP * sizeof(cpair);
+template <int LZ, int SL>
+__global__ void __launch_bounds__(kCols16Threads, 3) k_cols16(OpP<float2> p) {
+  pdl_begin();
+  using F = Fft16<LZ>;
+  constexpr int T = F::T, COLS = kCols16Threads / T / SL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int u = threadIdx.x / T, t = threadIdx.x % T;
+  cpair *line = reinterpret_cast<cpair *>(smem_raw) + size_t(u) * F::LP;
+  const int kx = blockIdx.x * COLS + u / SL, sl = SL * int(blockIdx.y) + u % SL;
+  int f = -1;
+  if (sl < p.nb && kx < p.lx) {
+    const int b = p.plist ? p.plist[p.s0 + sl] : p.s0 + sl;
+    f = p.fidx[b];
+    if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) f = -1;
+  }
+  const bool live = f >= 0;
+  const int nz = p.nz;
+  cpair *c = reinterpret_cast<cpair *>(p.T) + (live ? (size_t(sl) * p.lx + kx) * nz : 0);
+  const typename F::Base base(t, p.tw);
+  cpair v[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int j = t + m * T;
+    v[m] = m < 8 && live && j < nz ? c[j] : pzero();
+  }
+  F::template run<false, true>(v, line, t, base, WarpSync{});
+  if (live) {
+    const size_t plane = size_t(p.lx) * LZ;
+    const float2 *G = p.Ghat + size_t(f) * 3 * plane + size_t(kx) * LZ;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int k = t + m * T;
+      v[m] = green_product(v[m], __ldg(G + k), __ldg(G + plane + k), __ldg(G + 2 * plane + k));
+    }
+  }
+  F::template run<true, false>(v, line, t, base, WarpSync{});
+  if (live) {
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int j = t + m * T;
+      if (j < nz) c[j] = v[m];
+    }
+  }
 }
 
 template <typename C, int LX, int EPI, int V, int NTT>
@@ -385,8 +441,10 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
     with_plan<LZ>(a.precision, [&]<int V>() {
       using CF = ColCfg<C, LZ>;
       if constexpr (kPairSpectra<C>) {
-        if constexpr (LZ <= 512) {  // 1024 runs as pairs of 512-point transforms
-          cudaError_t e;
+        cudaError_t e = cudaSuccess;
+        // four slots per CTA unless the last group would leave much of its CTAs idle
+        [[maybe_unused]] const bool four = nb % 4 == 0 || nb >= 16;
+        if constexpr (LZ == 512) {
           auto launch = [&]<int SL>() {
             constexpr int COLS = CF::CC / SL;
             const size_t bytes = cols_pairs_smem<LZ, SL>();
@@ -394,11 +452,25 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
             if (e == cudaSuccess)
               launch_pdl(k_cols_pairs<LZ, V, SL>, dim3((a.lx + COLS - 1) / COLS, (nb + SL - 1) / SL), CF::NT, bytes, s, p);
           };
-          // four slots per CTA unless the last group would leave much of its CTAs idle
-          if (nb % 4 == 0 || nb >= 16) launch.template operator()<4>();
+          if (four) launch.template operator()<4>();
           else launch.template operator()<1>();
-          rc = e != cudaSuccess ? cuda_fail("k_cols_pairs smem", e) : check_launch("k_cols_pairs");
-        }
+        } else if constexpr (LZ >= 32 && LZ <= 256) {
+          auto launch = [&]<int SL>() {
+            constexpr int COLS = kCols16Threads / (LZ / 16) / SL;
+            e = allow_smem(k_cols16<LZ, SL>, kCols16Smem<LZ>);
+            if (e == cudaSuccess)
+              launch_pdl(k_cols16<LZ, SL>, dim3((a.lx + COLS - 1) / COLS, (nb + SL - 1) / SL), kCols16Threads,
+                         kCols16Smem<LZ>, s, p);
+          };
+          if (four) launch.template operator()<4>();
+          else launch.template operator()<1>();
+        } else if constexpr (LZ == 16) {
+          const size_t bytes = cols_smem<C, LZ>();
+          e = allow_smem(k_cols<C, LZ, V, kTileThreads>, bytes);
+          if (e == cudaSuccess)
+            launch_pdl(k_cols<C, LZ, V, kTileThreads>, dim3((a.lx + CF::CC - 1) / CF::CC, nb), CF::NT, bytes, s, p);
+        }  // 1024 runs as pairs of 512-point transforms
+        rc = e != cudaSuccess ? cuda_fail("k_cols smem", e) : check_launch("k_cols");
       } else {
         cudaError_t e;
         with_tile<C, LZ>(small, [&]<int NTT>() {
