@@ -181,14 +181,14 @@ template <typename C, int L> struct RegFFT {
   }
 
   // Store a pass's outputs (held in v as produced by butterflies()) at their Stockham positions.
-  template <int R, int NS, int LAY>
-  __host__ __device__ __forceinline__ static void scatter(const C (&v)[8], C *line, int t) {
+  template <int R, int NS, int LAY, typename Line>
+  __host__ __device__ __forceinline__ static void scatter(const C (&v)[8], Line line, int t) {
     constexpr int NB = 8 / R;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
       const int j = t + i * T, k = j % NS, base = (j - k) * R + k;
       if constexpr (kPairs) {  // base mod 8 + (r NS mod 8) < 8 in every plan: pad() splits into the sum
-        C *d = line + pad<LAY>(base);
+        const Line d = line + pad<LAY>(base);
 #pragma unroll
         for (int r = 0; r < R; ++r) d[r * NS + r * NS / 8] = v[i + r * NB];
       } else {
@@ -199,9 +199,10 @@ template <typename C, int L> struct RegFFT {
   }
 
   // Load the next pass's input (natural order) from a shared-memory line.
-  template <int LAY> __host__ __device__ __forceinline__ static void gather(C (&v)[8], const C *line, int t) {
+  template <int LAY, typename Line>
+  __host__ __device__ __forceinline__ static void gather(C (&v)[8], Line line, int t) {
     if constexpr (kPairs) {  // t mod 8 + (m T mod 8) < 8, as in scatter()
-      const C *d = line + pad<LAY>(t);
+      const Line d = line + pad<LAY>(t);
 #pragma unroll
       for (int m = 0; m < 8; ++m) v[m] = d[m * T + m * T / 8];
     } else {
@@ -225,12 +226,20 @@ __host__ __device__ __forceinline__ void pass_powers(const C *w1, C (&wp)[NB][R]
   }
 }
 
-// run() transforms the NLT lines held by the calling thread; sync() must order the shared-memory
+// A line whose elements lie `stride` apart in shared memory.
+template <typename C> struct StridedLine {
+  C *p;
+  int stride;
+  __host__ __device__ __forceinline__ StridedLine operator+(int i) const { return {p + i * stride, stride}; }
+  __host__ __device__ __forceinline__ C &operator[](int i) const { return p[i * stride]; }
+};
+
+// run() transforms the NLT lines held by the calling thread (lines: pointers, or StridedLine); sync() must order the shared-memory
 // accesses of every thread that shares those lines (a barrier over at least the line's T threads).
 // HIN: every line is zero beyond its first half (v[l][4..7] = 0 on entry; they are not read).
 template <int L, int V = 0> struct RegPlan {
-  template <typename C, int NLT, bool INV, bool HIN = false, typename Sync>
-  __host__ __device__ __forceinline__ static void run(C (&v)[NLT][8], C *const (&lines)[NLT], int t,
+  template <typename C, int NLT, bool INV, bool HIN = false, typename Line, typename Sync>
+  __host__ __device__ __forceinline__ static void run(C (&v)[NLT][8], const Line (&lines)[NLT], int t,
                                                       const TwReg<typename TwOf<C>::type, L, V> &tr, Sync &&sync) {
     using F = RegFFT<C, L>;
     using W = typename TwOf<C>::type;
@@ -247,10 +256,10 @@ template <int L, int V = 0> struct RegPlan {
             if constexpr (!LAST) {
               constexpr int LAY = F::kPairs ? 3 : layout_of<L, V>(p);
 #pragma unroll
-              for (int l = 0; l < NLT; ++l) F::template scatter<R, NS, LAY>(v[l], lines[l], t);
+              for (int l = 0; l < NLT; ++l) F::template scatter<R, NS, LAY, Line>(v[l], lines[l], t);
               sync();
 #pragma unroll
-              for (int l = 0; l < NLT; ++l) F::template gather<LAY>(v[l], lines[l], t);
+              for (int l = 0; l < NLT; ++l) F::template gather<LAY, Line>(v[l], lines[l], t);
               sync();
             }
           }(),

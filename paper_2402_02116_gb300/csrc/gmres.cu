@@ -499,6 +499,8 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
   op.active = nullptr;
   op.plist = nullptr;
   op.nb = B;
+  int tables_ready = 0;  // every pass of the solve has the same tables, model and scratch
+  op.tables_ready = &tables_ready;
   if ((rc = pow2_scales(rhs, op.precision, false, B, n, gb.partN, gb.scale, nullptr, nullptr, s))) return rc;
   if (!x_zero) {
     launch_pdl(k_gm_scale_x<C>, all, kRedThreads, 0, s, sp, gb.scale, x, 0);

@@ -26,6 +26,7 @@
 
 #include "fft.cuh"
 #include "krylov.cuh"
+#include "ls3d_slab.cuh"
 #include "mspace.cuh"
 #include "op_tiles.cuh"
 
@@ -45,7 +46,7 @@ template <typename C>
 __global__ void __launch_bounds__(128) k3_stress(int nz, int ny, int nx, typename RealOf<C>::type inv2h,
                                                  const typename RealOf<C>::type *m, Ref6 ref,
                                                  const C *u, const double *in_scale, const int *plist,
-                                                 const int *active, C *sig) {
+                                                 const int *active, C *sig, const typename RealOf<C>::type *dc) {
   pdl_begin();
   using R = typename RealOf<C>::type;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -68,7 +69,8 @@ __global__ void __launch_bounds__(128) k3_stress(int nz, int ny, int nx, typenam
   };
   const C e1 = D(0, 0), e2 = D(1, 1), e3 = D(2, 2);
   const C e4 = cadd(D(1, 2), D(2, 1)), e5 = cadd(D(0, 2), D(2, 0)), e6 = cadd(D(0, 1), D(1, 0));
-  auto dm = [&](int p) { return R(double(m[p * cells + cell]) - ref.v[p]); };
+  // the contrast, rounded beforehand where the caller has it (dc: [5][cells])
+  auto dm = [&](int p) { return dc ? dc[(p - 1) * cells + cell] : R(double(m[p * cells + cell]) - ref.v[p]); };
   const R c11 = dm(1), c13 = dm(2), c33 = dm(3), c55 = dm(4), c66 = dm(5), c12 = c11 - R(2) * c66;
   C *sb = sig + size_t(slot) * 6 * cells + cell;
   sb[0] = cadd(cadd(cscale(e1, c11), cscale(e2, c12)), cscale(e3, c13));
@@ -522,7 +524,7 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
   prof_mark(PROF_OPERATOR, false, s);
   const dim3 cg((a.nx + 127) / 128, a.nz * a.ny, nb);
   if (a.stencil) {
-    launch_pdl(k3_stress<C>, cg, 128, 0, s, a.nz, a.ny, a.nx, inv2h, m, ref, in, a.in_scale, a.plist, a.active, sig);
+    launch_pdl(k3_stress<C>, cg, 128, 0, s, a.nz, a.ny, a.nx, inv2h, m, ref, in, a.in_scale, a.plist, a.active, sig, nullptr);
     if ((rc = check_launch("k3_stress"))) return rc;
     launch_pdl(k3_source<C>, cg, 128, 0, s, a.nz, a.ny, a.nx, a.ly, a.lx, a.nf, inv2h, m, ref, in, a.in_scale, a.omega,
                                     a.fidx, a.plist, a.active, sig, T);
@@ -639,11 +641,142 @@ template <typename C> static int run3_typed(const OpArgs &a, cudaStream_t s) {
   return rc;
 }
 
+// Elements of the spectral scratch the slab path takes: T', the kx-major tables and the FP32 contrasts.
+struct SlabLayout {
+  size_t Rp, tables, contrast, total;  // offsets and total in complex64 elements
+};
+static SlabLayout slab_layout(const OpArgs &a) {
+  SlabLayout l;
+  l.Rp = (size_t(a.nz) * a.ny + 1) / 2 * 2;
+  const size_t cells = size_t(a.nz) * a.ny * a.nx;
+  l.tables = size_t(a.B) * a.lx * 3 * l.Rp;
+  l.contrast = l.tables + size_t(a.nf) * 6 * a.lz * a.ly * a.lx;
+  l.total = l.contrast + ((size_t(a.nf) + 5) * cells + 1) / 2;
+  return l;
+}
+
+template <typename F> static void with_slab_len(int ly, int lz, F &&f) {
+  auto z = [&]<int LY>() {
+    switch (lz) {
+      case 16: f.template operator()<LY, 16>(); break;
+      case 32: f.template operator()<LY, 32>(); break;
+      case 64: f.template operator()<LY, 64>(); break;
+      case 128: f.template operator()<LY, 128>(); break;
+      default: break;
+    }
+  };
+  switch (ly) {
+    case 32: z.template operator()<32>(); break;
+    case 64: z.template operator()<64>(); break;
+    case 128: z.template operator()<128>(); break;
+    default: break;
+  }
+}
+template <typename F> static void with_slab_x(int lx, F &&f) {
+  switch (lx) {
+    case 32: f.template operator()<32>(); break;
+    case 64: f.template operator()<64>(); break;
+    case 128: f.template operator()<128>(); break;
+    case 256: f.template operator()<256>(); break;
+    default: break;
+  }
+}
+
+// The slab path applies to complex64 grids whose FFT lengths it is built for, whose slab fits two CTAs
+// per SM, and whose batch leaves room for the kx-major tables in the spectral scratch (the scratch holds
+// [B][3][nz][ly][lx] values, T' takes ny / ly of it: about eight problems per frequency are enough).
+static bool slab_fits(const OpArgs &a) {
+  if (a.precision != DBI_C64 || a.lx < 32 || a.lx > 256) return false;
+  size_t smem = 0;
+  with_slab_len(a.ly, a.lz, [&]<int LY, int LZ>() { smem = slab_smem<LY, LZ>((a.nz + 1) / 2 * 2); });
+  if (smem == 0 || smem > 113 * 1024) return false;
+  return slab_layout(a).total <= size_t(a.B) * 3 * a.nz * a.ly * a.lx &&
+         size_t(a.nf) * 6 * a.lz <= 65535 && size_t(a.lx) * a.B <= size_t(INT32_MAX);
+}
+
+static int run3_slab(const OpArgs &a, cudaStream_t s) {
+  const int nb = a.plist ? a.nb : a.B;
+  if (nb <= 0) return DBI_OK;
+  const SlabLayout l = slab_layout(a);
+  const size_t cells = size_t(a.nz) * a.ny * a.nx;
+  float2 *T = static_cast<float2 *>(a.T), *sig = static_cast<float2 *>(a.T2);
+  const float *m = static_cast<const float *>(a.m);
+  SlabP p{};
+  p.nb = nb; p.nz = a.nz; p.ny = a.ny; p.nx = a.nx; p.lx = a.lx; p.nf = a.nf;
+  p.nzp = (a.nz + 1) / 2 * 2; p.rows = a.nz * a.ny; p.Rp = l.Rp;
+  p.inv2h = float(1.0 / (2.0 * a.h));
+  p.omega = a.omega; p.fidx = a.fidx; p.plist = a.plist; p.active = a.active;
+  p.u = static_cast<const float2 *>(a.in); p.sig = sig; p.ident = static_cast<const float2 *>(a.ident);
+  p.in_scale = a.in_scale; p.out_scale = a.out_scale;
+  p.out = static_cast<float2 *>(a.out); p.T = T;
+  cpair *G = reinterpret_cast<cpair *>(T + l.tables);
+  float *wr = reinterpret_cast<float *>(T + l.contrast), *dc = wr + size_t(a.nf) * cells;
+  p.G = G; p.wr = wr; p.dc = dc;
+  p.tw = static_cast<const float2 *>(a.tw);
+  int rc;
+  prof_mark(PROF_OPERATOR, false, s);
+  if (!a.tables_ready || !*a.tables_ready) {  // once per solve
+    launch_pdl(k3_tables_kx, dim3((a.lx + 31) / 32, (a.ly + 31) / 32, a.nf * 6 * a.lz), 256, 0, s, a.lz, a.ly, a.lx,
+               static_cast<const float2 *>(a.Ghat), G);
+    if ((rc = check_launch("k3_tables_kx"))) return rc;
+    if (a.stencil) {
+      launch_pdl(k3_contrast, unsigned((cells + 127) / 128), 128, 0, s, cells, a.nf, a.omega, m, a.ref[0], a.ref[1],
+                 a.ref[2], a.ref[3], a.ref[4], a.ref[5], wr, dc);
+      if ((rc = check_launch("k3_contrast"))) return rc;
+    }
+    if (a.tables_ready) *a.tables_ready = 1;
+  }
+  if (a.stencil) {
+    Ref6 ref;
+    for (int i = 0; i < 6; ++i) ref.v[i] = a.ref[i];
+    launch_pdl(k3_stress<float2>, dim3((a.nx + 127) / 128, a.nz * a.ny, nb), 128, 0, s, a.nz, a.ny, a.nx, p.inv2h, m,
+               ref, p.u, a.in_scale, a.plist, a.active, sig, dc);
+    if ((rc = check_launch("k3_stress"))) return rc;
+  }
+  rc = DBI_ERR_UNSUPPORTED;
+  with_slab_x(a.lx, [&]<int LX>() {
+    using F = Fft16<LX>;
+    constexpr int LINES = kSlabXThreads / F::T;
+    const size_t bytes = size_t(LINES) * F::LP * sizeof(cpair);
+    const dim3 grid((p.rows + 2 * LINES - 1) / (2 * LINES), 3, nb);
+    auto kern = a.stencil ? k3_src_x<LX, true> : k3_src_x<LX, false>;
+    cudaError_t e = allow_smem(kern, bytes);
+    if (e == cudaSuccess) launch_pdl(kern, grid, kSlabXThreads, bytes, s, p);
+    rc = e != cudaSuccess ? cuda_fail("k3_src_x smem", e) : check_launch("k3_src_x");
+  });
+  if (rc) return rc;
+  prof_mark(PROF_COLS, false, s);
+  rc = DBI_ERR_UNSUPPORTED;
+  with_slab_len(a.ly, a.lz, [&]<int LY, int LZ>() {
+    const size_t bytes = slab_smem<LY, LZ>(p.nzp);
+    p.spare = slab_rows<LZ>(p.nzp);
+    p.ahead = 2 * 152 / nb + 1;  // two CTAs per SM are in flight
+    cudaError_t e = allow_smem(k3_yz<LY, LZ>, bytes);
+    if (e == cudaSuccess) launch_pdl(k3_yz<LY, LZ>, unsigned(a.lx) * unsigned(nb), kSlabThreads, bytes, s, p);
+    rc = e != cudaSuccess ? cuda_fail("k3_yz smem", e) : check_launch("k3_yz");
+  });
+  prof_mark(PROF_COLS, true, s);
+  if (rc) return rc;
+  rc = DBI_ERR_UNSUPPORTED;
+  with_slab_x(a.lx, [&]<int LX>() {
+    using F = Fft16<LX>;
+    constexpr int LINES = kSlabXThreads / F::T;
+    const size_t bytes = size_t(LINES) * F::LP * sizeof(cpair);
+    const dim3 grid((p.rows + 2 * LINES - 1) / (2 * LINES), 3, nb);
+    cudaError_t e = allow_smem(k3_x_inv<LX>, bytes);
+    if (e == cudaSuccess) launch_pdl(k3_x_inv<LX>, grid, kSlabXThreads, bytes, s, p);
+    rc = e != cudaSuccess ? cuda_fail("k3_x_inv smem", e) : check_launch("k3_x_inv");
+  });
+  prof_mark(PROF_OPERATOR, true, s);
+  return rc;
+}
+
 int run_operator_3d(const OpArgs &a, cudaStream_t s) {
   if (a.epi != 0) {
     set_error("the 3D operator has no fused inner products (use GMRES)");
     return DBI_ERR_UNSUPPORTED;
   }
+  if (slab_fits(a)) return run3_slab(a, s);
   return a.precision == DBI_C64 ? run3_typed<float2>(a, s) : run3_typed<double2>(a, s);
 }
 

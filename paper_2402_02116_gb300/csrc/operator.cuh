@@ -64,6 +64,9 @@ struct OpArgs {
   // [B][3][nz][ly][lx] and T2 the stress [B][6][nz][ny][nx]; Ghat [nf][6][lz][ly][lx].
   int ny, ly;
   void *T2;
+  // Host flag of a run of passes with the same tables, model and scratch (a solve): 0 until the first
+  // pass has made its re-laid copies of them in T (ls3d_slab.cuh). NULL: every pass makes its own.
+  int *tables_ready;
 };
 
 // Partials per problem written by the operator kernels (one per CTA row block): the single-grid
