@@ -14,6 +14,7 @@
 #include "op_split3.cuh"
 #include "op_tiles.cuh"
 #include "operator.cuh"
+#include "rows_stream.cuh"
 #include "tune.cuh"
 
 namespace dbi {
@@ -91,6 +92,21 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowFwdMinBl
   extern __shared__ __align__(16) unsigned char smem_raw[];
   rows_forward_tile<C, LX, STENCIL, V, NTT>(BatchTile<C>{p, b, int(blockIdx.y), f}, blockIdx.x,
                                        reinterpret_cast<C *>(smem_raw));
+}
+
+// The forward row stage of complex64 lengths 128 to 512 in chunks of `chunk` rows (rows_stream.cuh).
+#ifndef DBI_STREAM_THREADS
+#define DBI_STREAM_THREADS 768
+#endif
+template <int LX, int V>
+__global__ void __launch_bounds__(LX / 2, DBI_STREAM_THREADS / (LX / 2)) k_rows_stream(OpP<float2> p, int chunk) {
+  pdl_begin();
+  const int b = problem_of(p), f = p.fidx[b];
+  if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int zb = blockIdx.x * chunk;
+  rows_stream<LX, V>(BatchTile<float2>{p, b, int(blockIdx.y), f}, zb, min(zb + chunk, p.nz),
+                     reinterpret_cast<float4 *>(smem_raw));
 }
 
 template <typename C, int LZ, int V, int NTT>
@@ -405,6 +421,20 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   if (!split_r) dispatch_len(a.lx, [&]<int LX>() {
     with_plan<LX>(a.precision, [&]<int V>() {
       cudaError_t e;
+      if constexpr (kPairSpectra<C> && LX >= 128 && LX <= 512) {
+        if (stencil) {
+          // rows per CTA: 32 while that leaves four waves of CTAs, at least 4
+          int chunk = 32;
+          const int wave = DBI_STREAM_THREADS / (LX / 2) * 152;
+          while (chunk > 4 && long((a.nz + chunk - 1) / chunk) * nb < 4L * wave) chunk /= 2;
+          const size_t bytes = StreamCfg<LX>::smem;
+          e = allow_smem(k_rows_stream<LX, V>, bytes);
+          if (e == cudaSuccess)
+            launch_pdl(k_rows_stream<LX, V>, dim3((a.nz + chunk - 1) / chunk, nb), LX / 2, bytes, s, p, chunk);
+          rc = e != cudaSuccess ? cuda_fail("k_rows_stream smem", e) : check_launch("k_rows_stream");
+          return;
+        }
+      }
       with_tile<C, LX>(small, [&]<int NTT>() {
         using RC = RowCfg<C, LX, NTT>;
         const size_t bytes = rows_forward_smem<C, LX, NTT>(a.nx, stencil);
