@@ -204,8 +204,8 @@ constexpr int kRedThreads = 256;  // threads per reduction block
 constexpr int kRedSlots = 4;      // doubles per block partial
 constexpr int kMaxParts = 512;    // partials per problem at most (operator kernels: one per row block)
 // Blocks per problem of a vector pass over B problems of n elements: 8 accesses per thread (16 bytes
-// each) where that gives enough blocks for every SM, else as many blocks as have work up to about
-// four per SM. (64 blocks whatever the size left 45 problems of 45 x 180 cells with one pair of points
+// each) where that gives enough blocks for every SM, else as many blocks as have work up to one wave
+// of four per SM (a second wave of a few blocks would double the time). (64 blocks whatever the size left 45 problems of 45 x 180 cells with one pair of points
 // per thread under the cost of reading the problem's scalars.)
 int red_blocks(size_t n, int B, int precision);
 

@@ -15,6 +15,7 @@
 #include "op_tiles.cuh"
 #include "operator.cuh"
 #include "rows_stream.cuh"
+#include "small64.cuh"
 #include "tune.cuh"
 
 namespace dbi {
@@ -232,6 +233,32 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowInvMinBl
   if constexpr (EPI != 0) finish_tile<EPI>(p.fin, b, a.part(), gridDim.x);
 }
 
+// The stages of small complex128 batches at lengths up to 128 (small64.cuh).
+template <int LX, bool STENCIL, int V> __global__ void __launch_bounds__(32) k_rows_forward_small(OpP<double2> p) {
+  pdl_begin();
+  const int b = problem_of(p), f = p.fidx[b];
+  if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  small64_rows_forward<LX, STENCIL, V>(BatchTile<double2>{p, b, int(blockIdx.y), f}, blockIdx.x,
+                                       reinterpret_cast<double2 *>(smem_raw));
+}
+template <int LZ, int V> __global__ void __launch_bounds__(32) k_cols_small(OpP<double2> p) {
+  pdl_begin();
+  const int b = problem_of(p), f = p.fidx[b];
+  if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  small64_cols<LZ, V>(BatchTile<double2>{p, b, int(blockIdx.y), f}, blockIdx.x, reinterpret_cast<double2 *>(smem_raw));
+}
+template <int LX, int EPI, int V> __global__ void __launch_bounds__(32) k_rows_inverse_small(OpP<double2> p) {
+  pdl_begin();
+  const int b = problem_of(p), f = p.fidx[b];
+  if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const BatchTile<double2> a{p, b, int(blockIdx.y), f};
+  small64_rows_inverse<LX, EPI, V>(a, blockIdx.x, reinterpret_cast<double2 *>(smem_raw));
+  if constexpr (EPI != 0) finish_tile<EPI>(p.fin, b, a.part(), gridDim.x);
+}
+
 // Stages of the L = 1024 complex64 operator as pairs of 512-point transforms (op_split.cuh).
 __global__ void __launch_bounds__(kSrcThreads) k_source_split(OpP<float2> p) {
   pdl_begin();
@@ -332,15 +359,15 @@ __global__ void __launch_bounds__(kS3Threads, 2) k_rows_inverse_s3(OpP<float2> p
 }
 
 // Threads per CTA of the ordinary stages: 256, or for complex128 batches too small to give every SM a
-// 256-thread tile, as few as hold whole lines and warps. FP64 runs at two lanes a cycle and SM, so
-// what counts there is the number of SMs: a 32 x 32 grid of one problem was one row tile and two
-// column tiles (68, 40 and 24 us for the three stages).
+// 256-thread tile, as few as hold whole lines and warps (beyond length 128; up to it the kernels of
+// small64.cuh run). FP64 runs at two lanes a cycle and SM, so what counts there is the number of SMs: a
+// 32 x 32 grid of one problem was one row tile and two column tiles (68, 40 and 24 us for the stages).
 template <int L> constexpr int kSmallThreads = L / 8 > 32 ? L / 8 : 32;
 inline bool small_tiles(int B, int nz, int lx, int precision) {
   return precision == DBI_C128 && lx <= 1024 && size_t(B) * ((size_t(nz) * lx + 2047) / 2048) < 2 * 152;
 }
 template <typename C, int L, typename F> inline void with_tile(bool small, F &&f) {
-  if constexpr (sizeof(C) == sizeof(double2)) {
+  if constexpr (sizeof(C) == sizeof(double2) && L > 128) {
     if (small) {
       f.template operator()<kSmallThreads<L>>();
       return;
@@ -435,6 +462,17 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           return;
         }
       }
+      if constexpr (sizeof(C) == sizeof(double2) && LX <= 128) {
+        if (small) {
+          const size_t bytes = small64_forward_smem<LX>(a.nx, stencil);
+          constexpr int U = Small64<LX>::UNITS;
+          auto kern = stencil ? k_rows_forward_small<LX, true, V> : k_rows_forward_small<LX, false, V>;
+          e = allow_smem(kern, bytes);
+          if (e == cudaSuccess) launch_pdl(kern, dim3((a.nz + U - 1) / U, nb), 32, bytes, s, p);
+          rc = e != cudaSuccess ? cuda_fail("k_rows_forward_small smem", e) : check_launch("k_rows_forward_small");
+          return;
+        }
+      }
       with_tile<C, LX>(small, [&]<int NTT>() {
         using RC = RowCfg<C, LX, NTT>;
         const size_t bytes = rows_forward_smem<C, LX, NTT>(a.nx, stencil);
@@ -502,7 +540,15 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
         }  // 1024 runs as pairs of 512-point transforms
         rc = e != cudaSuccess ? cuda_fail("k_cols smem", e) : check_launch("k_cols");
       } else {
-        cudaError_t e;
+        cudaError_t e = cudaSuccess;
+        if constexpr (LZ <= 128) {
+          if (small) {
+            constexpr int U = Small64<LZ>::UNITS;
+            launch_pdl(k_cols_small<LZ, V>, dim3((a.lx + U - 1) / U, nb), 32, Small64<LZ>::lines, s, p);
+            rc = check_launch("k_cols_small");
+            return;
+          }
+        }
         with_tile<C, LZ>(small, [&]<int NTT>() {
           using CN = ColCfg<C, LZ, NTT>;
           const size_t bytes = cols_smem<C, LZ, NTT>();
@@ -537,6 +583,16 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   if (!split_r) dispatch_len(a.lx, [&]<int LX>() {
     with_plan<LX>(a.precision, [&]<int V>() {
       cudaError_t e;
+      if constexpr (sizeof(C) == sizeof(double2) && LX <= 128) {
+        if (small) {
+          constexpr int U = Small64<LX>::UNITS;
+          auto kern = a.epi == 1 ? k_rows_inverse_small<LX, 1, V> : a.epi == 2 ? k_rows_inverse_small<LX, 2, V>
+                                                                               : k_rows_inverse_small<LX, 0, V>;
+          launch_pdl(kern, dim3((a.nz + U - 1) / U, nb), 32, Small64<LX>::lines, s, p);
+          rc = check_launch("k_rows_inverse_small");
+          return;
+        }
+      }
       with_tile<C, LX>(small, [&]<int NTT>() {
         using RC = RowCfg<C, LX, NTT>;
         const size_t bytes = rows_inverse_smem<C, LX, NTT>();
@@ -574,7 +630,10 @@ int operator_parts(int B, int nz, int lx, int precision) {
   if (split_rows(lx, precision)) return (nz + kSplitRows - 1) / kSplitRows;
   if (small_tiles(B, nz, lx, precision)) {
     int rows = 1;
-    dispatch_len(lx, [&]<int LX>() { rows = RowCfg<double2, LX, kSmallThreads<LX>>::ROWS; });
+    dispatch_len(lx, [&]<int LX>() {
+      if constexpr (LX <= 128) rows = Small64<LX>::UNITS;
+      else rows = RowCfg<double2, LX, kSmallThreads<LX>>::ROWS;
+    });
     return (nz + rows - 1) / rows;
   }
   return operator_parts_k(nz, lx, precision);

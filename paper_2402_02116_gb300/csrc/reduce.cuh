@@ -40,13 +40,11 @@ template <int NS, typename T> __device__ __forceinline__ void block_sum_store(T 
 __device__ __forceinline__ bool last_cta(int *arrived, int n) {
   __shared__ int last;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(arrived, 1) == n - 1;
-    if (last) {
-      *arrived = 0;
-      __threadfence();
-    }
+  if (threadIdx.x == 0) {  // release this CTA's writes (ordered before by the barrier), acquire the others'
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(__cvta_generic_to_global(arrived)) : "memory");
+    last = old == n - 1;
+    if (last) *arrived = 0;
   }
   __syncthreads();
   return last != 0;
