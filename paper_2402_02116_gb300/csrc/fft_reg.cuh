@@ -109,8 +109,10 @@ template <> struct TwOf<cpair> { using type = float2; };
 template <typename C, int L, int V = 0> struct TwReg {
   static constexpr int NW = PlanInfo<L, V>::nw;
   C w[NW];
-  // Base twiddles W_{Ns R}^{j mod Ns} of thread t's butterflies j = t + i L/8 in every pass > 0.
-  __host__ __device__ __forceinline__ TwReg(int t, const C *__restrict__ tw) {
+  // Base twiddles W_{Ns R}^{j mod Ns} of thread t's butterflies j = t + i L/8 in every pass > 0; the last
+  // pass is run as thread `tl` (RegPlan::run_regrouped).
+  __host__ __device__ __forceinline__ TwReg(int t, const C *__restrict__ tw) : TwReg(t, t, tw) {}
+  __host__ __device__ __forceinline__ TwReg(int t0, int tl, const C *__restrict__ tw) {
     using P = PlanInfo<L, V>;
     constexpr int TWS = kTwiddleN / L, T = L / 8;
     [&]<int... p>(std::integer_sequence<int, p...>) {
@@ -119,7 +121,7 @@ template <typename C, int L, int V = 0> struct TwReg {
             constexpr int q = p + 1, R = P::radix(q), NS = P::ns(q), NB = 8 / R;
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
-              const int k = (t + i * T) % NS;
+              const int k = ((q == P::np - 1 ? tl : t0) + i * T) % NS;
               w[P::woff(q) + i] = tw[k * (L / (NS * R)) * TWS];
             }
           }(),
@@ -261,6 +263,43 @@ template <int L, int V = 0> struct RegPlan {
 #pragma unroll
               for (int l = 0; l < NLT; ++l) F::template gather<LAY, Line>(v[l], lines[l], t);
               sync();
+            }
+          }(),
+          ...);
+    }(std::make_integer_sequence<int, P::np>{});
+  }
+
+  // As run(), for a group of lines whose threads change places at one exchange: up to exchange X (0 or the
+  // last) thread (lines, t) holds its points, after it thread (lines2, t2); `all` is a barrier over
+  // every thread of the group. A forward transform so ends, and an inverse one begins, with each
+  // point in the thread that writes or reads it in global memory. After the last exchange there is no
+  // barrier: the caller orders the next use of the lines.
+  template <typename C, int NLT, bool INV, int X, bool HIN = false, typename Sync, typename All>
+  __host__ __device__ __forceinline__ static void run_regrouped(C (&v)[NLT][8], C *const (&lines)[NLT], int t,
+                                                                C *const (&lines2)[NLT], int t2,
+                                                                const TwReg<typename TwOf<C>::type, L, V> &tr,
+                                                                Sync &&sync, All &&all) {
+    using F = RegFFT<C, L>;
+    using W = typename TwOf<C>::type;
+    using P = PlanInfo<L, V>;
+    static_assert(F::kPairs && (X == 0 || X == P::np - 2), "pairs; the first or the last exchange");
+    [&]<int... p>(std::integer_sequence<int, p...>) {
+      (
+          [&] {
+            constexpr int R = P::radix(p), NS = P::ns(p), NB = 8 / R;
+            W wp[NB][R];
+            if constexpr (NS > 1) pass_powers<W, R, INV, NB>(tr.w + P::woff(p), wp);
+#pragma unroll
+            for (int l = 0; l < NLT; ++l) F::template butterflies<R, NS, INV, HIN && p == 0>(v[l], wp);
+            if constexpr (p < P::np - 1) {
+#pragma unroll
+              for (int l = 0; l < NLT; ++l)
+                F::template scatter<R, NS, 3, C *>(v[l], p <= X ? lines[l] : lines2[l], p <= X ? t : t2);
+              if constexpr (p == X) all();
+              else sync();
+#pragma unroll
+              for (int l = 0; l < NLT; ++l) F::template gather<3, C *>(v[l], p < X ? lines[l] : lines2[l], p < X ? t : t2);
+              if constexpr (p < P::np - 2) sync();
             }
           }(),
           ...);

@@ -26,22 +26,13 @@ constexpr int kSplitRows = kTileThreads / kSplitT;    // rows (or columns) per 2
 constexpr int kSplitLP = RegFFT<cpair, kSplitM>::LP;  // padded line of pairs in shared memory
 static_assert(kSplitL == 1024, "the per-point twiddles come from the contiguous W_1024 table");
 
-// Transposition tile of the row stages, [rows][KP] pairs, the even kx of a row before its odd ones
-// (position q M + k holds kx = 2k + q, as the transforms of the two parities leave them): a quarter
-// warp's 16-byte accesses hit 8 distinct bank slots along a row and down the tile (4 rows x 2
-// positions, KP = 2 mod 8).
-constexpr int kSplitKP = kSplitL + 2;
-__device__ __forceinline__ int split_kx(int j) { return 2 * (j & (kSplitM - 1)) + (j >= kSplitM); }
-
-// Shared memory (bytes): the row stages run the two parities one after the other through one line
-// of pairs per row, whose memory the transposition tile reuses; the column stage runs both lines of a
-// column at once (the twiddle powers formed once, half the barriers).
-__host__ __device__ constexpr size_t split_lines_smem() { return size_t(kSplitRows) * kSplitLP * sizeof(cpair); }
-__host__ __device__ constexpr size_t split_cols_lines_smem() { return 2 * split_lines_smem(); }
-__host__ __device__ constexpr size_t split_tile_smem() { return size_t(kSplitRows) * kSplitKP * sizeof(cpair); }
-__host__ __device__ constexpr size_t split_rows_smem() {
-  return split_lines_smem() > split_tile_smem() ? split_lines_smem() : split_tile_smem();
+// Shared memory (bytes): both lines of pairs of a column or row (the twiddle powers formed once, half
+// the barriers); those of the rows at the pitch of the regrouped exchanges.
+constexpr int kSplitRP = row_pitch<kSplitM, kSplitRows>;
+__host__ __device__ constexpr size_t split_cols_lines_smem() {
+  return size_t(2) * kSplitRows * kSplitLP * sizeof(cpair);
 }
+__host__ __device__ constexpr size_t split_rows_smem() { return size_t(2) * kSplitRows * kSplitRP * sizeof(cpair); }
 __host__ __device__ constexpr size_t split_cols_smem() { return split_cols_lines_smem(); }
 __host__ __device__ constexpr size_t split_rows_inverse_smem() { return split_rows_smem(); }
 
@@ -163,17 +154,8 @@ __device__ __forceinline__ void source_rows(const A &a, int chunk, float2 *smem,
   if (j <= ze) step.template operator()<1>(j);
 }
 
-// The two parities, each an M-point transform of pairs held as 8 points per thread: v[q][m] is
+// The two parities are each an M-point transform of pairs held as 8 points per thread: v[q][m] is
 // point t + m T of parity q.
-// One parity at a time through one line (the row stages).
-template <bool INV, typename Sync>
-__device__ __forceinline__ void split_fft(cpair (&v)[2][8], cpair *line, int t, const TwReg<float2, kSplitM, 0> &tr,
-                                          Sync &&sync) {
-  cpair *const lines[1] = {line};
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-    RegPlan<kSplitM, 0>::template run<cpair, 1, INV>(reinterpret_cast<cpair(&)[1][8]>(v[q]), lines, t, tr, sync);
-}
 
 // Shared memory of the column stage with the column's Green's tables staged: the lines, then
 // Ghat(:, kx) of the three tables [3][L].
@@ -249,19 +231,20 @@ __device__ __forceinline__ void cols_tile_split(const A &a, int tile, float2 *sm
 }
 
 // Four rows z0 .. z0 + 3: the source rows (from the stencil kernel, or the raw input times its
-// scale), the forward transform along x (even and odd kx), transposed through shared memory into
-// the column-major spectra T[kx][z] in runs of four rows (64 bytes).
+// scale), the forward transform along x (even and odd kx), stored by the threads of the regrouped last
+// pass into the column-major spectra T[kx][z] in runs of four rows (64 bytes).
 template <typename A>
 __device__ __forceinline__ void rows_forward_tile_split(const A &a, int tile, float2 *smem, const float2 *src,
                                                         float scale) {
   using C = float2;
-  constexpr int T = kSplitT, ROWS = kSplitRows, KP = kSplitKP;
+  constexpr int T = kSplitT, ROWS = kSplitRows;
   const int z0 = tile * ROWS;
   const int nz = a.nz(), nx = a.nx();
   const int rr = threadIdx.x / T, t = threadIdx.x - rr * T, z = z0 + rr;
+  const int r = threadIdx.x % ROWS, tq = threadIdx.x / ROWS;
   const size_t plane = size_t(nz) * nx;
   const C *tw = a.tw();
-  const TwReg<C, kSplitM, 0> tr(t, tw);
+  const TwReg<C, kSplitM, 0> tr(t, tq, tw);
   cpair v[2][8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
@@ -273,34 +256,27 @@ __device__ __forceinline__ void rows_forward_tile_split(const A &a, int tile, fl
     v[1][m] = hmul(v[0][m], __ldg(tw + kTw1024 + x));  // W_L^x
   }
   cpair *ps = reinterpret_cast<cpair *>(smem);
-  split_fft<false>(v, ps + size_t(rr) * kSplitLP, t, tr, RowSync<T>{1 + rr});
-  // transpose through tile[rr][kx] (the lines' memory is free now)
-  __syncthreads();
-  cpair *row = ps + size_t(rr) * KP;
-#pragma unroll
-  for (int m = 0; m < 8; ++m) {  // kx = 2k and 2k + 1
-    row[t + m * T] = v[0][m];
-    row[kSplitM + t + m * T] = v[1][m];
-  }
-  __syncthreads();
-  cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0;
-  const int r = threadIdx.x % ROWS;
+  cpair *const lines[2] = {ps + size_t(rr) * kSplitRP, ps + size_t(ROWS + rr) * kSplitRP};
+  cpair *const lines2[2] = {ps + size_t(r) * kSplitRP, ps + size_t(ROWS + r) * kSplitRP};
+  RegPlan<kSplitM, 0>::template run_regrouped<cpair, 2, false, 1>(v, lines, t, lines2, tq, tr, RowSync<T>{1 + rr},
+                                                                  CtaSync{});
   if (z0 + r < nz) {
+    cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0 + r;
 #pragma unroll
-    for (int i = 0; i < kSplitL * ROWS / kTileThreads; ++i) {
-      const int j = threadIdx.x / ROWS + i * (kTileThreads / ROWS);
-      Tp[size_t(split_kx(j)) * nz + r] = ps[size_t(r) * KP + j];
+    for (int m = 0; m < 8; ++m) {  // kx = 2k and 2k + 1
+      Tp[size_t(2 * (tq + m * T)) * nz] = v[0][m];
+      Tp[size_t(2 * (tq + m * T) + 1) * nz] = v[1][m];
     }
   }
 }
 
-// Four rows: the spectra T[kx][z0 .. z0 + 3] through a transposition tile, the inverse
+// Four rows: the spectra T[kx][z0 .. z0 + 3], the inverse
 // transform along x (even and odd kx), y_x = even + W_L^{-x} odd for x < nx, then the epilogue of
 // rows_inverse_tile: out = ident - scale * y (or the scaled y) with the fused inner products.
 template <int EPI, typename A>
 __device__ __forceinline__ void rows_inverse_tile_split(const A &a, int tile, float2 *smem) {
   using C = float2;
-  constexpr int T = kSplitT, ROWS = kSplitRows, KP = kSplitKP;
+  constexpr int T = kSplitT, ROWS = kSplitRows;
   const int z0 = tile * ROWS;
   const int nz = a.nz(), nx = a.nx();
   const int rr = threadIdx.x / T, t = threadIdx.x - rr * T, z = z0 + rr;
@@ -308,30 +284,23 @@ __device__ __forceinline__ void rows_inverse_tile_split(const A &a, int tile, fl
   const TwReg<C, kSplitM, 0> tr(t, tw);
   cpair v[2][8];
   cpair *ps = reinterpret_cast<cpair *>(smem);
-  // the spectra into tile[r][kx] by asynchronous copies (zeros for rows beyond nz), all in flight at
-  // once and without register staging
+  // thread (r, tq) takes its points of row z0 + r straight into registers (zeros for rows beyond nz)
+  const int r = threadIdx.x % ROWS, tq = threadIdx.x / ROWS;
   {
-    const int r = threadIdx.x % ROWS;  // the same row for all of a thread's copies
     const bool in = z0 + r < nz;
     const cpair *T0 = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
 #pragma unroll
-    for (int i = 0; i < kSplitL * ROWS / kTileThreads; ++i) {
-      const int j = threadIdx.x / ROWS + i * (kTileThreads / ROWS);
-      cp_async16z(ps + size_t(r) * KP + j, T0 + size_t(split_kx(j)) * nz, in);
-    }
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  {
-    const cpair *row = ps + size_t(rr) * KP;
-#pragma unroll
     for (int m = 0; m < 8; ++m) {  // kx = 2k and 2k + 1
-      v[0][m] = row[t + m * T];
-      v[1][m] = row[kSplitM + t + m * T];
+      v[0][m] = in ? load_spectrum(T0 + size_t(2 * (tq + m * T)) * nz) : pzero();
+      v[1][m] = in ? load_spectrum(T0 + size_t(2 * (tq + m * T) + 1) * nz) : pzero();
     }
   }
-  __syncthreads();  // the lines reuse the tile's memory
-  split_fft<true>(v, ps + size_t(rr) * kSplitLP, t, tr, RowSync<T>{1 + rr});
+  prefetch_rows<kTileThreads>(a, a.ident(), z0, ROWS, sizeof(C));
+  if constexpr (EPI == 1) prefetch_rows<kTileThreads>(a, a.krhat(), z0, ROWS, sizeof(C));
+  cpair *const lines[2] = {ps + size_t(r) * kSplitRP, ps + size_t(ROWS + r) * kSplitRP};
+  cpair *const lines2[2] = {ps + size_t(rr) * kSplitRP, ps + size_t(ROWS + rr) * kSplitRP};
+  RegPlan<kSplitM, 0>::template run_regrouped<cpair, 2, true, 0>(v, lines, tq, lines2, t, tr, RowSync<T>{1 + rr},
+                                                                 CtaSync{});
   C y[2][8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {

@@ -20,23 +20,16 @@ constexpr int kS3L = 768, kS3M = 256;
 constexpr int kS3T = kS3M / 8;                    // threads per line: one warp
 constexpr int kS3Units = 4;                       // rows or columns per CTA
 constexpr int kS3Threads = kS3Units * 3 * kS3T;   // 384: a warp per (unit, residue)
-constexpr int kS3LP = RegFFT<cpair, kS3M>::LP;    // padded line of pairs in shared memory
-// Transposition tile row of the row stages. 16-byte accesses are served a quarter warp at a time:
-// with KP = 2 mod 8 the column-major accesses (four rows x two kx per quarter warp) hit 8 distinct
-// bank slots, and so do the residue-strided accesses 3k + q of a warp (3 is odd).
-constexpr int kS3KP = kS3L + 2;
+// Padded line of pairs in shared memory; at 2 mod 8 the lines of one residue of four rows (6 mod 8
+// apart) hit distinct bank slots with two consecutive points each.
+constexpr int kS3LP = row_pitch<kS3M, kS3Units>;
 constexpr int kS3UnitThreads = 3 * kS3T;          // 96 threads per row or column
 constexpr int kS3Tw = kTwiddleN / kS3L;           // W_L^j = tw[j * kS3Tw]
 constexpr int kS3Third = kTwiddleN / 3;           // W_3 = tw[kS3Third]
 
-// Shared memory (bytes): a line of pairs per warp; the row stages' transposition
-// tile [rr][KP] reuses that memory, and so do the residues' inverse
-// transforms that the combine step reads. Every stage takes the same amount.
-__host__ __device__ constexpr size_t s3_lines_smem() { return size_t(kS3Units) * 3 * kS3LP * sizeof(cpair); }
-__host__ __device__ constexpr size_t s3_tile_smem() { return size_t(kS3Units) * kS3KP * sizeof(cpair); }
-__host__ __device__ constexpr size_t s3_smem() {
-  return s3_lines_smem() > s3_tile_smem() ? s3_lines_smem() : s3_tile_smem();
-}
+// Shared memory (bytes): a line of pairs per warp; the residues' inverse transforms that the combine
+// step reads reuse it. Every stage takes the same amount.
+__host__ __device__ constexpr size_t s3_smem() { return size_t(kS3Units) * 3 * kS3LP * sizeof(cpair); }
 
 // Warp barrier: a line's exchanges stay inside its warp.
 struct WarpSync {
@@ -131,8 +124,8 @@ __device__ __forceinline__ void cols_tile_s3(const A &a, int tile, float2 *smem)
 }
 
 // Rows z0 .. z0 + 3: warp (row, q) folds the row (the source rows from the stencil kernel, or the
-// raw input times its scale) and transforms it (the spectra at kx = 3k + q); the pairs go through the
-// transposition tile into the column-major spectra T[kx][z] in runs of four rows.
+// raw input times its scale) and transforms it (the spectra at kx = 3k + q); the threads of the
+// regrouped last pass store the pairs into the column-major spectra T[kx][z] in runs of four rows.
 template <typename A>
 __device__ __forceinline__ void rows_forward_tile_s3(const A &a, int tile, float2 *smem, const float2 *src,
                                                      float scale) {
@@ -143,67 +136,49 @@ __device__ __forceinline__ void rows_forward_tile_s3(const A &a, int tile, float
   const int nz = a.nz(), nx = a.nx();
   const size_t plane = size_t(nz) * nx;
   const C *tw = a.tw();
-  const TwReg<C, kS3M, 0> tr(t, tw);
+  // thread (r, tq, qs) of the stores: row z0 + r, residue qs
+  const int r = threadIdx.x % kS3Units, tq = threadIdx.x / kS3Units % kS3T, qs = threadIdx.x / (kS3Units * kS3T);
+  const TwReg<C, kS3M, 0> tr(t, tq, tw);
   const int n = z < nz ? nx : 0;
   const C *row = src + size_t(z < nz ? z : 0) * nx;
   cpair *ps = reinterpret_cast<cpair *>(smem);
   cpair v[1][8];
   s3_fold(v[0], t, q, n, tw,
           [&](int j) { return mkpair(cscale(__ldg(row + j), scale), cscale(__ldg(row + plane + j), scale)); });
-  cpair *const lines[1] = {ps + size_t(w) * kS3LP};
-  RegPlan<kS3M, 0>::template run<cpair, 1, false>(v, lines, t, tr, WarpSync{});
-  __syncthreads();  // every warp is done with its line: the tile reuses their memory
-  cpair *trow = ps + size_t(rr) * kS3KP;
-#pragma unroll
-  for (int m = 0; m < 8; ++m) trow[3 * (t + m * kS3T) + q] = v[0][m];
-  __syncthreads();
-  constexpr int NST = kS3L * kS3Units / kS3Threads;  // 8 stores per thread
-  const int r = threadIdx.x % kS3Units;              // the same row for all of a thread's stores
+  cpair *const lines[1] = {ps + size_t(w) * kS3LP}, *const lines2[1] = {ps + size_t(3 * r + qs) * kS3LP};
+  RegPlan<kS3M, 0>::template run_regrouped<cpair, 1, false, 1>(v, lines, t, lines2, tq, tr, WarpSync{}, CtaSync{});
   if (z0 + r < nz) {
     cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0 + r;
 #pragma unroll
-    for (int i = 0; i < NST; ++i) {
-      const int kx = threadIdx.x / kS3Units + i * (kS3Threads / kS3Units);
-      Tp[size_t(kx) * nz] = ps[size_t(r) * kS3KP + kx];
-    }
+    for (int m = 0; m < 8; ++m) Tp[size_t(3 * (tq + m * kS3T) + qs) * nz] = v[0][m];
   }
 }
 
-// Rows z0 .. z0 + 3: the spectra T[kx][z0 .. z0 + 3] through the transposition tile, warp (row, q) the inverse transform of residue q, the residues combined
+// Rows z0 .. z0 + 3: the spectra T[kx][z0 .. z0 + 3] by warp (row, q) the inverse transform of residue q, the residues combined
 // into y_x for x < nx, then the epilogue of rows_inverse_tile: out = ident - scale * y (or the
 // scaled y) with the fused inner products.
 template <int EPI, typename A>
 __device__ __forceinline__ void rows_inverse_tile_s3(const A &a, int tile, float2 *smem) {
   using C = float2;
   const int w = threadIdx.x >> 5, t = threadIdx.x & 31;
-  const int rr = w / 3, q = w - 3 * rr;
+  const int rr = w / 3;
   const int z0 = tile * kS3Units, z = z0 + rr;
   const int nz = a.nz(), nx = a.nx();
   const C *tw = a.tw();
   const TwReg<C, kS3M, 0> tr(t, tw);
   cpair *ps = reinterpret_cast<cpair *>(smem);
-  constexpr int NLD = kS3L * kS3Units / kS3Threads;  // 8 copies per thread, all in flight
+  cpair v[1][8];
+  const int r = threadIdx.x % kS3Units, tq = threadIdx.x / kS3Units % kS3T, qs = threadIdx.x / (kS3Units * kS3T);
   {
-    const int r = threadIdx.x % kS3Units;
     const bool in = z0 + r < nz;
     const cpair *T0 = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
 #pragma unroll
-    for (int i = 0; i < NLD; ++i) {
-      const int kx = threadIdx.x / kS3Units + i * (kS3Threads / kS3Units);
-      cp_async16z(ps + size_t(r) * kS3KP + kx, T0 + size_t(kx) * nz, in);
-    }
+    for (int m = 0; m < 8; ++m) v[0][m] = in ? load_spectrum(T0 + size_t(3 * (tq + m * kS3T) + qs) * nz) : pzero();
   }
-  cp_async_wait_all();
-  __syncthreads();
-  cpair v[1][8];
-  {
-    const cpair *trow = ps + size_t(rr) * kS3KP;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) v[0][m] = trow[3 * (t + m * kS3T) + q];
-  }
-  __syncthreads();  // the lines reuse the tile's memory
-  cpair *const lines[1] = {ps + size_t(w) * kS3LP};
-  RegPlan<kS3M, 0>::template run<cpair, 1, true>(v, lines, t, tr, WarpSync{});
+  prefetch_rows<kS3Threads>(a, a.ident(), z0, kS3Units, sizeof(C));
+  if constexpr (EPI == 1) prefetch_rows<kS3Threads>(a, a.krhat(), z0, kS3Units, sizeof(C));
+  cpair *const lines[1] = {ps + size_t(3 * r + qs) * kS3LP}, *const lines2[1] = {ps + size_t(w) * kS3LP};
+  RegPlan<kS3M, 0>::template run_regrouped<cpair, 1, true, 0>(v, lines, tq, lines2, t, tr, WarpSync{}, CtaSync{});
   cpair yp[4];
   s3_combine(v[0], ps, w, t, tw, yp);
   C y[2][4];

@@ -3,7 +3,8 @@
 // (group.cu). A tile is the work of one 256-thread CTA:
 //   rows_forward_tile  : ROWS = 2048 / L rows of one problem: contrast source by central
 //                        differences (fields zero outside D), zero-pad to lx, forward FFT along x,
-//                        transpose through shared memory into the column-major spectra T[c][kx][z]
+//                        transposed into the column-major spectra, T[kx][z] pairs (complex64: by the
+//                        threads of the last pass) or T[c][kx][z] (complex128: through shared memory)
 //   cols_tile          : CC = 2048 / L columns kx of one problem: forward FFT along z of the nz
 //                        non-zero rows padded to lz, 2x2 multiply by Ghat(kz, kx), inverse FFT
 //                        along z, keep z < nz
@@ -44,16 +45,28 @@ template <> struct Cfg<double2> {
 };
 constexpr int kTileThreads = 256;
 
+// Pitch of the lines of pairs of ROWS rows transformed side by side. The row stages read and write the
+// column-major spectra from registers, thread (row, t) = (i % ROWS, i / ROWS): runs of ROWS points are
+// contiguous in T, and the threads take these places at the exchange next to the global access
+// (RegPlan::run_regrouped), which saves the transposition tile (a third of the shared-memory traffic
+// that bounded the stages: forward and inverse at length 1024 30.2 -> 27.1 and 48.3 -> 46.0 us per 16
+// problems of 512^2, at 512 277 -> 262 and 177 -> 163 us per 256 of 256^2). With the pitch 8 / ROWS mod 8 (odd from 8 rows on) a quarter warp's 16-byte
+// accesses hit 8 distinct bank slots down the rows too.
+constexpr int row_pitch_from(int p, int rows) {
+  return p % 8 == (rows >= 8 ? 1 : 8 / rows) % 8 ? p : row_pitch_from(p + 1, rows);
+}
+template <int LX, int ROWS> constexpr int row_pitch = row_pitch_from(RegFFT<cpair, LX>::LP, ROWS);
+// Barrier over the CTA.
+struct CtaSync {
+  __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+
 template <typename C, int LX, int NTT = kTileThreads> struct RowCfg {
   static constexpr int T = LX / 8;
   static constexpr int ROWS = NTT / T;
   static constexpr int NT = ROWS * T;
   static constexpr int LP = RegFFT<C, LX>::LP;
-  // complex64: lines of pairs, and the transposition tile [ROWS][KP] of pairs. A quarter warp's
-  // 16-byte accesses hit 8 distinct bank slots both along a row (consecutive kx) and down the tile
-  // (min(ROWS, 8) rows x consecutive kx).
-  static constexpr int PLP = RegFFT<cpair, LX>::LP;
-  static constexpr int KP = LX + (ROWS >= 8 ? 1 : 8 / ROWS);
+  static constexpr int PLP = row_pitch<LX, ROWS>;
 };
 template <typename C, int LZ, int NTT = kTileThreads> struct ColCfg {
   static constexpr int T = LZ / 8;
@@ -71,7 +84,7 @@ template <typename C> constexpr bool kPairSpectra = sizeof(C) == sizeof(float2);
 // input to a forward transform and never needed on output of an inverse one.
 constexpr int kHalf = 4;
 
-// Transposition tile of the rows kernels: [2][LX][ROWS + 1] (padded against bank conflicts).
+// Transposition tile of the complex128 rows kernels: [2][LX][ROWS + 1] (padded against bank conflicts).
 template <typename C, int LX, int NTT = kTileThreads> constexpr size_t tile_elems() {
   return size_t(2) * LX * (RowCfg<C, LX, NTT>::ROWS + 1);
 }
@@ -98,7 +111,7 @@ template <typename C, int LX, int NTT = kTileThreads> inline size_t rows_forward
   using RC = RowCfg<C, LX, NTT>;
   const size_t lines = kPairSpectra<C> ? size_t(RC::ROWS) * RC::PLP * sizeof(cpair)
                                        : size_t(2) * RC::ROWS * RC::LP * sizeof(C);
-  const size_t tile = kPairSpectra<C> ? size_t(RC::ROWS) * RC::KP * sizeof(cpair) : tile_elems<C, LX, NTT>() * sizeof(C);
+  const size_t tile = kPairSpectra<C> ? 0 : tile_elems<C, LX, NTT>() * sizeof(C);
   size_t sg = 0;
   if (stencil) {
     if constexpr (kStripStencil<C, LX, NTT>) sg = stencil_strip_smem<C, LX>(nx);
@@ -112,7 +125,7 @@ template <typename C, int LZ, int NTT = kTileThreads> inline size_t cols_smem() 
 }
 template <typename C, int LX, int NTT = kTileThreads> inline size_t rows_inverse_smem() {
   using RC = RowCfg<C, LX, NTT>;
-  if (kPairSpectra<C>) return size_t(RC::ROWS) * std::max(RC::PLP, RC::KP) * sizeof(cpair);
+  if (kPairSpectra<C>) return size_t(RC::ROWS) * RC::PLP * sizeof(cpair);
   return std::max(size_t(2) * RC::ROWS * RC::LP, tile_elems<C, LX, NTT>()) * sizeof(C);
 }
 
@@ -324,25 +337,18 @@ template <int LX, int V, typename A>
 __device__ __forceinline__ void rows_forward_pairs(const A &a, int z0, int rr, int t, const float2 (&v)[2][8],
                                                    cpair *smem, const TwReg<float2, LX, V> &tr) {
   using RC = RowCfg<float2, LX>;
-  constexpr int ROWS = RC::ROWS, T = RC::T, KP = RC::KP;
-  const int nz = a.nz();
+  constexpr int ROWS = RC::ROWS, T = RC::T, LAST = PlanInfo<LX, V>::np - 2;
+  const int nz = a.nz(), r = threadIdx.x % ROWS, tq = threadIdx.x / ROWS;
   cpair p[1][8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) p[0][m] = mkpair(v[0][m], v[1][m]);
-  cpair *const line[1] = {smem + size_t(rr) * RC::PLP};
-  RegPlan<LX, V>::template run<cpair, 1, false, true>(p, line, t, tr, RowSync<T>{1 + rr});
-  __syncthreads();
-#pragma unroll
-  for (int m = 0; m < 8; ++m) smem[size_t(rr) * KP + t + m * T] = p[0][m];
-  __syncthreads();
-  cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0;
-  const int r = threadIdx.x % ROWS;
+  cpair *const line[1] = {smem + size_t(rr) * RC::PLP}, *const line2[1] = {smem + size_t(r) * RC::PLP};
+  RegPlan<LX, V>::template run_regrouped<cpair, 1, false, LAST, true>(p, line, t, line2, tq, tr, RowSync<T>{1 + rr},
+                                                                      CtaSync{});
+  cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0 + r;
   if (z0 + r < nz) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int kx = threadIdx.x / ROWS + i * (RC::NT / ROWS);
-      Tp[size_t(kx) * nz + r] = smem[size_t(r) * KP + kx];
-    }
+    for (int m = 0; m < 8; ++m) Tp[size_t(tq + m * T) * nz] = p[0][m];
   }
 }
 
@@ -360,7 +366,7 @@ __device__ __forceinline__ void rows_forward_tile(const A &a, int tile, C *smem)
   const size_t plane = size_t(nz) * nx;
   const C *u1 = a.in(), *u3 = u1 + plane;
   const Rl isc = a.isc();
-  const TwReg<C, LX, V> tr(t, a.tw());
+  const TwReg<C, LX, V> tr(t, kPairSpectra<C> ? int(threadIdx.x) / ROWS : t, a.tw());
   C v[2][8];
 
   if constexpr (STENCIL && kStripStencil<C, LX, NTT>) {
@@ -572,6 +578,29 @@ __device__ __forceinline__ void cols_tile(const A &a, int tile, C *smem) {
   }
 }
 
+// A point of the spectra, read once: not kept in L1 (whose lines in flight limit these 64-byte runs).
+__device__ __forceinline__ cpair load_spectrum(const cpair *p) {
+  const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
+  cpair r;
+  reinterpret_cast<float4 &>(r) = v;
+  return r;
+}
+
+// Starts fetching rows z0 .. z0 + rows - 1 of both components of a field (NULL: none) into L2, for the
+// epilogue after the transform (the inverse row stage of 96 problems of 384^2: 214 -> 190 us, of
+// 256 of 256^2 184 -> 177 us; copies into shared memory instead cost the L1 its lines and took 268 us).
+template <int NT, typename A>
+__device__ __forceinline__ void prefetch_rows(const A &a, const void *field, int z0, int rows, int elem) {
+  const int R = min(rows, a.nz() - z0);
+  if (!field || R <= 0) return;
+  const size_t run = size_t(R) * a.nx() * elem, plane = size_t(a.nz()) * a.nx() * elem;
+  const char *p = static_cast<const char *>(field) + size_t(z0) * a.nx() * elem;
+  for (size_t o = threadIdx.x * size_t(128); o < run; o += size_t(NT) * 128) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p + o)));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p + plane + o)));
+  }
+}
+
 // Inverse FFT along x of ROWS rows, keep x < nx, out = ident - osc * result (or the scaled
 // result when there is no identity term).
 template <typename C, int LX, int EPI, int V, int NTT = kTileThreads, typename A>
@@ -585,26 +614,18 @@ __device__ __forceinline__ void rows_inverse_tile(const A &a, int tile, C *smem)
   const TwReg<C, LX, V> tr(t, a.tw());
   C v[2][8];
   if constexpr (kPairSpectra<C>) {
-    // ROWS consecutive z of every kx into tile[r][kx] by asynchronous copies (zeros beyond nz), then
-    // each thread takes its row
-    constexpr int KP = RC::KP;
-    cpair *tile_p = reinterpret_cast<cpair *>(smem);
-    const int r = threadIdx.x % ROWS;
+    // thread (r, tq) takes its points of row z0 + r straight into registers (zeros beyond nz)
+    cpair *lines_p = reinterpret_cast<cpair *>(smem);
+    const int r = threadIdx.x % ROWS, tq = threadIdx.x / ROWS;
     const bool in = z0 + r < nz;
     const cpair *Tp = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int kx = threadIdx.x / ROWS + i * (RC::NT / ROWS);
-      cp_async16z(tile_p + size_t(r) * KP + kx, Tp + size_t(kx) * nz, in);
-    }
-    cp_async_wait_all();
-    __syncthreads();
     cpair p[1][8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) p[0][m] = tile_p[size_t(rr) * KP + t + m * T];
-    __syncthreads();  // the FFT lines reuse the tile
-    cpair *const line[1] = {tile_p + size_t(rr) * RC::PLP};
-    RegPlan<LX, V>::template run<cpair, 1, true>(p, line, t, tr, RowSync<T>{1 + rr});
+    for (int m = 0; m < 8; ++m) p[0][m] = in ? load_spectrum(Tp + size_t(tq + m * T) * nz) : pzero();
+    prefetch_rows<RC::NT>(a, a.ident(), z0, ROWS, sizeof(C));
+    if constexpr (EPI == 1) prefetch_rows<RC::NT>(a, a.krhat(), z0, ROWS, sizeof(C));
+    cpair *const line[1] = {lines_p + size_t(r) * RC::PLP}, *const line2[1] = {lines_p + size_t(rr) * RC::PLP};
+    RegPlan<LX, V>::template run_regrouped<cpair, 1, true, 0>(p, line, tq, line2, t, tr, RowSync<T>{1 + rr}, CtaSync{});
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       v[0][m] = comp0(p[0][m]);

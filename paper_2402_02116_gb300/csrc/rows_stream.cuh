@@ -15,10 +15,10 @@ namespace dbi {
 
 template <int LX> struct StreamCfg {
   static constexpr int T = LX / 8, ROWS = 4, NT = LX / 2, W = NT + 2;
-  static constexpr int PLP = RegFFT<cpair, LX>::LP, KP = LX + 2;  // as RowCfg, four rows
-  // u and sigma rows [2][W] each, the sources [4][NT], then the FFT lines / the transposition tile
+  static constexpr int PLP = row_pitch<LX, ROWS>;
+  // u and sigma rows [2][W] each, the sources [4][NT], then the FFT lines
   static constexpr size_t ring = size_t(4) * W, src = size_t(ROWS) * NT;
-  static constexpr size_t fft = size_t(ROWS) * (PLP > KP ? PLP : KP);
+  static constexpr size_t fft = size_t(ROWS) * PLP;
   static constexpr size_t smem = (ring + src + fft) * sizeof(cpair);
 };
 
@@ -27,7 +27,7 @@ template <int LX, int V, typename A>
 __device__ __forceinline__ void rows_stream(const A &a, int zb, int ze, float4 *smem) {
   using S = StreamCfg<LX>;
   using C = float2;
-  constexpr int T = S::T, NT = S::NT, W = S::W, KP = S::KP;
+  constexpr int T = S::T, NT = S::NT, W = S::W;
   const int nz = a.nz(), nx = a.nx(), x = threadIdx.x;
   const size_t plane = size_t(nz) * nx;
   const bool col = x < nx;
@@ -121,7 +121,8 @@ __device__ __forceinline__ void rows_stream(const A &a, int zb, int ze, float4 *
   step.template operator()<1>(j0, nullptr);
   step.template operator()<0>(j0 + 1, nullptr);
   const int rr = threadIdx.x / T, t = threadIdx.x - rr * T;
-  const TwReg<C, LX, V> tr(t, a.tw());
+  const int r = threadIdx.x % 4, tq = threadIdx.x / 4;
+  const TwReg<C, LX, V> tr(t, tq, a.tw());
   for (int z0 = zb; z0 < ze; z0 += 4) {
     step.template operator()<1>(z0 + 1, so);
     step.template operator()<0>(z0 + 2, so + NT);
@@ -130,20 +131,13 @@ __device__ __forceinline__ void rows_stream(const A &a, int zb, int ze, float4 *
     cpair p[1][8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) p[0][m] = m < kHalf ? reinterpret_cast<const cpair *>(so)[rr * NT + t + m * T] : pzero();
-    cpair *const line[1] = {ps + size_t(rr) * S::PLP};
-    RegPlan<LX, V>::template run<cpair, 1, false, true>(p, line, t, tr, RowSync<T>{1 + rr});
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < 8; ++m) ps[size_t(rr) * KP + t + m * T] = p[0][m];
-    __syncthreads();
-    cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0;
-    const int r = threadIdx.x % 4;
+    cpair *const line[1] = {ps + size_t(rr) * S::PLP}, *const line2[1] = {ps + size_t(r) * S::PLP};
+    RegPlan<LX, V>::template run_regrouped<cpair, 1, false, PlanInfo<LX, V>::np - 2, true>(
+        p, line, t, line2, tq, tr, RowSync<T>{1 + rr}, CtaSync{});
+    cpair *Tp = reinterpret_cast<cpair *>(a.T()) + z0 + r;
     if (z0 + r < nz) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int kx = threadIdx.x / 4 + i * (NT / 4);
-        Tp[size_t(kx) * nz + r] = ps[size_t(r) * KP + kx];
-      }
+      for (int m = 0; m < 8; ++m) Tp[size_t(tq + m * T) * nz] = p[0][m];
     }
   }
 }

@@ -2,7 +2,8 @@
 // CTAs whose lanes hold one component each (T = L / 8 lanes per line, the two components of a row
 // or column side by side). FP64 runs at about two lanes a cycle and SM, so a warp's FP64 instruction
 // count is its time: with both components per thread the three stages of one 32 x 32 problem took 24,
-// 19 and 15 us, its whole BiCGSTAB solve 1.10 ms, and with one component 0.84 ms. The spectra T[c][kx][z] are read and written from registers (strided, but they stay in L2).
+// 19 and 15 us and its BiCGSTAB solve 1.10 ms, with one component 0.84 ms. The spectra T[c][kx][z]
+// are read and written from registers (strided, but they stay in L2).
 #pragma once
 
 #include "op_tiles.cuh"
