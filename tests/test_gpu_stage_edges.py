@@ -2,7 +2,8 @@
 stage (rows_stream.cuh: row counts that end inside a chunk of 4 to 32 rows, widths at and below half the
 length), the 16-points-per-thread columns (fft16.cuh: each length, problem counts that do and don't fill
 a CTA's slots) and the stages of small complex128 batches (small64.cuh), each alone and inside a solve
-whose scalar steps run in the last CTA of a launch (krylov_finish.cuh).
+whose scalar steps run in the last CTA of a launch (krylov_finish.cuh). The literal form's complex64
+kernels (form_k.cu) likewise: each length, problem counts that do and don't fill a CTA's slots.
 
 Tolerances: those of the other operator tests, 1e-5 (complex64: FP32 rounding 6e-8 times the depth of the
 transforms and the stencil's cancellation) and 1e-10 (complex128) of A u, 20 times that of the
@@ -24,14 +25,15 @@ def oracle_for(w):
     return O.LSOracle(w.nz, w.nx, w.h, w.lz, w.lx, w.rho0, w.alpha0, w.beta0, w.omegas)
 
 
-def check_apply(precision, nz, nx, n_src, freqs, **lens):
+def check_apply(precision, nz, nx, n_src, freqs, literal=False, **lens):
     w = inputs.small_case(nz, nx, n_src=n_src, freqs=freqs, amp=0.15, **lens)
     P, orc, fs = DeviceProblem(w, precision), oracle_for(w), w.problem_fidx()
     u = inputs.seeded_complex((5, 2, nz, nx), nz + nx)
     pick = torch.arange(P.B, device=P.device) % 5
-    out = P.apply(P.to_field(u)[pick].contiguous())
+    out = (P.apply_k if literal else P.apply)(P.to_field(u)[pick].contiguous())
+    apply = orc.apply_k if literal else orc.apply
     for b in sorted({0, P.B // 2, P.B - 2, P.B - 1} & set(range(P.B))):
-        got, want = out[b].cpu().numpy(), orc.apply(u[b % 5], w.model, fs[b])
+        got, want = out[b].cpu().numpy(), apply(u[b % 5], w.model, fs[b])
         assert np.linalg.norm(got - want) < TOL[precision] * np.linalg.norm(want), b
         assert np.linalg.norm(got - want) < 20 * TOL[precision] * np.linalg.norm(want - u[b % 5]), b
 
@@ -71,3 +73,10 @@ def test_solves_match_oracle(precision, nz, nx, n_src):
     for b in (0, P.B - 1):
         want = orc.solve(orc.incident(f[b], w.src_cells[s[b]], w.src_force[s[b]]), w.model, f[b], tol=1e-12)
         assert np.linalg.norm(u[b].cpu().numpy() - want) <= bound * np.linalg.norm(want), b
+
+
+@pytest.mark.parametrize("nz, nx, lens", [(1, 3, {}), (9, 8, {}), (8, 9, {}), (17, 33, {}), (33, 65, {}), (64, 129, {}),
+                                          (130, 20, {}), (5, 300, {}), (300, 5, {}), (7, 6, dict(lz=64, lx=512))])
+@pytest.mark.parametrize("n_src", [1, 2, 9])
+def test_literal_form_pairs(nz, nx, lens, n_src):
+    check_apply(dbi.C64, nz, nx, n_src, (6.0, 11.0), literal=True, **lens)
