@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_scale_v(Span sp, const int *
   DBI_PROBLEM_LOOP(sp) v[off + i] = cscale(v[off + i], f);
 }
 
-// Partials of h_i = <v_i, w> for the basis vectors i of group blockIdx.z (i <= j), w = v_(j+1),
+// Partials of h_i = <v_i, w> for the basis vectors i of group blockIdx.y (i <= j), w = v_(j+1),
 // and (group 0 of the first pass) of ||w||^2. The second Gram-Schmidt pass (round = 1) runs only
 // for the problems that re-orthogonalise.
 template <typename C>
@@ -198,11 +198,11 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_dots(Span sp, const int *pli
                                                          size_t vstride, int j, int round, double *partD) {
   pdl_begin();
   using A = typename Acc<C>::type;
-  const int b = problem_at(plist, blockIdx.y);
+  const int b = problem_at(plist, blockIdx.z);
   if (!active[b] || (round == 1 && !st[b].need2)) return;
-  const int i0 = blockIdx.z * kDotGroup;
+  const int i0 = blockIdx.y * kDotGroup;
   const int nv = min(kDotGroup, j + 1 - i0);
-  const bool norm = round == 0 && blockIdx.z == 0;
+  const bool norm = round == 0 && blockIdx.y == 0;
   const C *w = V + size_t(j + 1) * vstride;
   A re[kDotGroup], im[kDotGroup], ww = 0;
 #pragma unroll
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_dots(Span sp, const int *pli
   }
   acc[2 * kDotGroup] = ww;
   acc[2 * kDotGroup + 1] = 0;
-  block_sum_store<kDotSlots>(acc, partD + ((size_t(b) * kDotGroups + blockIdx.z) * kRedBlocks + blockIdx.x) * kDotSlots);
+  block_sum_store<kDotSlots>(acc, partD + ((size_t(b) * kDotGroups + blockIdx.y) * kRedBlocks + blockIdx.x) * kDotSlots);
 }
 
 // h_i = <v_i, K v_j> (i <= j) from the partials, in a fixed order; hc[b][i] = h_i and column j
@@ -283,6 +283,8 @@ __global__ void k_gm_hsum(const int *plist, const int *active, GState *st, const
 
 // w -= sum_(i <= j) h_i v_i, partials of ||w||^2. The basis vectors are read eight at a time so
 // that their loads are in flight together.
+// The problems run in the order opposite to the dots' (problem-major there): the last ones' basis is still
+// in L2 (64 problems of 256^2, restart 30, both passes together 9.9 -> 9.5 ms).
 template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_gm_update(Span sp, const int *plist, const int *active,
                                                            const GState *st, C *__restrict__ V, size_t vstride,
@@ -291,7 +293,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_update(Span sp, const int *p
   pdl_begin();
   using A = typename Acc<C>::type;
   __shared__ C h[kGmresMaxRestart + kDotGroup];
-  const int b = problem_at(plist, blockIdx.y);
+  const int b = problem_at(plist, gridDim.y - 1 - blockIdx.y);
   if (!active[b] || (round == 1 && !st[b].need2)) return;
   for (int i = threadIdx.x; i < kGmresMaxRestart + kDotGroup; i += blockDim.x)
     h[i] = i <= j ? from_z<C>(hc[size_t(b) * (m + 1) + i]) : czero<C>();
@@ -359,27 +361,42 @@ __global__ void k_gm_need2(const int *plist, const int *active, GState *st, cons
 __global__ void k_gm_close(const int *plist, int *active, GState *st, double2 *H, double2 *g, double *cs,
                            double2 *sn, const double *partN, int j, int m, double tol, int max_iter) {
   pdl_begin();
+  // the column and the earlier rotations come to shared memory at once and the column goes back at
+  // once: with each step of the chain a round trip to L2 the kernel took 20.6 us at restart 30, now 15.3 us
+  __shared__ double2 h[kGmresMaxRestart + 1], sr[kGmresMaxRestart];
+  __shared__ double cr[kGmresMaxRestart];
   const int b = problem_at(plist, blockIdx.x);
   if (!active[b]) return;
-  double s[1];
-  gather_n<1>(partN + size_t(b) * kRedBlocks * kRedSlots, kRedBlocks, s);
-  if (threadIdx.x != 0) return;
-  GState k = st[b];
-  const double hn = sqrt(s[0]);
   double2 *Hb = H + size_t(b) * (m + 1) * m;
   double *cb = cs + size_t(b) * m;
   double2 *sb = sn + size_t(b) * m;
   double2 *gb = g + size_t(b) * (m + 1);
-  for (int i = 0; i < j; ++i) {  // (h_i, h_(i+1)) <- (c h_i + s h_(i+1), -conj(s) h_i + c h_(i+1))
-    const double2 a0 = Hb[size_t(i) * m + j], a1 = Hb[size_t(i + 1) * m + j];
-    const double c = cb[i];
-    const double2 sv = sb[i];
-    Hb[size_t(i) * m + j] = make_double2(c * a0.x + sv.x * a1.x - sv.y * a1.y, c * a0.y + sv.x * a1.y + sv.y * a1.x);
-    Hb[size_t(i + 1) * m + j] =
-        make_double2(-(sv.x * a0.x + sv.y * a0.y) + c * a1.x, -(sv.x * a0.y - sv.y * a0.x) + c * a1.y);
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+    h[i] = Hb[size_t(i) * m + j];
+    if (i < j) {
+      cr[i] = cb[i];
+      sr[i] = sb[i];
+    }
   }
+  double s[1];
+  gather_n<1>(partN + size_t(b) * kRedBlocks * kRedSlots, kRedBlocks, s);
+  __syncthreads();
+  double2 a = h[0];
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < j; ++i) {  // (h_i, h_(i+1)) <- (c h_i + s h_(i+1), -conj(s) h_i + c h_(i+1))
+      const double2 a0 = a, a1 = h[i + 1];
+      const double c = cr[i];
+      const double2 sv = sr[i];
+      h[i] = make_double2(c * a0.x + sv.x * a1.x - sv.y * a1.y, c * a0.y + sv.x * a1.y + sv.y * a1.x);
+      a = make_double2(-(sv.x * a0.x + sv.y * a0.y) + c * a1.x, -(sv.x * a0.y - sv.y * a0.x) + c * a1.y);
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < j; i += blockDim.x) Hb[size_t(i) * m + j] = h[i];
+  if (threadIdx.x != 0) return;
+  GState k = st[b];
+  const double hn = sqrt(s[0]);
   // rotation of (a, hn), hn real >= 0: c = |a| / t, s = (a / |a|) hn / t, r = (a / |a|) t
-  const double2 a = Hb[size_t(j) * m + j];
   const double aa = hypot(a.x, a.y), t = hypot(aa, hn);
   double c;
   double2 sv, r;
@@ -417,25 +434,48 @@ __global__ void k_gm_close(const int *plist, int *active, GState *st, double2 *H
 }
 
 // End of a cycle: y from R y = g by back substitution for every problem that ran this cycle.
-__global__ void k_gm_solve_y(int B, GState *st, const double2 *H, const double2 *g, double2 *y, int m) {
+// One warp per problem, column by column from the last (one thread per problem, row by row: 223 us at
+// restart 30; now 42 us).
+__global__ void __launch_bounds__(32) k_gm_solve_y(GState *st, const double2 *H, const double2 *g, double2 *y, int m) {
   pdl_begin();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  GState k = st[b];
-  k.kx = k.incycle ? k.k : 0;
-  k.incycle = 0;
-  st[b] = k;
+  __shared__ double2 acc[kGmresMaxRestart];
+  const int b = blockIdx.x, lane = threadIdx.x;
+  const int kx = st[b].incycle ? st[b].k : 0;
+  __syncwarp();
+  if (lane == 0) {
+    st[b].kx = kx;
+    st[b].incycle = 0;
+  }
   const double2 *Hb = H + size_t(b) * (m + 1) * m;
-  const double2 *gb = g + size_t(b) * (m + 1);
-  double2 *yb = y + size_t(b) * m;
-  for (int i = k.kx - 1; i >= 0; --i) {
-    double2 acc = gb[i];
-    for (int l = i + 1; l < k.kx; ++l) {
-      const double2 p = zmul(Hb[size_t(i) * m + l], yb[l]);
-      acc.x -= p.x;
-      acc.y -= p.y;
+  for (int i = lane; i < kx; i += 32) acc[i] = g[size_t(b) * (m + 1) + i];
+  constexpr int Q = (kGmresMaxRestart + 31) / 32;
+  double2 col[Q], next[Q];  // rows lane + 32 q of columns i and i - 1
+  auto load = [&](int i, double2 (&c)[Q]) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int l = lane + 32 * q;
+      c[q] = l <= i ? Hb[size_t(l) * m + i] : make_double2(0.0, 0.0);
     }
-    yb[i] = zdiv(acc, Hb[size_t(i) * m + i]);
+  };
+  load(kx - 1, col);
+  for (int i = kx - 1; i >= 0; --i) {
+    load(i - 1, next);
+    double2 d = make_double2(0.0, 0.0);  // H_ii, from the lane that holds row i
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (i / 32 == q) d = make_double2(__shfl_sync(0xffffffffu, col[q].x, i % 32), __shfl_sync(0xffffffffu, col[q].y, i % 32));
+    __syncwarp();
+    const double2 yi = zdiv(acc[i], d);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int l = lane + 32 * q;
+      if (l < i) {
+        const double2 p = zmul(col[q], yi);
+        acc[l] = make_double2(acc[l].x - p.x, acc[l].y - p.y);
+      }
+      col[q] = next[q];
+    }
+    if (lane == 0) y[size_t(b) * m + i] = yi;
   }
 }
 
@@ -550,7 +590,7 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
           launch_pdl(k_gm_need2, nrun, 32, 0, s, plist, gb.active, gb.st, gb.partN);
           if ((rc = check_launch("k_gm_need2"))) return rc;
         }
-        const dim3 g3(kRedBlocks, nrun, (j + 1 + kDotGroup - 1) / kDotGroup);
+        const dim3 g3(kRedBlocks, (j + 1 + kDotGroup - 1) / kDotGroup, nrun);
         launch_pdl(k_gm_dots<C>, g3, kRedThreads, 0, s, sp, plist, gb.active, gb.st, V, vstride, j, round, gb.partD);
         if ((rc = check_launch("k_gm_dots"))) return rc;
         launch_pdl(k_gm_hsum, nrun, 2 * kGmresMaxRestart + 32, 0, s, plist, gb.active, gb.st, gb.partD, gb.hc, gb.H, j,
@@ -572,7 +612,7 @@ static int gmres_typed(OpArgs op, const GmresBufs &gb, int m, const void *rhs_, 
         if (nact == 0) break;
       }
     }
-    launch_pdl(k_gm_solve_y, (B + 127) / 128, 128, 0, s, B, gb.st, gb.H, gb.g, gb.y, m);
+    launch_pdl(k_gm_solve_y, B, 32, 0, s, gb.st, gb.H, gb.g, gb.y, m);
     if ((rc = check_launch("k_gm_solve_y"))) return rc;
     launch_pdl(k_gm_update_x<C>, all, kRedThreads, 0, s, sp, gb.st, V, vstride, gb.y, m, x);
     if ((rc = check_launch("k_gm_update_x"))) return rc;
