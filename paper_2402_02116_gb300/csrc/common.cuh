@@ -93,6 +93,12 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src, bool valid
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 #endif
 
+// blockIdx.y from the last to the first. Every second kernel of a chain of passes over a batch takes its
+// problems in this order: the ones the kernel before it has written last are still in L2. (Operator on 384
+// problems of 512^2 5.74 -> 5.70 ms, on 96 of 384^2 1.040 -> 1.034 ms; gradient step of 32 of 512^2
+// 113.5 -> 112.1 ms.)
+__device__ __forceinline__ int reversed_y() { return int(gridDim.y) - 1 - int(blockIdx.y); }
+
 // Programmatic dependent launch: launch_pdl starts a kernel while the one before it on the stream is
 // still draining, and pdl_begin(), the first statement of every kernel launched so, holds its threads
 // until the earlier kernels have completed and their writes are visible (then lets the next launch

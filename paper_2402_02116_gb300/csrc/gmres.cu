@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gm_update(Span sp, const int *p
   pdl_begin();
   using A = typename Acc<C>::type;
   __shared__ C h[kGmresMaxRestart + kDotGroup];
-  const int b = problem_at(plist, gridDim.y - 1 - blockIdx.y);
+  const int b = problem_at(plist, reversed_y());
   if (!active[b] || (round == 1 && !st[b].need2)) return;
   for (int i = threadIdx.x; i < kGmresMaxRestart + kDotGroup; i += blockDim.x)
     h[i] = i <= j ? from_z<C>(hc[size_t(b) * (m + 1) + i]) : czero<C>();

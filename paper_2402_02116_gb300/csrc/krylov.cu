@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_s(Span sp, const int *pl
                                                           double *partS) {
   pdl_begin();
   using A = typename Acc<C>::type;
-  const int b = problem_at(plist, blockIdx.y);
+  const int b = problem_at(plist, reversed_y());
   if (!active[b]) return;
   const C al = state_alpha<C>(st[b]);
   A ss = 0;
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *p
                                                            C *__restrict__ r, double *partC) {
   pdl_begin();
   using A = typename Acc<C>::type;
-  const int b = problem_at(plist, blockIdx.y);
+  const int b = problem_at(plist, reversed_y());
   if (!active[b]) return;
   const C al = state_alpha<C>(st[b]), o = state_omega<C>(st[b]);
   A re = 0, im = 0, rr = 0;

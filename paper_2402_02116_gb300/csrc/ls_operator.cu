@@ -46,9 +46,9 @@ template <typename C> struct OpP {
   C *S;  // [slots][2][nz][nx] contrast-source scratch of the split row stages (L = 1024, 768), or NULL
 };
 
-// Problem of this CTA's launch slot (blockIdx.y); the spectral scratch is indexed by the slot.
-template <typename C> __device__ __forceinline__ int problem_of(const OpP<C> &p) {
-  const int sl = p.s0 + int(blockIdx.y);
+// Problem of this CTA's launch slot y (blockIdx.y, or reversed_y()); the spectral scratch is indexed by the slot.
+template <typename C> __device__ __forceinline__ int problem_of(const OpP<C> &p, int y = blockIdx.y) {
+  const int sl = p.s0 + y;
   return p.plist ? p.plist[sl] : sl;
 }
 
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kTileThreads, Cfg<float2>::colMinBlocks) k_col
   cpair *lines = reinterpret_cast<cpair *>(smem_raw);
   float2 *Gs = reinterpret_cast<float2 *>(lines + size_t(CF::CC) * CF::PLP);
   const int u = threadIdx.x / CF::T, t = threadIdx.x - u * CF::T;
-  const int kx = blockIdx.x * COLS + u / SL, sl0 = SL * int(blockIdx.y), sl = sl0 + u % SL;
+  const int kx = blockIdx.x * COLS + u / SL, sl0 = SL * reversed_y(), sl = sl0 + u % SL;
   auto prob = [&](int slot) { return p.plist ? p.plist[p.s0 + slot] : p.s0 + slot; };
   auto freq = [&](int slot) {  // the slot's table, or -1 when it has no work
     if (slot >= p.nb) return -1;
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kCols16Threads, 3) k_cols16(OpP<float2> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int u = threadIdx.x / T, t = threadIdx.x % T;
   cpair *line = reinterpret_cast<cpair *>(smem_raw) + size_t(u) * F::LP;
-  const int kx = blockIdx.x * COLS + u / SL, sl = SL * int(blockIdx.y) + u % SL;
+  const int kx = blockIdx.x * COLS + u / SL, sl = SL * reversed_y() + u % SL;
   int f = -1;
   if (sl < p.nb && kx < p.lx) {
     const int b = p.plist ? p.plist[p.s0 + sl] : p.s0 + sl;
@@ -262,10 +262,10 @@ template <int LX, int EPI, int V> __global__ void __launch_bounds__(32) k_rows_i
 // Stages of the L = 1024 complex64 operator as pairs of 512-point transforms (op_split.cuh).
 __global__ void __launch_bounds__(kSrcThreads) k_source_split(OpP<float2> p) {
   pdl_begin();
-  const int b = problem_of(p), f = p.fidx[b];
+  const int b = problem_of(p, reversed_y()), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const BatchTile<float2> a{p, b, int(blockIdx.y), f};
+  const BatchTile<float2> a{p, b, reversed_y(), f};
   source_rows(a, blockIdx.x, reinterpret_cast<float2 *>(smem_raw), a.S());
 }
 
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_rows_forward_split(OpP<floa
   else rows_forward_tile_split(a, blockIdx.x, smem, a.in(), a.isc());
 }
 
-// Column kx = blockIdx.x of the four launch slots 4 blockIdx.y .. + 3 (64 threads each). The
+// Column kx = blockIdx.x of the four launch slots 4 y .. + 3 (y = reversed_y()) (64 threads each). The
 // column's Green's tables of the first slot's frequency are staged in shared memory by
 // asynchronous copies issued before the forward transforms, so their latency is hidden; slots of
 // that frequency (consecutive slots share it, problems being frequency-major) read them there,
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_cols_split(OpP<float2> p) {
   float2 *smem = reinterpret_cast<float2 *>(smem_raw);
   float4 *Gs = reinterpret_cast<float4 *>(smem + split_cols_lines_smem() / sizeof(float2));
   const int g = threadIdx.x / kSplitT, kx = blockIdx.x;
-  const int sl0 = 4 * int(blockIdx.y), sl = sl0 + g;
+  const int sl0 = 4 * reversed_y(), sl = sl0 + g;
   auto prob = [&](int slot) { return p.plist ? p.plist[p.s0 + slot] : p.s0 + slot; };
   auto freq = [&](int slot) {  // the slot's table, or -1 when it has no work
     if (slot >= p.nb) return -1;
@@ -341,10 +341,10 @@ __global__ void __launch_bounds__(kS3Threads, 2) k_rows_forward_s3(OpP<float2> p
 
 __global__ void __launch_bounds__(kS3Threads, 2) k_cols_s3(OpP<float2> p) {
   pdl_begin();
-  const int b = problem_of(p), f = p.fidx[b];
+  const int b = problem_of(p, reversed_y()), f = p.fidx[b];
   if ((p.active && !p.active[b]) || unsigned(f) >= unsigned(p.nf)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cols_tile_s3(BatchTile<float2>{p, b, int(blockIdx.y), f}, blockIdx.x, reinterpret_cast<float2 *>(smem_raw));
+  cols_tile_s3(BatchTile<float2>{p, b, reversed_y(), f}, blockIdx.x, reinterpret_cast<float2 *>(smem_raw));
 }
 
 template <int EPI>

@@ -21,10 +21,10 @@ template <typename C> __device__ __forceinline__ C from_z(double2 z) {
   return mk<C>(R(z.x), R(z.y));
 }
 
-// Grid-stride loop over the n elements of problem b (unrolled for memory parallelism).
 // Problem of this CTA: plist[blockIdx.y] when the launch runs a compacted list of problems.
 __device__ __forceinline__ int problem_at(const int *plist, int slot) { return plist ? plist[slot] : slot; }
 
+// Grid-stride loop over the n elements of problem b (unrolled for memory parallelism).
 #define DBI_PROBLEM_LOOP(sp)                                                                  \
   const size_t off = (sp).offset(b), cnt = (sp).count(b);                                     \
   _Pragma("unroll 4")                                                                         \
