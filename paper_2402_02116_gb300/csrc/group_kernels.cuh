@@ -163,7 +163,9 @@ template <typename C> __device__ __forceinline__ C *group_S(const GroupP<C> &g, 
   return g.S + size_t(M.S0) + size_t(q) * 2 * M.nz * M.nx;
 }
 
-template <typename C> __global__ void __launch_bounds__(kSrcThreads) kg_source_split(GroupP<C> g) {
+// (two CTAs per SM: with a few registers more than 64 a single one is resident, and the kernel took 602 us
+// instead of 366 us for the members of 384^2 and 512^2 of a 40-problem batch)
+template <typename C> __global__ void __launch_bounds__(kSrcThreads, 2) kg_source_split(GroupP<C> g) {
   static_assert(sizeof(C) == sizeof(float2), "complex64 only");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *smem = reinterpret_cast<C *>(smem_raw);
