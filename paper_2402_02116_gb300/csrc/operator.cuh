@@ -37,7 +37,7 @@ struct OpArgs {
   const void *in;       // device [B][2][nz][nx] complex
   const void *ident;    // device [B][2][nz][nx] complex or NULL
   void *out;            // device [B][2][nz][nx] complex
-  void *T;              // device [B][2][lx][nz] complex scratch (column-major spectra)
+  void *T;              // device scratch, column-major spectra: complex64 [B][lx][nz] pairs, complex128 [B][2][lx][nz]
   const void *Ghat;     // device [nf][3][lx][lz] complex (column-major)
   const void *Dhat;     // device [nf][6][lx][lz] derivative tables: the paper-literal form (Eq. 9)
                         // replaces the stencil pass (form_k.cu; T then holds [B][7][lx][nz])
