@@ -27,17 +27,17 @@ template <typename C> __host__ __device__ __forceinline__ C mk(typename RealOf<C
 }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return mk<C>(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return mk<C>(a.x - b.x, a.y - b.y); }
-template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
+template <typename C> __host__ __device__ __forceinline__ C cmul(C a, C b) {
   return mk<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 // a * conj(b)
-template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
+template <typename C> __host__ __device__ __forceinline__ C cmulc(C a, C b) {
   return mk<C>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 template <typename C> __device__ __forceinline__ C cscale(C a, typename RealOf<C>::type s) {
   return mk<C>(a.x * s, a.y * s);
 }
-template <typename C> __device__ __forceinline__ C cconj(C a) { return mk<C>(a.x, -a.y); }
+template <typename C> __host__ __device__ __forceinline__ C cconj(C a) { return mk<C>(a.x, -a.y); }
 // multiply by -i (forward) or +i (inverse)
 template <typename C, bool INV> __device__ __forceinline__ C mul_mi(C a) {
   return INV ? mk<C>(-a.y, a.x) : mk<C>(a.y, -a.x);

@@ -55,28 +55,61 @@ __device__ __forceinline__ void s3_fold(cpair (&v)[8], int t, int q, int n, cons
   }
 }
 
+// A value of the twiddle table.
+__host__ __device__ __forceinline__ float2 s3_tw(const float2 *p) {
+#ifdef __CUDA_ARCH__
+  return __ldg(p);
+#else
+  return *p;
+#endif
+}
+
 // The residues' inverse transforms of one row or column (held by its three warps in natural
-// order) combined: y_j = sum_q W_L^{-jq} v_q[j mod M] for the unit's points j = u + 96 i (i < 4).
-// The warps first store v_q into their own lines; one CTA barrier later every thread reads the
-// three residues of its points. Every thread of the CTA must call it.
-__device__ __forceinline__ void s3_combine(const cpair (&v)[8], cpair *smem, int w, int t, const float2 *tw,
-                                           cpair (&y)[4]) {
+// order) combined: y_j = sum_q W_L^{-jq} v_q[j mod M] for the unit's points j = u + 96 i (i < 4) of
+// thread u = 32 (w mod 3) + t. The warps first store v_q into their own lines, behind a barrier of their lanes
+// (`warp`): the transform before may leave the last exchange's reads of the line unordered
+// (run_regrouped). One CTA barrier (`all`) later every thread reads the three residues of its points.
+// Every thread of the CTA must call it.
+template <typename Warp, typename All>
+__host__ __device__ __forceinline__ void s3_combine(const cpair (&v)[8], cpair *smem, int w, int t, const float2 *tw,
+                                                    cpair (&y)[4], Warp &&warp, All &&all) {
   using C = float2;
   cpair *own = smem + size_t(w) * kS3LP;
+  warp();
 #pragma unroll
   for (int m = 0; m < 8; ++m) own[t + m * kS3T] = v[m];
-  __syncthreads();
-  const int unit = w / 3, u = threadIdx.x - unit * kS3UnitThreads;
+  all();
+  const int unit = w / 3, u = (w - 3 * unit) * kS3T + t;
   const cpair *base = smem + size_t(3 * unit) * kS3LP;  // lines of warps 3 unit + q
   // W_L^{-j} = W_L^{-u} W_8^{-i} and W_L^{-2j} = W_L^{-2u} W_4^{-i} for j = u + 96 i (96 = L / 8)
-  const C wu1 = cconj(__ldg(tw + u * kS3Tw)), wu2 = cconj(__ldg(tw + 2 * u * kS3Tw));
+  const C wu1 = cconj(s3_tw(tw + u * kS3Tw)), wu2 = cconj(s3_tw(tw + 2 * u * kS3Tw));
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int j = u + i * kS3UnitThreads, jm = j & (kS3M - 1);
-    const C w1 = i ? cmulc(wu1, __ldg(tw + i * (kTwiddleN / 8))) : wu1;
-    const C w2 = i ? cmulc(wu2, __ldg(tw + i * (kTwiddleN / 4))) : wu2;
+    const C w1 = i ? cmulc(wu1, s3_tw(tw + i * (kTwiddleN / 8))) : wu1;
+    const C w2 = i ? cmulc(wu2, s3_tw(tw + i * (kTwiddleN / 4))) : wu2;
     y[i] = hadd(base[jm], hadd(hmul(base[kS3LP + jm], w1), hmul(base[2 * kS3LP + jm], w2)));
   }
+}
+
+// Inverse transform of the four rows of a tile, thread `tid` of the CTA: on entry v holds the points
+// tq + 32 m (m < 8) of residue qs of row r as the thread read them from memory (s3_place), afterwards y the
+// outputs x = u + 96 i of row w / 3.
+struct S3Place {
+  int r, tq, qs;
+};
+__host__ __device__ __forceinline__ S3Place s3_place(int tid) {
+  return {tid % kS3Units, tid / kS3Units % kS3T, tid / (kS3Units * kS3T)};
+}
+template <typename Warp, typename All>
+__host__ __device__ __forceinline__ void s3_rows_inverse(cpair (&v)[1][8], cpair *smem, int tid,
+                                                         const TwReg<float2, kS3M, 0> &tr, const float2 *tw,
+                                                         cpair (&y)[4], Warp &&warp, All &&all) {
+  const S3Place p = s3_place(tid);
+  const int w = tid / kS3T, t = tid % kS3T;
+  cpair *const lines[1] = {smem + size_t(3 * p.r + p.qs) * kS3LP}, *const lines2[1] = {smem + size_t(w) * kS3LP};
+  RegPlan<kS3M, 0>::template run_regrouped<cpair, 1, true, 0>(v, lines, p.tq, lines2, t, tr, warp, all);
+  s3_combine(v[0], smem, w, t, tw, y, warp, all);
 }
 
 // Columns kx = 4 tile .. 4 tile + 3: warp (column, q) folds the column's nz points (both
@@ -112,7 +145,7 @@ __device__ __forceinline__ void cols_tile_s3(const A &a, int tile, float2 *smem)
   }
   RegPlan<kS3M, 0>::template run<cpair, 1, true>(v, lines, t, tr, WarpSync{});
   cpair y[4];
-  s3_combine(v[0], ps, w, t, tw, y);
+  s3_combine(v[0], ps, w, t, tw, y, WarpSync{}, CtaSync{});
   if (live) {
     const int u = threadIdx.x - cc * kS3UnitThreads;
 #pragma unroll
@@ -136,8 +169,7 @@ __device__ __forceinline__ void rows_forward_tile_s3(const A &a, int tile, float
   const int nz = a.nz(), nx = a.nx();
   const size_t plane = size_t(nz) * nx;
   const C *tw = a.tw();
-  // thread (r, tq, qs) of the stores: row z0 + r, residue qs
-  const int r = threadIdx.x % kS3Units, tq = threadIdx.x / kS3Units % kS3T, qs = threadIdx.x / (kS3Units * kS3T);
+  const auto [r, tq, qs] = s3_place(threadIdx.x);  // of the stores: row z0 + r, residue qs
   const TwReg<C, kS3M, 0> tr(t, tq, tw);
   const int n = z < nz ? nx : 0;
   const C *row = src + size_t(z < nz ? z : 0) * nx;
@@ -168,19 +200,18 @@ __device__ __forceinline__ void rows_inverse_tile_s3(const A &a, int tile, float
   const TwReg<C, kS3M, 0> tr(t, tw);
   cpair *ps = reinterpret_cast<cpair *>(smem);
   cpair v[1][8];
-  const int r = threadIdx.x % kS3Units, tq = threadIdx.x / kS3Units % kS3T, qs = threadIdx.x / (kS3Units * kS3T);
   {
-    const bool in = z0 + r < nz;
-    const cpair *T0 = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + r : 0);
+    const S3Place at = s3_place(threadIdx.x);
+    const bool in = z0 + at.r < nz;
+    const cpair *T0 = reinterpret_cast<const cpair *>(a.T()) + (in ? z0 + at.r : 0);
 #pragma unroll
-    for (int m = 0; m < 8; ++m) v[0][m] = in ? load_spectrum(T0 + size_t(3 * (tq + m * kS3T) + qs) * nz) : pzero();
+    for (int m = 0; m < 8; ++m)
+      v[0][m] = in ? load_spectrum(T0 + size_t(3 * (at.tq + m * kS3T) + at.qs) * nz) : pzero();
   }
   prefetch_rows<kS3Threads>(a, a.ident(), z0, kS3Units, sizeof(C));
   if constexpr (EPI == 1) prefetch_rows<kS3Threads>(a, a.krhat(), z0, kS3Units, sizeof(C));
-  cpair *const lines[1] = {ps + size_t(3 * r + qs) * kS3LP}, *const lines2[1] = {ps + size_t(w) * kS3LP};
-  RegPlan<kS3M, 0>::template run_regrouped<cpair, 1, true, 0>(v, lines, tq, lines2, t, tr, WarpSync{}, CtaSync{});
   cpair yp[4];
-  s3_combine(v[0], ps, w, t, tw, yp);
+  s3_rows_inverse(v, ps, threadIdx.x, tr, tw, yp, WarpSync{}, CtaSync{});
   C y[2][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
