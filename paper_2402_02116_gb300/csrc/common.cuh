@@ -99,18 +99,21 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // 113.5 -> 112.1 ms.)
 __device__ __forceinline__ int reversed_y() { return int(gridDim.y) - 1 - int(blockIdx.y); }
 
-// Programmatic dependent launch: launch_pdl starts a kernel while the one before it on the stream is
-// still draining, and pdl_begin(), the first statement of every kernel launched so, holds its threads
-// until the earlier kernels have completed and their writes are visible (then lets the next launch
-// start in turn). What overlaps is the launch itself, about 1 us per kernel: a solve on a small grid
-// is a chain of hundreds of launches of a few microseconds each. A launch of several waves does not
-// let the next one in early (its waiting CTAs only skew the distribution of the last wave: 256^2 x 256
-// apply 975 us without, 994 us with). Every thread must pass pdl_begin() before any exit, so that
-// a kernel's completion implies that of all the kernels before it.
+// Programmatic dependent launch: launch_pdl lets a kernel's launch begin while the one before it on the
+// stream is still draining, and pdl_begin(), the first statement of every kernel launched so, holds its
+// threads until the earlier kernels have completed and their writes are visible. What overlaps is the
+// launch itself, about 1 us per kernel: a solve on a small grid is a chain of hundreds of launches of a
+// few microseconds each (16 BiCGSTAB iterations on one problem of 8 x 8 0.89 -> 0.71 ms, of 256^2
+// 1.36 -> 1.03 ms). No kernel triggers its successor early (griddepcontrol.launch_dependents): the waiting
+// CTAs would take the slots that are free at that moment, several on one SM beside SMs that stay empty, and
+// keep them. With the trigger in launches of up to 8 x 152 CTAs the same 16 iterations took, on 4
+// problems of 100^2 in complex128, 7.3 ms against 4.6 ms without, on 64 of 8 x 200 in complex64 1.04
+// against 0.86 ms, and on one small problem as long as without it (32^2 in complex128 1.58 against 1.55 ms).
+// Every thread must pass pdl_begin() before any exit, so that a kernel's completion implies that of all
+// the kernels before it.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (gridDim.x * gridDim.y * gridDim.z <= 8 * 152) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <typename... KA>
 inline cudaError_t launch_pdl(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
