@@ -180,6 +180,11 @@ int red_blocks(size_t n, int B, int precision) {
   return int(k < 1 ? 1 : k > size_t(kRedBlocks) ? size_t(kRedBlocks) : k);
 }
 
+int red_parts(size_t items) {
+  const size_t k = (items + kRedThreads - 1) / kRedThreads;
+  return int(k < 1 ? 1 : k > size_t(kRedBlocks) ? size_t(kRedBlocks) : k);
+}
+
 size_t bytes_scales(int B) { return 3 * align256(size_t(B) * sizeof(double)) + 256 + bytes_partials(B); }
 
 int imaging_chunks(int B) { return B < 16 ? (B > 0 ? B : 1) : 16; }

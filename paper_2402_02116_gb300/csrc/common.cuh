@@ -213,8 +213,12 @@ constexpr int kRedSlots = 4;      // doubles per block partial
 constexpr int kMaxParts = 512;    // partials per problem at most (operator kernels: one per row block)
 // Blocks per problem of a vector pass over B problems of n elements: 8 accesses per thread (16 bytes
 // each) where that gives enough blocks for every SM, else as many blocks as have work up to one wave
-// of four per SM (a second wave of a few blocks would double the time). (64 blocks whatever the size left 45 problems of 45 x 180 cells with one pair of points
-// per thread under the cost of reading the problem's scalars.)
+// of four per SM (a second wave of a few blocks would double the time). (64 blocks whatever the size left 45
+// problems of 45 x 180 cells with one pair of points per thread under the cost of reading the problem's
+// scalars.) In complex64 the sums of a pass are split into red_parts partials whatever its blocks (problem_sums,
+// vec.cuh).
 int red_blocks(size_t n, int B, int precision);
+// Partials of a sum over the items of a problem: the chunks of problem_sums that have any.
+int red_parts(size_t items);
 
 }  // namespace dbi

@@ -2,7 +2,7 @@
 // (source, frequency) problem.
 //
 // Per iteration i (van der Vorst's BiCGSTAB, <a, b> = sum conj(a) b):
-//   p = r + beta (p - omega v)                  k_update_p      (beta from the previous k_check)
+//   p = r + beta (p - omega v)                  k_update_p      (beta from the previous k_update_xr)
 //   v = A p, partials of <rhat, v>              operator (inner product in k_rows_inverse)
 //   alpha = rho / <rhat, v>                     the last CTA of each problem's k_rows_inverse (k_alpha
 //                                               for uneven batches and the paper-literal form)
@@ -15,7 +15,8 @@
 // behind a launch), 13 % of a 45 x 180 solve's iteration.
 // Every scalar lives on the device in FP64. Each reduction is two-stage and deterministic: each
 // thread sums its elements, the CTA sums its threads in a fixed tree, and every consumer sums the
-// CTA partials of its problem in the same fixed order. Converged problems drop out
+// partials of its problem in the same fixed order; in complex64 the split into partials follows from the
+// grid alone (problem_sums). Converged problems drop out
 // (their CTAs return at once); the host polls an active-problem counter every check_every
 // iterations. A breakdown (rho or omega vanishing) restarts the problem from its iterate.
 #include <cmath>
@@ -85,35 +86,32 @@ template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_init(Span sp, const KState *st, const C *__restrict__ rhs,
                                                       C *__restrict__ v, C *__restrict__ r,
                                                       C *__restrict__ rhat, C *__restrict__ p,
-                                                      C *__restrict__ x, int x_zero, double *part) {
+                                                      C *__restrict__ x, int x_zero, int nchunk, double *part) {
   pdl_begin();
   const int b = blockIdx.y;
   using A = typename Acc<C>::type;
   using R = typename RealOf<C>::type;
   const R sc = R(st[blockIdx.y].scale);
-  A bb = 0, rr = 0;
-  DBI_PROBLEM_LOOP(sp) {
-    const C bi = cscale(rhs[off + i], sc);
-    const C ax = x_zero ? czero<C>() : v[off + i];
+  problem_sums<2, C, false>(sp, b, nchunk, part + size_t(b) * kRedBlocks * kRedSlots, [&]<int N>(size_t o, A (&acc)[2]) {
+    const C bi = cscale(rhs[o], sc);
+    const C ax = x_zero ? czero<C>() : v[o];
     const C ri = csub(bi, ax);
-    r[off + i] = ri;
-    rhat[off + i] = ri;
-    p[off + i] = czero<C>();
-    v[off + i] = czero<C>();
-    if (x_zero) x[off + i] = czero<C>();
-    bb += bi.x * bi.x + bi.y * bi.y;
-    rr += ri.x * ri.x + ri.y * ri.y;
-  }
-  A acc[2] = {bb, rr};
-  block_sum_store<2>(acc, part + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
+    r[o] = ri;
+    rhat[o] = ri;
+    p[o] = czero<C>();
+    v[o] = czero<C>();
+    if (x_zero) x[o] = czero<C>();
+    acc[0] += bi.x * bi.x + bi.y * bi.y;
+    acc[1] += ri.x * ri.x + ri.y * ri.y;
+  });
 }
 
-__global__ void k_init_state(KState *st, int *active, int *counters, int *arrived, const double *part, int nblk,
+__global__ void k_init_state(KState *st, int *active, int *counters, int *arrived, const double *part, int nparts,
                              double tol, int max_iter) {
   pdl_begin();
   const int b = blockIdx.x;
   double s[2];
-  gather_n<2>(part + size_t(b) * kRedBlocks * kRedSlots, nblk, s);
+  gather_n<2>(part + size_t(b) * kRedBlocks * kRedSlots, nparts, s);
   if (threadIdx.x == 0) {
     arrived[b] = 0;
     KState k{};
@@ -187,26 +185,24 @@ template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_update_s(Span sp, const int *plist, const KState *st,
                                                           const int *active, const C *__restrict__ r,
                                                           const C *__restrict__ v, C *__restrict__ s,
-                                                          double *partS) {
+                                                          int nchunk, double *partS) {
   pdl_begin();
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, reversed_y());
   if (!active[b]) return;
   const C al = state_alpha<C>(st[b]);
-  A ss = 0;
-  problem_loop_pairs<C>(sp, b, [&]<int N>(size_t o) {
+  double *pb = partS + size_t(b) * kRedBlocks * kRedSlots;
+  problem_sums<1, C>(sp, b, nchunk, pb, [&]<int N>(size_t o, A (&acc)[1]) {
     C ri[N], vi[N];
     ldN(r + o, ri);
     ldN(v + o, vi);
 #pragma unroll
     for (int n = 0; n < N; ++n) {
       ri[n] = csub(ri[n], cmul(al, vi[n]));
-      ss += ri[n].x * ri[n].x + ri[n].y * ri[n].y;
+      acc[0] += ri[n].x * ri[n].x + ri[n].y * ri[n].y;
     }
     stN(s + o, ri);
   });
-  A acc[1] = {ss};
-  block_sum_store<1>(acc, partS + (size_t(b) * kRedBlocks + blockIdx.x) * kRedSlots);
 }
 
 // omega of every active problem (one warp each), likewise.
@@ -225,14 +221,14 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *p
                                                            int max_iter, const C *__restrict__ p,
                                                            const C *__restrict__ s, const C *__restrict__ t,
                                                            const C *__restrict__ rhat, C *__restrict__ x,
-                                                           C *__restrict__ r, double *partC) {
+                                                           C *__restrict__ r, int nchunk, double *partC) {
   pdl_begin();
   using A = typename Acc<C>::type;
   const int b = problem_at(plist, reversed_y());
   if (!active[b]) return;
   const C al = state_alpha<C>(st[b]), o = state_omega<C>(st[b]);
-  A re = 0, im = 0, rr = 0;
-  problem_loop_pairs<C>(sp, b, [&]<int N>(size_t e) {
+  double *pb = partC + size_t(b) * kRedBlocks * kRedSlots;
+  problem_sums<3, C>(sp, b, nchunk, pb, [&]<int N>(size_t e, A (&acc)[3]) {
     C si[N], xi[N], pi[N], ti[N], hi[N];
     ldN(s + e, si);
     ldN(x + e, xi);
@@ -244,21 +240,18 @@ __global__ void __launch_bounds__(kRedThreads) k_update_xr(Span sp, const int *p
       xi[n] = cadd(xi[n], cadd(cmul(al, pi[n]), cmul(o, si[n])));
       const C ri = csub(si[n], cmul(o, ti[n]));
       si[n] = ri;  // (reused as the new residual)
-      re += hi[n].x * ri.x + hi[n].y * ri.y;
-      im += hi[n].x * ri.y - hi[n].y * ri.x;
-      rr += ri.x * ri.x + ri.y * ri.y;
+      acc[0] += hi[n].x * ri.x + hi[n].y * ri.y;
+      acc[1] += hi[n].x * ri.y - hi[n].y * ri.x;
+      acc[2] += ri.x * ri.x + ri.y * ri.y;
     }
     stN(x + e, xi);
     stN(r + e, si);
   });
-  A acc[3] = {re, im, rr};
-  double *pb = partC + size_t(b) * kRedBlocks * kRedSlots;
-  block_sum_store<3>(acc, pb + size_t(blockIdx.x) * kRedSlots);
   // convergence test, breakdown restart and beta for the next iteration, by the problem's last CTA
   // (the decision itself is bicgstab_decide in krylov.cuh)
   if (!last_cta(arrived + b, gridDim.x)) return;
   double q[3];
-  gather_n<3>(pb, gridDim.x, q);
+  gather_n<3>(pb, nchunk, q);
   if (threadIdx.x != 0) return;
   KState k = st[b];
   const int act = bicgstab_decide(k, q, tol, max_iter);
@@ -401,7 +394,11 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
   C *x = static_cast<C *>(x_);
   C *r = static_cast<C *>(sb.r), *rhat = static_cast<C *>(sb.rhat), *p = static_cast<C *>(sb.p);
   C *v = static_cast<C *>(sb.v), *sv = static_cast<C *>(sb.s), *t = static_cast<C *>(sb.t);
-  const int nblk = group ? kRedBlocks : red_blocks(sp.n, B, op.precision);  // CTAs per problem of the vector kernels
+  // the vector kernels: CTAs per problem, and partials of their sums (complex64: over pairs of elements;
+  // k_init's over single ones)
+  constexpr bool kSingle = sizeof(C) == sizeof(float2);
+  const int nblk = group ? kRedBlocks : red_blocks(sp.n, B, op.precision);
+  const int nsum = !group && kSingle ? red_parts(sp.n / 2) : nblk, nsum_init = !group && kSingle ? red_parts(sp.n) : nblk;
   const dim3 grid(nblk, B);
   int rc;
   cudaError_t e = cudaMemsetAsync(sb.counters, 0, 3 * sizeof(int), s);
@@ -411,7 +408,7 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
                                : operator_parts(op.B, op.nz, op.lx, op.precision);
   // the single-grid operator finishes alpha and omega in its last kernel
   const bool fused = !group && !op.Dhat;
-  const KrylovFinish fin{sb.st, sb.arrived, sb.partS, nblk, o.tol};
+  const KrylovFinish fin{sb.st, sb.arrived, sb.partS, nsum, o.tol};
   if (fused) op.finish = &fin;
   op.stencil = true;
   op.active = nullptr;
@@ -425,9 +422,10 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
     op.in = x; op.ident = x; op.out = v;
     if ((rc = run_operator(op, s))) return rc;
   }
-  launch_pdl(k_init<C>, grid, kRedThreads, 0, s, sp, sb.st, rhs, v, r, rhat, p, x, x_zero ? 1 : 0, sb.partA);
+  launch_pdl(k_init<C>, grid, kRedThreads, 0, s, sp, sb.st, rhs, v, r, rhat, p, x, x_zero ? 1 : 0, nsum_init, sb.partA);
   if ((rc = check_launch("k_init"))) return rc;
-  launch_pdl(k_init_state, B, 32, 0, s, sb.st, sb.active, sb.counters, sb.arrived, sb.partA, nblk, o.tol, o.max_iter);
+  launch_pdl(k_init_state, B, 32, 0, s, sb.st, sb.active, sb.counters, sb.arrived, sb.partA, nsum_init, o.tol,
+             o.max_iter);
   if ((rc = check_launch("k_init_state"))) return rc;
   if (!x_zero) {
     launch_pdl(k_zero_flagged<C>, grid, kRedThreads, 0, s, sp, sb.st, x);
@@ -470,16 +468,16 @@ static int bicgstab_typed(OpArgs op, const SolverBufs &sb, const void *rhs_, voi
       launch_pdl(k_alpha, nrun, 32, 0, st, plist, sb.st, sb.active, nparts, sb.partA);
       if ((rc2 = check_launch("k_alpha"))) return rc2;
     }
-    launch_pdl(k_update_s<C>, g2, kRedThreads, 0, st, sp, plist, sb.st, sb.active, r, v, sv, sb.partS);
+    launch_pdl(k_update_s<C>, g2, kRedThreads, 0, st, sp, plist, sb.st, sb.active, r, v, sv, nsum, sb.partS);
     if ((rc2 = check_launch("k_update_s"))) return rc2;
     op.epi = 2; op.in = sv; op.ident = sv; op.out = t; op.part_out = sb.partB;
     if ((rc2 = run_operator(op, st))) return rc2;
     if (!fused) {
-      launch_pdl(k_omega, nrun, 32, 0, st, plist, sb.st, sb.active, nparts, sb.partB, sb.partS, nblk, o.tol);
+      launch_pdl(k_omega, nrun, 32, 0, st, plist, sb.st, sb.active, nparts, sb.partB, sb.partS, nsum, o.tol);
       if ((rc2 = check_launch("k_omega"))) return rc2;
     }
     launch_pdl(k_update_xr<C>, g2, kRedThreads, 0, st, sp, plist, sb.st, sb.active, sb.counters, parity, sb.arrived, o.tol,
-                                               o.max_iter, p, sv, t, rhat, x, r, sb.partC);
+                                               o.max_iter, p, sv, t, rhat, x, r, nsum, sb.partC);
     return check_launch("k_update_xr");
   };
   const int K = o.check_every;

@@ -2,7 +2,10 @@
 //
 // A reduction is two-stage: every CTA sums its threads' values in a fixed tree and stores one
 // partial per slot; every consumer sums a problem's partials in a fixed order. The same inputs
-// therefore always give the same bits, whichever kernel consumes them.
+// therefore always give the same bits, whichever kernel consumes them. In complex64 on 2D grids a problem's
+// bits do not depend on the batch around it either; in complex128 the tiles and CTAs of a small batch (ls_operator.cu,
+// red_blocks) and in 3D the path (ls3d.cu) follow the batch, and a problem alone agrees with the same
+// problem in a batch to rounding.
 #pragma once
 
 #include "common.cuh"
