@@ -174,7 +174,7 @@ size_t bytes_partials(int B) {
 int red_blocks(size_t n, int B, int precision) {
   const size_t items = precision == DBI_C64 ? (n + 1) / 2 : n;  // 16-byte accesses
   const size_t enough = (items + 8 * kRedThreads - 1) / (8 * kRedThreads);
-  const size_t most = (items + kRedThreads - 1) / kRedThreads, fill = size_t(4 * 152) / size_t(B > 0 ? B : 1);
+  const size_t most = (items + kRedThreads - 1) / kRedThreads, fill = 4 * kSMs / size_t(B > 0 ? B : 1);
   size_t k = enough;
   if (k < fill) k = fill < most ? fill : most;
   return int(k < 1 ? 1 : k > size_t(kRedBlocks) ? size_t(kRedBlocks) : k);

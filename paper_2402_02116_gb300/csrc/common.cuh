@@ -206,6 +206,9 @@ size_t bytes_scales(int B);
 // problem chunks of the adjoint imaging (each accumulates its own FP64 partial image)
 int imaging_chunks(int B);
 
+// SMs of a GB300: the unit of the rules that fit a batch's work to the chip.
+constexpr size_t kSMs = 152;
+
 // Geometry of the FP64 partial sums of the Krylov reductions.
 constexpr int kRedBlocks = 64;    // blocks per problem in a reduction pass, at most (and the stride of partials)
 constexpr int kRedThreads = 256;  // threads per reduction block

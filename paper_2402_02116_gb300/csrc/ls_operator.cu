@@ -361,11 +361,33 @@ __global__ void __launch_bounds__(kS3Threads, 2) k_rows_inverse_s3(OpP<float2> p
 
 // Threads per CTA of the ordinary stages: 256, or for complex128 batches too small to give every SM a
 // 256-thread tile, as few as hold whole lines and warps (beyond length 128; up to it the kernels of
-// small64.cuh run). FP64 runs at two lanes a cycle and SM, so what counts there is the number of SMs: a
-// 32 x 32 grid of one problem was one row tile and two column tiles (68, 40 and 24 us for the stages).
+// small64.cuh run). FP64 runs at two lanes a cycle and SM, so what counts there is the SM with the most
+// rows or columns: a 32 x 32 grid of one problem was one row tile and two column tiles (68, 40 and 24 us for
+// the stages).
 template <int L> constexpr int kSmallThreads = L / 8 > 32 ? L / 8 : 32;
-inline bool small_tiles(int B, int nz, int lx, int precision) {
-  return precision == DBI_C128 && lx <= 1024 && size_t(B) * ((size_t(nz) * lx + 2047) / 2048) < 2 * 152;
+inline size_t ceil_div(size_t a, size_t b) { return (a + b - 1) / b; }
+// The row stages on small tiles, of one row each from length 128 on. Such a tile also forms the stress of
+// its own halo rows, about as much work as 0.35 (length 128) or 0.6 rows; so they pay where the busiest SM has
+// less to do with them. Measured, as shares of the pass: with 80 to 112 of the 256-thread tiles (of 152 SMs) -9
+// to -2 % at length 128, -2 to +10 at 256, +7 at 1024; with 128 to 152 of them up to +21 %; with 156 to 182
+// -13 to 0 %; with 240 to 304 up to +27 %; with fewer than 76 -25 to -50 %. Up to length 64 they win up to two
+// waves (-12 % at 128, -8 % at 152 tiles of 32^2). A pass without the stencil has no halo (16 convolutions of 100^2
+// 345 us on small tiles, 374 us on the others).
+inline bool small_rows(int B, int nz, int lx, int precision, bool stencil) {
+  if (precision != DBI_C128 || lx > 1024) return false;
+  const size_t rows = size_t(2048 / lx), tiles = size_t(B) * ceil_div(nz, rows);
+  const size_t halo = !stencil ? 0 : lx <= 128 ? 7 : 12;  // in 1/20 rows
+  if (tiles >= 2 * kSMs) return false;
+  return lx <= 64 || ceil_div(size_t(B) * nz, kSMs) * (20 + halo) < ceil_div(tiles, kSMs) * (20 * rows + halo);
+}
+// The column stage on small tiles: no halo, but fewer warps behind each other's latency. They pay unless the
+// last wave of 256-thread tiles is nearly full: -22 to -10 % of the pass with 16 to 76 tiles, -9 % at 96,
+// -5 to 0 % at 128, +1 to +3 % at 144 to 152; -17 % at 160 to 176, -6 to 0 % at 256, up to +3 % at 272 to 304;
+// -11 % at 320, -4 % at 384.
+inline bool small_cols(int B, int lz, int lx, int precision) {
+  if (precision != DBI_C128 || lz > 1024) return false;
+  const size_t tiles = size_t(B) * ceil_div(lx, 2048 / lz);
+  return tiles < 4 * kSMs && 8 * tiles <= 7 * kSMs * ceil_div(tiles, kSMs);
 }
 template <typename C, int L, typename F> inline void with_tile(bool small, F &&f) {
   if constexpr (sizeof(C) == sizeof(double2) && L > 128) {
@@ -415,7 +437,9 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
   p.part_out = a.part_out;
   p.S = nullptr;
   int rc = DBI_OK;
-  const bool stencil = a.stencil, small = small_tiles(a.B, a.nz, a.lx, a.precision);
+  const bool stencil = a.stencil;
+  const bool small_r = small_rows(a.B, a.nz, a.lx, a.precision, stencil);
+  const bool small_c = small_cols(a.B, a.lz, a.lx, a.precision);
   const int kr = split_kind(a.lx, a.precision), kc = split_kind(a.lz, a.precision);
   const bool split_r = kr != 0, split_c = kc != 0;
   if (split_r) p.S = p.T + size_t(cap) * 2 * a.lx * a.nz;  // after the chunk's spectra
@@ -453,7 +477,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
         if (stencil) {
           // rows per CTA: 32 while that leaves four waves of CTAs, at least 4
           int chunk = 32;
-          const int wave = DBI_STREAM_THREADS / (LX / 2) * 152;
+          const int wave = DBI_STREAM_THREADS / (LX / 2) * int(kSMs);
           while (chunk > 4 && long((a.nz + chunk - 1) / chunk) * nb < 4L * wave) chunk /= 2;
           const size_t bytes = StreamCfg<LX>::smem;
           e = allow_smem(k_rows_stream<LX, V>, bytes);
@@ -464,7 +488,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
         }
       }
       if constexpr (sizeof(C) == sizeof(double2) && LX <= 128) {
-        if (small) {
+        if (small_r) {
           const size_t bytes = small64_forward_smem<LX>(a.nx, stencil);
           constexpr int U = Small64<LX>::UNITS;
           auto kern = stencil ? k_rows_forward_small<LX, true, V> : k_rows_forward_small<LX, false, V>;
@@ -474,7 +498,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           return;
         }
       }
-      with_tile<C, LX>(small, [&]<int NTT>() {
+      with_tile<C, LX>(small_r, [&]<int NTT>() {
         using RC = RowCfg<C, LX, NTT>;
         const size_t bytes = rows_forward_smem<C, LX, NTT>(a.nx, stencil);
         dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
@@ -543,14 +567,14 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
       } else {
         cudaError_t e = cudaSuccess;
         if constexpr (LZ <= 128) {
-          if (small) {
+          if (small_c) {
             constexpr int U = Small64<LZ>::UNITS;
             launch_pdl(k_cols_small<LZ, V>, dim3((a.lx + U - 1) / U, nb), 32, Small64<LZ>::lines, s, p);
             rc = check_launch("k_cols_small");
             return;
           }
         }
-        with_tile<C, LZ>(small, [&]<int NTT>() {
+        with_tile<C, LZ>(small_c, [&]<int NTT>() {
           using CN = ColCfg<C, LZ, NTT>;
           const size_t bytes = cols_smem<C, LZ, NTT>();
           dim3 grid((a.lx + CN::CC - 1) / CN::CC, nb);
@@ -585,7 +609,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
     with_plan<LX>(a.precision, [&]<int V>() {
       cudaError_t e;
       if constexpr (sizeof(C) == sizeof(double2) && LX <= 128) {
-        if (small) {
+        if (small_r) {
           constexpr int U = Small64<LX>::UNITS;
           auto kern = a.epi == 1 ? k_rows_inverse_small<LX, 1, V> : a.epi == 2 ? k_rows_inverse_small<LX, 2, V>
                                                                                : k_rows_inverse_small<LX, 0, V>;
@@ -594,7 +618,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           return;
         }
       }
-      with_tile<C, LX>(small, [&]<int NTT>() {
+      with_tile<C, LX>(small_r, [&]<int NTT>() {
         using RC = RowCfg<C, LX, NTT>;
         const size_t bytes = rows_inverse_smem<C, LX, NTT>();
         dim3 grid((a.nz + RC::ROWS - 1) / RC::ROWS, nb);
@@ -629,7 +653,7 @@ template <typename C> static int run_typed(const OpArgs &a, cudaStream_t s) {
 int operator_parts(int B, int nz, int lx, int precision) {
   static_assert(kS3Units == kSplitRows, "split row tiles hold the same number of rows");
   if (split_rows(lx, precision)) return (nz + kSplitRows - 1) / kSplitRows;
-  if (small_tiles(B, nz, lx, precision)) {
+  if (small_rows(B, nz, lx, precision, true)) {
     int rows = 1;
     dispatch_len(lx, [&]<int LX>() {
       if constexpr (LX <= 128) rows = Small64<LX>::UNITS;
