@@ -168,13 +168,17 @@ template <int LZ, int SL> constexpr size_t cols_pairs_smem() {
   return size_t(CF::CC) * CF::PLP * sizeof(cpair) + (SL == 1 ? 0 : size_t(CF::CC / SL) * 3 * LZ * sizeof(float2));
 }
 
-// The complex64 column stage of lengths 32 to 256 with 16 points per thread (fft16.cuh): T lanes of one
+// The complex64 column stage of lengths 128 and 256 with 16 points per thread (fft16.cuh): T lanes of one
 // warp take one column of one slot, every exchange stays inside them, and the CTA meets at no
 // barrier. SL slots of a column sit side by side, so that their warp or CTA finds the column's Green's
-// tables in L1. 168 registers, 3 CTAs per SM (128 spill). 45 problems of 45 x 180 (lz = 128): 17.2 us
-// against 24 us with 8 points per thread; 120^2 x 256 problems (lz = 256) 91 us. At length 512
+// tables in L1. 168 registers, 3 CTAs per SM (128 spill). Against 8 points per thread (k_cols) the whole
+// operator pass took, on 256 problems, 64.3 against 73.1 us of 64^2 (lz = 128) and 214 against 237 us of
+// 128^2 (lz = 256); on one problem both take the same. At lengths 32 and 64, with 2 and 4 lanes per
+// line, it is k_cols that is faster: 16 BiCGSTAB iterations on 1, 16 and 256 problems of 32^2 (lz = 64) 864,
+// 929 and 1196 us against 893, 950 and 1240 us, of 16 x 64 (lz = 32) 664, 683 and 1020 against 696, 709 and
+// 996 us, of 16^2 790, 809 and 1182 against 809, 838 and 1181 us. At length 512
 // (two 256-point transforms per half-pruned one, the two half warps combining by lane exchanges) the
-// same form took 408 to 444 us for 256 problems of 256^2 with more rounding error or more table loads,
+// 16-point form took 408 to 444 us for 256 problems of 256^2 with more rounding error or more table loads,
 // against 422 us of the 8-point form above, which stays there.
 constexpr int kCols16Threads = 128;
 template <int LZ> constexpr size_t kCols16Smem = size_t(kCols16Threads / (LZ / 16)) * Fft16<LZ>::LP * sizeof(cpair);
@@ -547,7 +551,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           };
           if (four) launch.template operator()<4>();
           else launch.template operator()<1>();
-        } else if constexpr (LZ >= 32 && LZ <= 256) {
+        } else if constexpr (LZ >= 128 && LZ <= 256) {
           auto launch = [&]<int SL>() {
             constexpr int COLS = kCols16Threads / (LZ / 16) / SL;
             e = allow_smem(k_cols16<LZ, SL>, kCols16Smem<LZ>);
@@ -557,7 +561,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           };
           if (four) launch.template operator()<4>();
           else launch.template operator()<1>();
-        } else if constexpr (LZ == 16) {
+        } else if constexpr (LZ <= 64) {
           const size_t bytes = cols_smem<C, LZ>();
           e = allow_smem(k_cols<C, LZ, V, kTileThreads>, bytes);
           if (e == cudaSuccess)
