@@ -750,9 +750,9 @@ static int run3_slab(const OpArgs &a, cudaStream_t s) {
   with_slab_len(a.ly, a.lz, [&]<int LY, int LZ>() {
     const size_t bytes = slab_smem<LY, LZ>(p.nzp);
     p.spare = slab_rows<LZ>(p.nzp);
-    p.ahead = 2 * 152 / nb + 1;  // two CTAs per SM are in flight
+    p.ahead = 512 / kSlabThreads<LY, LZ> * int(kSMs) / nb + 1;  // the slabs in flight
     cudaError_t e = allow_smem(k3_yz<LY, LZ>, bytes);
-    if (e == cudaSuccess) launch_pdl(k3_yz<LY, LZ>, unsigned(a.lx) * unsigned(nb), kSlabThreads, bytes, s, p);
+    if (e == cudaSuccess) launch_pdl(k3_yz<LY, LZ>, unsigned(a.lx) * unsigned(nb), kSlabThreads<LY, LZ>, bytes, s, p);
     rc = e != cudaSuccess ? cuda_fail("k3_yz smem", e) : check_launch("k3_yz");
   });
   prof_mark(PROF_COLS, true, s);

@@ -17,13 +17,15 @@
 // along y, two neighbouring ky along z.
 #pragma once
 
+#include <algorithm>
+
 #include "fft16.cuh"
 #include "operator.cuh"
 #include "op_tiles.cuh"
 
 namespace dbi {
 
-constexpr int kSlabXThreads = 128, kSlabThreads = 256;
+constexpr int kSlabXThreads = 128;
 
 struct WarpBarrier {
   __device__ __forceinline__ void operator()() const { __syncwarp(); }
@@ -214,6 +216,10 @@ template <int LX> __global__ void __launch_bounds__(kSlabXThreads) k3_x_inv(Slab
 // (two neighbouring rows hold the exchange line of their pair) and 8 mod 16, so that the z transforms'
 // 16-byte accesses (ky pairs of a column, rows P / 2 = 4 mod 8 slots apart) spread over the banks.
 template <int LY> constexpr int kSlabP = ((LY + LY / 16 + 7) / 16) * 16 + 8;
+// Threads per slab: as many as the z transforms have lanes, 64 to 256. (With 256 on every slab most of a
+// CTA idled at short lengths: one pass over 160 wavefields of 9 x 11 x 13 cells, ly = lz = 32, took 219 us, now
+// 121 us, and 205 us as separate passes; of 16^3 305, 209 and 304 us.)
+template <int LY, int LZ> constexpr int kSlabThreads = std::clamp(LY / 2 * (LZ / 8), 64, 256);
 // Slab rows: 3 nzp, or the z exchange's line if that is longer, rounded up to even.
 template <int LZ> inline int slab_rows(int nzp) {
   const int lp = RegFFT<cpair, LZ>::LP;
@@ -238,10 +244,10 @@ __device__ __forceinline__ cpair pmad(cpair acc, cpair g, cpair v, pair64 nim) {
 // thread has few loads in flight), so every CTA also starts the L2 fetch of the slab that follows its own
 // wave and of an eighth of that slab's tables.
 template <int LY, int LZ>
-__global__ void __launch_bounds__(kSlabThreads, 2) k3_yz(SlabP p) {
+__global__ void __launch_bounds__(kSlabThreads<LY, LZ>, 512 / kSlabThreads<LY, LZ>) k3_yz(SlabP p) {
   pdl_begin();
   using F = Fft16<LY>;
-  constexpr int P = kSlabP<LY>, TY = F::T, TZ = LZ / 8, KPW = 32 / TZ;
+  constexpr int P = kSlabP<LY>, TY = F::T, TZ = LZ / 8, KPW = 32 / TZ, NT = kSlabThreads<LY, LZ>;
   const int slot = int(blockIdx.x % unsigned(p.nb)), kx = int(blockIdx.x / unsigned(p.nb));
   const int b = slab_problem(p, slot);
   if (b < 0) return;
@@ -259,7 +265,7 @@ __global__ void __launch_bounds__(kSlabThreads, 2) k3_yz(SlabP p) {
   const typename F::Base base(ty, p.tw);
   // along y: line l = (c, z / 2), all lanes of a warp take part in its exchanges
   auto lines_y = [&](auto &&body) {
-    for (int l0 = (threadIdx.x >> 5) * (32 / TY); l0 < nlines; l0 += kSlabThreads / TY) {
+    for (int l0 = (threadIdx.x >> 5) * (32 / TY); l0 < nlines; l0 += NT / TY) {
       const int l = l0 + (threadIdx.x & 31) / TY;
       const bool live = l < nlines;
       const int c = live ? l / half : 0, z0 = live ? 2 * (l - c * half) : 0;
@@ -290,7 +296,7 @@ __global__ void __launch_bounds__(kSlabThreads, 2) k3_yz(SlabP p) {
     const int lane = threadIdx.x & 31, tz = lane / KPW;
     const TwReg<float2, LZ, 0> tr(tz, p.tw);
     const cpair *Gk = p.G + (size_t(p.fidx[b]) * p.lx + kx) * kTable;
-    for (int k0 = (threadIdx.x >> 5) * KPW; k0 < LY / 2; k0 += kSlabThreads / 32 * KPW) {
+    for (int k0 = (threadIdx.x >> 5) * KPW; k0 < LY / 2; k0 += NT / 32 * KPW) {
       const int kp = k0 + lane % KPW;
       cpair *col = reinterpret_cast<cpair *>(slab) + kp;  // row i at col[i P / 2]
       const StridedLine<cpair> line[1] = {{col, P / 2}};
