@@ -95,6 +95,9 @@ __global__ void __launch_bounds__(NTT, NTT == kTileThreads ? Cfg<C>::rowFwdMinBl
                                        reinterpret_cast<C *>(smem_raw));
 }
 
+// Lengths whose forward row stage walks down the rows (with the stencil).
+template <typename C, int LX> constexpr bool kRowsStream = kPairSpectra<C> && LX >= 128 && LX <= 512;
+
 // The forward row stage of complex64 lengths 128 to 512 in chunks of `chunk` rows (rows_stream.cuh). 768
 // threads per SM (80 registers each); with 512 the stage was no faster.
 #ifndef DBI_STREAM_THREADS
@@ -475,9 +478,10 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
     }
   }
   if (!split_r) dispatch_len(a.lx, [&]<int LX>() {
+    if constexpr (!kPairSpectra<C> || LX <= 512)  // (complex64 of length 1024 is split)
     with_plan<LX>(a.precision, [&]<int V>() {
       cudaError_t e;
-      if constexpr (kPairSpectra<C> && LX >= 128 && LX <= 512) {
+      if constexpr (kRowsStream<C, LX>) {
         if (stencil) {
           // rows per CTA: 32 while that leaves four waves of CTAs, at least 4
           int chunk = 32;
@@ -510,7 +514,8 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
           e = allow_smem(kernel, bytes);
           if (e == cudaSuccess) launch_pdl(kernel, grid, RC::NT, bytes, s, p);
         };
-        if (stencil) launch(k_rows_forward<C, LX, true, V, NTT>);
+        if constexpr (kRowsStream<C, LX>) launch(k_rows_forward<C, LX, false, V, NTT>);
+        else if (stencil) launch(k_rows_forward<C, LX, true, V, NTT>);
         else launch(k_rows_forward<C, LX, false, V, NTT>);
       });
       rc = e != cudaSuccess ? cuda_fail("k_rows_forward smem", e) : check_launch("k_rows_forward");
@@ -610,6 +615,7 @@ template <typename C> static int run_chunk(const OpArgs &a, int s0, int nb, int 
     }
   }
   if (!split_r) dispatch_len(a.lx, [&]<int LX>() {
+    if constexpr (!kPairSpectra<C> || LX <= 512)  // (complex64 of length 1024 is split)
     with_plan<LX>(a.precision, [&]<int V>() {
       cudaError_t e;
       if constexpr (sizeof(C) == sizeof(double2) && LX <= 128) {
