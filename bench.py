@@ -389,8 +389,8 @@ def measured_alu_peak(dev, clocks):
 # (nz, nx, lz, lx) -> (problems in the captured launch, frequencies, bytes). The Green's spectra
 # [nf][3][lx][lz] are read once per launch; the rest grows with the problems a launch processes.
 COLS_DRAM = {
-    # one k_cols_split launch over 6 sources x 6 frequencies (profiles/operator_kernels_vti512_6src_6f.md)
-    (512, 512, 1024, 1024): (36, 6, 473_260_032 + 252_288_768),
+    # one k_cols_split launch over 8 sources x 6 frequencies (profiles/operator_kernels_pairs.md)
+    (512, 512, 1024, 1024): (48, 6, 561_916_672 + 346_642_944),
 }
 
 
@@ -654,7 +654,6 @@ def reference_values(w):
 # ---------------------------------------------------------------------------------------------
 # roofline arithmetic of the column pass (per D-cell per operator pass)
 # ---------------------------------------------------------------------------------------------
-COLS_DRAM_BYTES_PER_PROBLEM = 4.35e6  # ncu, k_cols before the per-exchange line layout
 
 
 def cols_bytes_per_cell_apply(w):
@@ -1163,16 +1162,16 @@ def run_formk(args):
     cols_s = cols_ms * 1e-3
     flops = formk_cols_flops_per_cell_apply(w) * cells * args.steps
     algo_bytes = formk_cols_bytes_per_cell_apply(w) * cells * args.steps
-    # DRAM bytes per launch from one ncu capture of kk_cols over 32 wavefields of this grid (8
-    # frequencies): 373.98 MB, of which the nine kernel tables are 151 MB; the rest grows with the
+    # DRAM bytes per launch from one ncu capture of kk_cols_pairs over 64 wavefields of this grid (8
+    # frequencies): 603.94 MB, of which the nine kernel tables are 151 MB; the rest grows with the
     # wavefields a launch processes
     traffic = None
     if (w.nz, w.nx, w.lz, w.lx, w.nf) == (256, 256, 512, 512, 8):
         tables = 9 * w.lz * w.lx * 8 * w.nf
-        traffic = tables + (373.98e6 - tables) / 32 * cells * args.steps / (w.nz * w.nx) / max(cols_launches, 1)
+        traffic = tables + (603.94e6 - tables) / 64 * cells * args.steps / (w.nz * w.nx) / max(cols_launches, 1)
     roof = {"bound": "alu", "achieved": flops / cols_s / 1e12, "peak": peak_tf, "unit": "TFLOP/s",
             "peak_source": peak_src, "peak_nominal": nominal_tf,
-            "traffic": traffic, "kernel": "kk_cols (five forward column FFTs, 2 x 5 kernel, two inverse)",
+            "traffic": traffic, "kernel": "kk_cols_pairs (five forward column FFTs, 2 x 5 kernel, two inverse)",
             "hbm_frac_of_algorithmic_bytes": algo_bytes / cols_s / (peaks.get("hbm_gbs", 6800.0) * 1e9),
             "launches_timed": cols_launches, "avg_launch_ms": cols_ms / max(cols_launches, 1),
             "share_of_step_time": cols_ms / ms_k if ms_k > 0 else None}

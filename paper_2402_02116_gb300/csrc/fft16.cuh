@@ -80,7 +80,7 @@ template <bool INV, bool HALF> __host__ __device__ __forceinline__ void pdft16(c
   }
 }
 
-// w^1 .. w^15 from the table's values of w, w^4 and w^8, by at most three products in sequence.
+// w^1 .. w^15 from the table's values of w, w^4 and w^8, by at most four products in sequence (w^15 = w^8 w^7).
 __host__ __device__ __forceinline__ void powers16(float2 w1, float2 w4, float2 w8, float2 (&w)[16]) {
   w[1] = w1;
   w[2] = hmul(w1, w1);
@@ -99,7 +99,7 @@ template <int L> struct Fft16 {
 
   // The thread's base twiddles of the second pass, read once per kernel: W_L^j of its NB butterflies
   // j = t + i T, or at R2 = 16 (one butterfly) W_L^j, W_L^{4j} and W_L^{8j}, from which the powers take
-  // at most three products in sequence (from W_L^j alone the operator's error grew by a tenth).
+  // at most four products in sequence (from W_L^j alone the operator's error grew by a tenth).
   static constexpr int kBase = R2 == 16 ? 3 : NB;
   struct Base {
     float2 w[kBase];
