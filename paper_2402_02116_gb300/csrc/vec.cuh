@@ -74,15 +74,26 @@ template <int N, typename C> __device__ __forceinline__ void stN(C *p, const C (
 // a problem follows the batch (red_blocks), but neither how much of a sum is added in FP32 nor its bits do.
 // (With one FP32 sum per warp over all of its CTA's items a warp added 512 elements of a 128^2 problem of 64,
 // now 64; the solves keep their time.) Complex128: FP64 throughout, one partial per CTA (nchunk =
-// gridDim.x; by chunks the FP64 shuffles cost 2 to 3 % of a solve).
+// gridDim.x; chunks cost 2 to 3 % of a solve, k_update_xr of 15 problems of up to 256^2 85 against 72 us).
 constexpr int kMaxChunks = 16;
 template <int NS, typename C, bool PAIRS = true, typename F>
 __device__ __forceinline__ void problem_sums(const Span &sp, int b, int nchunk, double *part, F &&f) {
   using A = typename Acc<C>::type;
+  const size_t off = sp.offset(b), cnt = sp.count(b);
+  if constexpr (sizeof(C) != sizeof(float2)) {
+    A acc[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k] = 0;
+#pragma unroll 4
+    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < cnt; i += size_t(gridDim.x) * blockDim.x)
+      f.template operator()<1>(off + i, acc);
+    block_sum_store<NS>(acc, part + size_t(blockIdx.x) * kRedSlots);
+    return;
+  }
   constexpr int kWarps = kRedThreads / 32;
   __shared__ double sh[kMaxChunks][NS][kWarps];
-  const size_t off = sp.offset(b), cnt = sp.count(b), step = size_t(sizeof(C) == sizeof(float2) ? kRedBlocks : gridDim.x) * kRedThreads;
-  const bool two = PAIRS && sizeof(C) == sizeof(float2) && ((off | cnt) & 1) == 0;
+  const size_t step = size_t(kRedBlocks) * kRedThreads;
+  const bool two = PAIRS && ((off | cnt) & 1) == 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int n = 0;
   for (int c = blockIdx.x; c < nchunk; c += gridDim.x, ++n) {
@@ -91,7 +102,7 @@ __device__ __forceinline__ void problem_sums(const Span &sp, int b, int nchunk, 
 #pragma unroll
     for (int k = 0; k < NS; ++k) acc[k] = 0;
     if (two) {
-      if constexpr (PAIRS && sizeof(C) == sizeof(float2)) {
+      if constexpr (PAIRS) {
 #pragma unroll 2
         for (size_t i = i0; i < cnt / 2; i += step) f.template operator()<2>(off + 2 * i, acc);
       }
