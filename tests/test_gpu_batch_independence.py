@@ -1,8 +1,8 @@
 """A problem's solution does not depend on the batch it is solved in: alone, and as the first and the last of
 a batch that shares the SMs among many problems, the complex64 BiCGSTAB gives the same bits and the same
 iteration counts. (How a problem's sums are split into partials follows from the size of its grid; the batch only
-sets how many CTAs work on them.) Grids on which a batch of 45 takes 1, 4, 9 and 64 CTAs per problem
-for the partials, ragged ones among them."""
+sets how many CTAs work on them.) Grids on which a batch of 45 takes 1, 13, 13 and 16 CTAs per problem and a
+problem alone 1, 32, 64 and 64, ragged ones among them."""
 import pytest
 import torch
 
